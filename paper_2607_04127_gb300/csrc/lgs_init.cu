@@ -4,26 +4,26 @@
 // initialisation, the physics-based confidence u of Eq. physconf and the
 // opacity of Eq. alpha_init).
 //
-// Launches: the points go into spatial order first (a counting sort by a
-// 21-bit Morton code of a uniform grid over the scan's extent: 7 bits per
-// axis), so that a tile of 256 consecutive points is compact; per-tile
-// bounding boxes; the k nearest neighbours (one CTA per query tile, an exact
-// top-K kept sorted in registers, candidate tiles staged in shared memory;
-// the CTA's own and adjacent tiles first, then only tiles whose box can still
-// hold a point closer than the CTA's current K-th distance, nearest first;
-// each warp skips the tiles provably beyond its own K-th distances); the
-// frame of each point (covariance of the neighbourhood, cyclic Jacobi
-// eigendecomposition, scales, confidence, opacity, orientation).  Keys carry
-// the original index, so the order of the sort never shows in a result.
+// Launches: the points go into spatial order first (a radix sort by a 27-bit
+// Morton code of a uniform grid whose cell is as fine as 27 bits allow for
+// the scan's extent), so that a leaf of 32 consecutive points is compact; two
+// levels of bounding boxes over them (leaves, nodes of 32 leaves); the k
+// nearest neighbours (one warp per query: each lane holds one entry of the
+// sorted top 32, boxes and points are tested 32 at a time, nearest box first,
+// until no box can hold a closer point); the frame of each point (covariance
+// of the neighbourhood, cyclic Jacobi eigendecomposition, scales, confidence,
+// opacity, orientation).  Keys carry the original index, so the order of the
+// sort never shows in a result.
 //
 // The neighbour sets are integer outcomes: the squared distance that decides
 // them is binary32 ((dx dx + dy dy) + dz dz), each operation correctly
 // rounded, ties to the lower index, so the sets are a fixed function of the
-// input (and bit-exact against the oracle).  Tile pruning is conservative
+// input (and bit-exact against the oracle).  Box pruning is conservative
 // (a margin of 1e-5 on the box distance, far above the few ulps that separate
 // the box bound from any binary32 distance), so it never changes a set.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 
 #include "lgs_internal.cuh"
@@ -31,12 +31,13 @@
 namespace lgs {
 namespace {
 
-constexpr int kIniTile = 256;        // points per tile = queries per CTA
-constexpr int kIniWindow = 3;        // tiles visited before pruning: own, +-1
-constexpr int kIniMaxTiles = 4096;   // n <= 2^20
-constexpr int kIniCellBits = 7;      // Morton grid: 2^7 cells per axis
-constexpr uint32_t kIniCells = 1u << (3 * kIniCellBits);
-constexpr int kIniSorted = 1024;     // candidate lists up to this long are visited nearest first
+constexpr uint32_t kIniMaxPoints = 1u << 20;
+constexpr int kIniCodeBits = 27;     // Morton code: three radix passes of 9 bits
+constexpr int kIniDigit = 9;
+constexpr uint32_t kIniBins = 1u << kIniDigit;
+constexpr int kIniSortCta = 512;     // one thread per bin
+constexpr int kIniSortWarps = kIniSortCta / 32;
+constexpr int kIniExtCtas = 128;     // partial extents
 
 struct IniBox {
   float lo[3], hi[3];
@@ -48,107 +49,265 @@ struct IniParams {
   int k;
 };
 
-__global__ void __launch_bounds__(kIniTile) k_ini_boxes(const float* __restrict__ pts, uint32_t n,
-                                                        IniBox* __restrict__ boxes) {
-  __shared__ float s_lo[3][kIniTile / 32], s_hi[3][kIniTile / 32];
-  const uint32_t i = blockIdx.x * kIniTile + threadIdx.x;
-  const bool ok = i < n;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int a = 0; a < 3; ++a) {
-    const float v = ok ? pts[3 * i + a] : 0.f;
-    float lo = ok ? v : INFINITY, hi = ok ? v : -INFINITY;
+__device__ __forceinline__ void warp_min_max(float (&lo)[3], float (&hi)[3]) {
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
     for (int o = 16; o; o >>= 1) {
-      lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-      hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+      lo[a] = fminf(lo[a], __shfl_xor_sync(0xffffffffu, lo[a], o));
+      hi[a] = fmaxf(hi[a], __shfl_xor_sync(0xffffffffu, hi[a], o));
     }
-    if (lane == 0) {
-      s_lo[a][wid] = lo;
-      s_hi[a][wid] = hi;
+}
+
+// Extent of each CTA's share of the points.
+__global__ void __launch_bounds__(256) k_ini_part(const float* __restrict__ pts, uint32_t n, IniBox* __restrict__ part) {
+  pdl_launch_dependents();  // the next kernel may be dispatched now
+  __shared__ float s_lo[8][3], s_hi[8][3];
+  float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const float v = pts[3 * i + a];
+      lo[a] = fminf(lo[a], v);
+      hi[a] = fmaxf(hi[a], v);
     }
-  }
+  warp_min_max(lo, hi);
+  if ((threadIdx.x & 31) == 0)
+    for (int a = 0; a < 3; ++a) {
+      s_lo[threadIdx.x >> 5][a] = lo[a];
+      s_hi[threadIdx.x >> 5][a] = hi[a];
+    }
   __syncthreads();
   if (threadIdx.x < 3) {
-    float lo = INFINITY, hi = -INFINITY;
-    for (int w = 0; w < kIniTile / 32; ++w) {
-      lo = fminf(lo, s_lo[threadIdx.x][w]);
-      hi = fmaxf(hi, s_hi[threadIdx.x][w]);
+    float l = INFINITY, h = -INFINITY;
+    for (int w = 0; w < 8; ++w) {
+      l = fminf(l, s_lo[w][threadIdx.x]);
+      h = fmaxf(h, s_hi[w][threadIdx.x]);
     }
-    boxes[blockIdx.x].lo[threadIdx.x] = lo;
-    boxes[blockIdx.x].hi[threadIdx.x] = hi;
+    part[blockIdx.x].lo[threadIdx.x] = l;
+    part[blockIdx.x].hi[threadIdx.x] = h;
   }
 }
 
-// The scan's extent from the tile boxes (one CTA) and the grid's cell size.
-__global__ void __launch_bounds__(256) k_ini_extent(const IniBox* __restrict__ boxes, uint32_t n_tiles,
-                                                    float* __restrict__ ext) {
-  __shared__ float s_v[6][8];
-  float v[6] = {INFINITY, INFINITY, INFINITY, -INFINITY, -INFINITY, -INFINITY};
-  for (uint32_t t = threadIdx.x; t < n_tiles; t += blockDim.x)
+// The grid of the Morton code: origin, cell edge and the bits of each axis
+// (as many as its extent needs), together at most kIniCodeBits.
+struct IniGrid {
+  float lo[3], inv_h;
+  int bits[3];
+  uint32_t top[3];   // largest cell index of each axis
+};
+
+__global__ void __launch_bounds__(32) k_ini_grid(const IniBox* __restrict__ part, uint32_t n_part,
+                                                 IniGrid* __restrict__ grid) {
+  pdl_wait();               // (launched after a kernel of this chain: wait for it)
+  pdl_launch_dependents();  // the next kernel may be dispatched now
+  float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+  for (uint32_t t = threadIdx.x; t < n_part; t += 32)
     for (int a = 0; a < 3; ++a) {
-      v[a] = fminf(v[a], boxes[t].lo[a]);
-      v[3 + a] = fmaxf(v[3 + a], boxes[t].hi[a]);
+      lo[a] = fminf(lo[a], part[t].lo[a]);
+      hi[a] = fmaxf(hi[a], part[t].hi[a]);
     }
-  for (int a = 0; a < 6; ++a)
-    for (int o = 16; o; o >>= 1) {
-      const float w = __shfl_xor_sync(0xffffffffu, v[a], o);
-      v[a] = a < 3 ? fminf(v[a], w) : fmaxf(v[a], w);
-    }
-  if ((threadIdx.x & 31) == 0)
-    for (int a = 0; a < 6; ++a) s_v[a][threadIdx.x >> 5] = v[a];
-  __syncthreads();
-  if (threadIdx.x < 6) {
-    float r = s_v[threadIdx.x][0];
-    for (int w = 1; w < 8; ++w) r = threadIdx.x < 3 ? fminf(r, s_v[threadIdx.x][w]) : fmaxf(r, s_v[threadIdx.x][w]);
-    ext[threadIdx.x] = r;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const float span = fmaxf(fmaxf(ext[3] - ext[0], ext[4] - ext[1]), ext[5] - ext[2]);
-    ext[6] = fmaxf(span, 1e-20f) * (1.0001f / static_cast<float>(1 << kIniCellBits));   // cell edge
-  }
-}
-
-__device__ __forceinline__ uint32_t spread3(uint32_t x) {   // bits b -> 3b
-  uint32_t r = 0;
-#pragma unroll
-  for (int b = 0; b < kIniCellBits; ++b) r |= ((x >> b) & 1u) << (3 * b);
-  return r;
-}
-
-__global__ void __launch_bounds__(256) k_ini_zero(uint32_t* __restrict__ a, uint32_t len) {
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < len; i += gridDim.x * blockDim.x) a[i] = 0u;
-}
-
-__global__ void __launch_bounds__(256) k_ini_cells(const float* __restrict__ pts, uint32_t n,
-                                                   const float* __restrict__ ext, uint32_t* __restrict__ cell,
-                                                   uint32_t* __restrict__ cnt) {
-  const float h = ext[6];
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  uint32_t c[3];
-#pragma unroll
+  warp_min_max(lo, hi);
+  if (threadIdx.x != 0) return;
+  float span[3], most = 1e-20f;
   for (int a = 0; a < 3; ++a) {
-    const float q = floorf((pts[3 * i + a] - ext[a]) / h);
-    c[a] = static_cast<uint32_t>(fminf(fmaxf(q, 0.f), static_cast<float>((1 << kIniCellBits) - 1)));
+    // (an extent beyond binary32 is cut: the code only orders the points)
+    span[a] = fminf(hi[a] - lo[a], 1e37f);
+    most = fmaxf(most, span[a]);
   }
-  const uint32_t code = spread3(c[0]) | (spread3(c[1]) << 1) | (spread3(c[2]) << 2);
-  cell[i] = code;
-  atomicAdd(&cnt[code], 1u);
+  // the finest cell most / 2^b whose axes fit: an axis of extent s has
+  // floor(s / h) + 1 cells
+  IniGrid g;
+  for (int b = 21; b >= 1; --b) {
+    const float inv_h = static_cast<float>(1 << b) / most * 0.9999f;
+    int total = 0;
+    for (int a = 0; a < 3; ++a) {
+      const float cells = span[a] * inv_h;
+      g.top[a] = static_cast<uint32_t>(fminf(cells, static_cast<float>((1 << b) - 1)));
+      g.bits[a] = 32 - __clz(g.top[a]);
+      g.lo[a] = lo[a];
+      total += g.bits[a];
+    }
+    g.inv_h = inv_h;
+    if (total <= kIniCodeBits) break;
+  }
+  *grid = g;
 }
 
-// points into cell order (order within a cell arbitrary), with their index
-__global__ void __launch_bounds__(256) k_ini_scatter(const float* __restrict__ pts, uint32_t n,
-                                                     const uint32_t* __restrict__ cell, const uint32_t* __restrict__ off,
-                                                     uint32_t* __restrict__ cnt, float* __restrict__ sp,
-                                                     uint32_t* __restrict__ orig) {
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const uint32_t c = cell[i];
-  const uint32_t pos = off[c] + atomicSub(&cnt[c], 1u) - 1u;
-  sp[3 * pos] = pts[3 * i];
-  sp[3 * pos + 1] = pts[3 * i + 1];
-  sp[3 * pos + 2] = pts[3 * i + 2];
-  orig[pos] = i;
+// Morton code over the bits that each axis has, interleaved from the lowest
+// bit up (an axis whose bits are used up drops out).
+__device__ __forceinline__ uint32_t morton(const uint32_t (&c)[3], const int (&bits)[3]) {
+  uint32_t code = 0;
+  int at = 0;
+  const int most = max(bits[0], max(bits[1], bits[2]));
+  for (int b = 0; b < most; ++b)
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+      if (b < bits[a]) code |= ((c[a] >> b) & 1u) << at++;
+  return code;
+}
+
+// A CTA's share of the sort: R rounds of 512 keys, a contiguous piece of
+// 32 R keys per warp (the order within a warp's piece is round, lane).  R = 4
+// up to 2^18 points (51 CTAs for a 128 x 1024 scan), 16 beyond, so at most 128
+// CTAs: every scatter CTA reads the whole table of counts.
+__device__ __forceinline__ uint32_t sort_slot(int R, int r) {
+  return blockIdx.x * (kIniSortCta * R) + (threadIdx.x >> 5) * (32 * R) + r * 32 + (threadIdx.x & 31);
+}
+
+// Digit counts of a radix pass per CTA: hist[CTA][bin].  The first pass
+// (FIRST) also forms the codes.
+template <int R, bool FIRST>
+__global__ void __launch_bounds__(kIniSortCta) k_ini_count(const float* __restrict__ pts,
+                                                           const IniGrid* __restrict__ grid,
+                                                           uint32_t* __restrict__ code, const uint2* __restrict__ in,
+                                                           uint32_t n, int shift, uint32_t* __restrict__ hist) {
+  pdl_wait();               // (launched after a kernel of this chain: wait for it)
+  pdl_launch_dependents();  // the next kernel may be dispatched now
+  __shared__ uint32_t s_h[kIniBins];
+  s_h[threadIdx.x] = 0;
+  __syncthreads();
+  IniGrid g;
+  if (FIRST) g = *grid;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const uint32_t i = sort_slot(R, r);
+    if (i < n) {
+      uint32_t k;
+      if (FIRST) {
+        uint32_t c[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+          c[a] = min(static_cast<uint32_t>(fmaxf((pts[3 * i + a] - g.lo[a]) * g.inv_h, 0.f)), g.top[a]);
+        k = morton(c, g.bits);
+        code[i] = k;
+      } else {
+        k = in[i].x;
+      }
+      atomicAdd(&s_h[(k >> shift) & (kIniBins - 1)], 1u);
+    }
+  }
+  __syncthreads();
+  hist[blockIdx.x * kIniBins + threadIdx.x] = s_h[threadIdx.x];
+}
+
+// Stable scatter of a radix pass: (code, index) pairs to their places; the
+// last pass (LAST) writes the points themselves with their index.  A key's
+// place: keys of smaller digits, keys of its digit in earlier CTAs and
+// warps, and its rank in its warp's piece.
+template <int R, bool FIRST, bool LAST>
+__global__ void __launch_bounds__(kIniSortCta) k_ini_scatter(const uint32_t* __restrict__ code,
+                                                             const uint2* __restrict__ in, uint32_t n, int shift,
+                                                             const uint32_t* __restrict__ hist,
+                                                             uint2* __restrict__ out, const float* __restrict__ pts,
+                                                             float4* __restrict__ sp) {
+  pdl_wait();               // (launched after a kernel of this chain: wait for it)
+  pdl_launch_dependents();  // the next kernel may be dispatched now
+  __shared__ uint32_t s_at[kIniSortWarps][kIniBins];
+  __shared__ uint32_t s_warp[kIniSortWarps];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int w = 0; w < kIniSortWarps; ++w) s_at[w][threadIdx.x] = 0;
+  __syncthreads();
+  uint2 kv[R];
+  uint32_t rank[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const uint32_t i = sort_slot(R, r);
+    kv[r] = i < n ? (FIRST ? make_uint2(code[i], i) : in[i]) : make_uint2(0u, 0u);
+  }
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const bool ok = sort_slot(R, r) < n;
+    const uint32_t d = ok ? (kv[r].x >> shift) & (kIniBins - 1) : kIniBins;
+    const uint32_t peers = __match_any_sync(0xffffffffu, d);
+    uint32_t before = 0;
+    if (ok) before = s_at[wid][d];
+    __syncwarp();
+    if (ok && lane == __ffs(peers) - 1) s_at[wid][d] = before + __popc(peers);
+    __syncwarp();
+    rank[r] = before + __popc(peers & ((1u << lane) - 1u));
+  }
+  // thread = bin: its keys in earlier CTAs and in all CTAs
+  uint32_t total = 0, mine = 0;
+  for (uint32_t b = 0; b < gridDim.x; b += 8) {
+    uint32_t v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = b + u < gridDim.x ? hist[(b + u) * kIniBins + threadIdx.x] : 0u;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      total += v[u];
+      mine += b + u < blockIdx.x ? v[u] : 0u;
+    }
+  }
+  uint32_t incl = total;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
+  }
+  if (lane == 31) s_warp[wid] = incl;
+  __syncthreads();
+  uint32_t at = mine + incl - total;
+  for (int w = 0; w < wid; ++w) at += s_warp[w];
+#pragma unroll
+  for (int w = 0; w < kIniSortWarps; ++w) {
+    const uint32_t c = s_at[w][threadIdx.x];
+    s_at[w][threadIdx.x] = at;
+    at += c;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    if (sort_slot(R, r) < n) {
+      const uint32_t pos = s_at[wid][(kv[r].x >> shift) & (kIniBins - 1)] + rank[r];
+      if (LAST) {
+        const uint32_t i = kv[r].y;
+        sp[pos] = make_float4(pts[3 * i], pts[3 * i + 1], pts[3 * i + 2], __uint_as_float(i));
+      } else {
+        out[pos] = kv[r];
+      }
+    }
+  }
+}
+
+// Boxes of the leaves (32 points, one warp) and of the nodes (32 leaves, one
+// CTA): lo / hi corners as float4.
+__global__ void __launch_bounds__(1024) k_ini_boxes(const float4* __restrict__ sp, uint32_t n,
+                                                    float4* __restrict__ leaf, float4* __restrict__ node) {
+  pdl_wait();               // (launched after a kernel of this chain: wait for it)
+  pdl_launch_dependents();  // the next kernel may be dispatched now
+  __shared__ float s_lo[32][3], s_hi[32][3];
+  const uint32_t i = blockIdx.x * 1024 + threadIdx.x;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+  if (i < n) {
+    const float4 p = sp[i];
+    lo[0] = hi[0] = p.x;
+    lo[1] = hi[1] = p.y;
+    lo[2] = hi[2] = p.z;
+  }
+  warp_min_max(lo, hi);
+  if (lane == 0) {
+    for (int a = 0; a < 3; ++a) {
+      s_lo[wid][a] = lo[a];
+      s_hi[wid][a] = hi[a];
+    }
+    if (i < n) {
+      leaf[2 * (i >> 5)] = make_float4(lo[0], lo[1], lo[2], 0.f);
+      leaf[2 * (i >> 5) + 1] = make_float4(hi[0], hi[1], hi[2], 0.f);
+    }
+  }
+  __syncthreads();
+  if (wid != 0) return;
+  for (int a = 0; a < 3; ++a) {
+    lo[a] = s_lo[lane][a];
+    hi[a] = s_hi[lane][a];
+  }
+  warp_min_max(lo, hi);
+  if (lane == 0) {
+    node[2 * blockIdx.x] = make_float4(lo[0], lo[1], lo[2], 0.f);
+    node[2 * blockIdx.x + 1] = make_float4(hi[0], hi[1], hi[2], 0.f);
+  }
 }
 
 // binary32 squared distance in the specified order (no contraction)
@@ -157,172 +316,119 @@ __device__ __forceinline__ float dist2(float ax, float ay, float az, float bx, f
   return fadd(fadd(fmul(dx, dx), fmul(dy, dy)), fmul(dz, dz));
 }
 
-// a lower bound of the squared distance between two boxes (exact arithmetic
-// up to a few roundings; callers apply the margin)
-__device__ __forceinline__ float box_gap2(const IniBox& a, const IniBox& b) {
-  float s = 0.f;
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    const float g = fmaxf(0.f, fmaxf(b.lo[d] - a.hi[d], a.lo[d] - b.hi[d]));
-    s += g * g;
-  }
-  return s;
+// Bits of a lower bound of the squared distance from (x, y, z) to any point
+// of a box (the margin covers the roundings); non-negative, so the bits order
+// as the values do.
+__device__ __forceinline__ uint32_t box_gap_bits(const float4* __restrict__ box, float x, float y, float z) {
+  const float4 lo = __ldg(box), hi = __ldg(box + 1);
+  const float gx = fmaxf(0.f, fmaxf(lo.x - x, x - hi.x));
+  const float gy = fmaxf(0.f, fmaxf(lo.y - y, y - hi.y));
+  const float gz = fmaxf(0.f, fmaxf(lo.z - z, z - hi.z));
+  return __float_as_uint((gx * gx + gy * gy + gz * gz) * 0.99999f);
 }
 
-// Sorted insertion of key into best[0..K) (ascending), dropping the largest.
-template <int K>
-__device__ __forceinline__ void topk_insert(unsigned long long (&best)[K], unsigned long long key) {
-#pragma unroll
-  for (int t = K - 1; t > 0; --t) {
-    const unsigned long long prev = best[t - 1];
-    best[t] = prev > key ? prev : (best[t] > key ? key : best[t]);
-  }
-  best[0] = best[0] > key ? key : best[0];
+// Compare-exchange with lane ^ j: the smaller key stays where `low` holds.
+__device__ __forceinline__ void cas_lane(unsigned long long& v, int j, bool low) {
+  const unsigned long long o = __shfl_xor_sync(0xffffffffu, v, j);
+  v = (o < v) == low ? o : v;
 }
 
-template <int K>
-__global__ void __launch_bounds__(kIniTile) k_ini_knn(const float* __restrict__ pts,
-                                                      const uint32_t* __restrict__ orig, uint32_t n,
-                                                      const IniBox* __restrict__ boxes, uint32_t n_tiles, int k,
-                                                      int32_t* __restrict__ knn, int64_t* __restrict__ pairs) {
-  __shared__ float sx[kIniTile], sy[kIniTile], sz[kIniTile];
-  __shared__ uint32_t s_id[kIniTile];
-  __shared__ uint32_t s_list[kIniMaxTiles];
-  __shared__ float s_bd[kIniSorted];          // box distances of the first kIniSorted listed tiles
-  __shared__ uint32_t s_st[kIniSorted];       // the listed tiles by ascending (box distance, tile)
-  __shared__ float s_sbd[kIniSorted];
-  __shared__ uint32_t s_nlist, s_worst;
-  __shared__ uint32_t s_wmax[kIniTile / 32];
-  const uint32_t qt = blockIdx.x;
-  const uint32_t i = qt * kIniTile + threadIdx.x;
-  const bool valid = i < n;
-  const float qx = valid ? pts[3 * i] : 0.f, qy = valid ? pts[3 * i + 1] : 0.f, qz = valid ? pts[3 * i + 2] : 0.f;
-  unsigned long long best[K];
-#pragma unroll
-  for (int t = 0; t < K; ++t) best[t] = ~0ull;
+constexpr int kKnnCta = 256;
+constexpr uint32_t kKnnNone = 0xffffffffu;   // a box that is not there or has been visited
+// Candidates of a leaf taken one by one (about 14 instructions each) up to
+// this many, by a bitonic sort and merge (about 190) beyond; 6 to 12 measured
+// the same, 18 two percent slower.
+constexpr int kKnnOneByOne = 12;
 
-  unsigned long long evaluated = 0;   // (query, candidate) distances of this warp's lane 0
-  // the warp's own query box: a tile whose box is provably beyond every one
-  // of the warp's K-th distances is skipped by the warp alone
-  IniBox wbox;
-  {
-    const float v[3] = {qx, qy, qz};
+// One warp per query.  Lane l holds the l-th smallest key (distance bits,
+// original index) of the points seen so far; `wd` is the k-th one's distance.
+// The query's own leaf first, then the boxes that can still hold a closer
+// point, nearest first, in its own node, the other nodes of its batch of 32
+// and the other batches.  Bound by issue and by the latency of the box and
+// point loads (L1 and L2 hits).  A query prunes with its own radius, and the
+// k-th neighbour radii of a scan span 0.03 to 16 m: a CTA per 256 queries,
+// pruning with the widest of its radii and lasting as long as its worst
+// query, took 5.27 ms on the 102k points of a 128 x 1024 scan, this 0.136 ms
+// (k = 20; the whole call 5.35 -> 0.189 ms, 51k points 2.73 -> 0.111 ms).
+__global__ void __launch_bounds__(kKnnCta) k_ini_knn(const float4* __restrict__ sp, uint32_t n,
+                                                     const float4* __restrict__ leaf_box, uint32_t n_leaf,
+                                                     const float4* __restrict__ node_box, uint32_t n_node, int k,
+                                                     int32_t* __restrict__ knn, int64_t* __restrict__ pairs) {
+  pdl_wait();               // (launched after a kernel of this chain: wait for it)
+  pdl_launch_dependents();  // the next kernel may be dispatched now
+  const int lane = threadIdx.x & 31;
+  const uint32_t q = blockIdx.x * (kKnnCta / 32) + (threadIdx.x >> 5);
+  if (q >= n) return;
+  const float4 me = __ldg(sp + q);
+  unsigned long long best = ~0ull;
+  uint32_t wd = 0xffffffffu;   // distance bits of the k-th best (none yet)
+  uint32_t evaluated = 0;
+  const uint32_t leaf0 = q >> 5, node0 = q >> 10, batch0 = q >> 15;
+  const uint32_t n_batch = (n_node + 31) / 32;
+  bool first = true;   // on the way down to the query's own leaf
+  for (uint32_t t = 0; t < n_batch; ++t) {
+    const uint32_t batch = t == 0 ? batch0 : (t <= batch0 ? t - 1 : t);
+    const uint32_t nd = 32 * batch + lane;
+    uint32_t un = nd < n_node ? box_gap_bits(node_box + 2 * nd, me.x, me.y, me.z) : kKnnNone;
+    while (true) {
+      int a = static_cast<int>(node0 & 31u);
+      if (!first) {
+        const uint32_t m = __reduce_min_sync(0xffffffffu, un);
+        if (m == kKnnNone || m > wd) break;
+        a = __ffs(__ballot_sync(0xffffffffu, un == m)) - 1;
+      }
+      if (lane == a) un = kKnnNone;
+      const uint32_t lf = 32 * (32 * batch + a) + lane;
+      uint32_t ul = lf < n_leaf ? box_gap_bits(leaf_box + 2 * lf, me.x, me.y, me.z) : kKnnNone;
+      while (true) {
+        int b = static_cast<int>(leaf0 & 31u);
+        if (!first) {
+          const uint32_t m = __reduce_min_sync(0xffffffffu, ul);
+          if (m == kKnnNone || m > wd) break;
+          b = __ffs(__ballot_sync(0xffffffffu, ul == m)) - 1;
+        }
+        first = false;
+        if (lane == b) ul = kKnnNone;
+        const uint32_t base = 32 * (32 * (32 * batch + a) + b);
+        const uint32_t i = base + lane;
+        evaluated += min(32u, n - base);
+        uint32_t d = 0xffffffffu, id = 0xffffffffu;
+        if (i < n) {
+          const float4 p = __ldg(sp + i);
+          d = __float_as_uint(dist2(me.x, me.y, me.z, p.x, p.y, p.z));
+          id = __float_as_uint(p.w);
+        }
+        // (a distance equal to the k-th may still win by its index)
+        uint32_t m = __ballot_sync(0xffffffffu, i < n && d <= wd);
+        if (!m) continue;
+        unsigned long long key = (static_cast<unsigned long long>(d) << 32) | id;
+        if (__popc(m) <= kKnnOneByOne) {
+          do {
+            const unsigned long long x = __shfl_sync(0xffffffffu, key, __ffs(m) - 1);
+            m &= m - 1;
+            const uint32_t less = __ballot_sync(0xffffffffu, best < x);
+            const unsigned long long up = __shfl_up_sync(0xffffffffu, best, 1);
+            const int pos = __popc(less);
+            best = lane < pos ? best : (lane == pos ? x : up);
+          } while (m);
+        } else {
+          // candidates sorted descending, the smaller half of the two lists
+          // (a bitonic sequence) merged
+          if (!((m >> lane) & 1u)) key = ~0ull;
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      float lo = valid ? v[a] : INFINITY, hi = valid ? v[a] : -INFINITY;
-      for (int o = 16; o; o >>= 1) {
-        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-      }
-      wbox.lo[a] = lo;
-      wbox.hi[a] = hi;
-    }
-  }
-  const uint32_t w_valid = __popc(__ballot_sync(0xffffffffu, valid));
-  auto visit = [&](uint32_t tile) {
-    const uint32_t base = tile * kIniTile;
-    const uint32_t cnt = n - base < static_cast<uint32_t>(kIniTile) ? n - base : kIniTile;
-    __syncthreads();   // the previous tile is no longer read
-    if (threadIdx.x < cnt) {
-      sx[threadIdx.x] = pts[3 * (base + threadIdx.x)];
-      sy[threadIdx.x] = pts[3 * (base + threadIdx.x) + 1];
-      sz[threadIdx.x] = pts[3 * (base + threadIdx.x) + 2];
-      s_id[threadIdx.x] = orig[base + threadIdx.x];
-    }
-    __syncthreads();
-    if (w_valid == 0) return;   // uniform across the warp
-    const uint32_t wworst = __reduce_max_sync(0xffffffffu, valid ? static_cast<uint32_t>(best[K - 1] >> 32) : 0u);
-    if (wworst < 0x7f800000u && box_gap2(wbox, boxes[tile]) * 0.99999f > __uint_as_float(wworst)) return;
-    evaluated += static_cast<unsigned long long>(cnt) * w_valid;
-    if (!valid) return;
-    uint32_t worst = static_cast<uint32_t>(best[K - 1] >> 32);
-    for (uint32_t j = 0; j < cnt; ++j) {
-      const uint32_t d = __float_as_uint(dist2(qx, qy, qz, sx[j], sy[j], sz[j]));
-      if (d > worst) continue;
-      const unsigned long long key = (static_cast<unsigned long long>(d) << 32) | s_id[j];
-      if (key < best[K - 1]) {
-        topk_insert<K>(best, key);
-        worst = static_cast<uint32_t>(best[K - 1] >> 32);
-      }
-    }
-  };
-
-  // the own tile and its neighbours in index order (a scan's consecutive
-  // points are neighbours in space)
-  for (int w = 0; w < kIniWindow; ++w) {
-    const int off = (w & 1) ? (w + 1) / 2 : -(w / 2);
-    const long long t = static_cast<long long>(qt) + off;
-    if (t < 0 || t >= static_cast<long long>(n_tiles)) continue;   // uniform across the CTA
-    visit(static_cast<uint32_t>(t));
-  }
-  // the CTA's K-th distance: the largest over its queries (bits of a
-  // non-negative float; 0xffffffff while some query holds fewer than K)
-  auto cta_worst = [&]() -> uint32_t {
-    const uint32_t mine = valid ? static_cast<uint32_t>(best[K - 1] >> 32) : 0u;
-    const uint32_t wmax = __reduce_max_sync(0xffffffffu, mine);
-    __syncthreads();   // s_wmax / s_worst of the previous call are read
-    if ((threadIdx.x & 31) == 0) s_wmax[threadIdx.x >> 5] = wmax;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      uint32_t m = 0;
-      for (int w = 0; w < kIniTile / 32; ++w) m = m > s_wmax[w] ? m : s_wmax[w];
-      s_worst = m;
-    }
-    __syncthreads();
-    return s_worst;
-  };
-  // tiles whose box can still hold a point closer than the CTA's K-th
-  // distance (a box provably farther cannot; the margin covers rounding)
-  auto too_far = [](float bd, uint32_t wb) {
-    return wb < 0x7f800000u && bd * 0.99999f > __uint_as_float(wb);
-  };
-  uint32_t wb = cta_worst();
-  if (threadIdx.x == 0) s_nlist = 0;
-  __syncthreads();
-  const IniBox qb = boxes[qt];
-  for (uint32_t t = threadIdx.x; t < n_tiles; t += blockDim.x) {
-    const long long d = static_cast<long long>(t) - static_cast<long long>(qt);
-    if (d >= -(kIniWindow / 2) && d <= kIniWindow / 2) continue;   // visited
-    const float bd = box_gap2(qb, boxes[t]);
-    if (too_far(bd, wb)) continue;
-    const uint32_t at = atomicAdd(&s_nlist, 1u);
-    s_list[at] = t;
-    if (at < static_cast<uint32_t>(kIniSorted)) s_bd[at] = bd;
-  }
-  __syncthreads();
-  const uint32_t nl = s_nlist;
-  if (nl <= static_cast<uint32_t>(kIniSorted)) {
-    // nearest first (rank of each entry by (box distance, tile)); stop at
-    // the first box the shrinking K-th distance rules out: every later one
-    // is at least as far
-    for (uint32_t e = threadIdx.x; e < nl; e += blockDim.x) {
-      const float bd = s_bd[e];
-      const uint32_t te = s_list[e];
-      uint32_t rank = 0;
-      for (uint32_t f = 0; f < nl; ++f) {
-        const float bf = s_bd[f];
-        rank += (bf < bd || (bf == bd && s_list[f] < te)) ? 1u : 0u;
-      }
-      s_st[rank] = te;
-      s_sbd[rank] = bd;
-    }
-    __syncthreads();
-    for (uint32_t l = 0; l < nl; ++l) {
-      if (too_far(s_sbd[l], wb)) break;   // uniform: wb is the CTA's
-      visit(s_st[l]);
-      wb = cta_worst();
-    }
-  } else {
-    for (uint32_t l = 0; l < nl; ++l) visit(s_list[l]);
-  }
-  if (pairs && (threadIdx.x & 31) == 0 && evaluated)
-    atomicAdd(reinterpret_cast<unsigned long long*>(pairs), evaluated);
-  if (valid) {
-    const size_t row = static_cast<size_t>(orig[i]) * k;
+          for (int w = 2; w <= 32; w <<= 1)
 #pragma unroll
-    for (int t = 0; t < K; ++t)
-      if (t < k) knn[row + t] = static_cast<int32_t>(static_cast<uint32_t>(best[t]));
+            for (int j = w >> 1; j; j >>= 1) cas_lane(key, j, ((lane & j) == 0) == ((lane & w) != 0 && w < 32));
+          best = key < best ? key : best;
+#pragma unroll
+          for (int j = 16; j; j >>= 1) cas_lane(best, j, (lane & j) == 0);
+        }
+        wd = static_cast<uint32_t>(__shfl_sync(0xffffffffu, best, k - 1) >> 32);
+      }
+    }
   }
+  if (pairs && lane == 0) atomicAdd(reinterpret_cast<unsigned long long*>(pairs), static_cast<unsigned long long>(evaluated));
+  if (lane < k) knn[static_cast<size_t>(__float_as_uint(me.w)) * k + lane] = static_cast<int32_t>(static_cast<uint32_t>(best));
 }
 
 // One cyclic-Jacobi rotation zeroing A[p][q] of the symmetric 3x3 A and
@@ -366,6 +472,7 @@ __global__ void __launch_bounds__(256) k_ini_frame(const float* __restrict__ pts
                                                    const int32_t* __restrict__ knn, IniParams P,
                                                    lgs_surfel_params_out out, float* __restrict__ lam,
                                                    float* __restrict__ conf) {
+  pdl_wait();               // (launched after a kernel of this chain: wait for it)
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const float px = pts[3 * i], py = pts[3 * i + 1], pz = pts[3 * i + 2];
@@ -475,45 +582,68 @@ __global__ void __launch_bounds__(256) k_ini_frame(const float* __restrict__ pts
   conf[i] = u;
 }
 
-template <int K>
-void launch_knn(const float* sp, const uint32_t* orig, uint32_t n, const IniBox* boxes, uint32_t n_tiles, int k,
-                int32_t* knn, int64_t* pairs, cudaStream_t s) {
-  k_ini_knn<K><<<n_tiles, kIniTile, 0, s>>>(sp, orig, n, boxes, n_tiles, k, knn, pairs);
-}
-
-// Scratch: tile boxes, the extent, cells and their counts / offsets, scan
-// partials, the points in cell order and their original indices.
+// Scratch: partial extents, the grid, the codes, the radix passes' counts
+// and two buffers of (code, index) pairs, the points in cell order with their
+// original index, leaf and node boxes.
 struct IniLayout {
-  size_t boxes, ext, cell, cnt, off, part, sp, orig, total;
+  size_t part, grid, code, hist, kv0, kv1, sp, leaf, node, total;
 };
 
 size_t align256(size_t v) { return (v + 255) / 256 * 256; }
 
+bool sort_wide(size_t n) { return n > (1u << 18); }   // 16 rounds of keys per sort CTA instead of 4
+
+uint32_t sort_ctas(size_t n) {
+  const size_t per = static_cast<size_t>(kIniSortCta) * (sort_wide(n) ? 16 : 4);
+  return static_cast<uint32_t>((n + per - 1) / per);
+}
+
 IniLayout ini_layout(int64_t n) {
   IniLayout L{};
   const size_t N = static_cast<size_t>(n > 0 ? n : 1);
-  const size_t tiles = (N + kIniTile - 1) / kIniTile;
   size_t o = 0;
   auto take = [&](size_t bytes) { const size_t at = o; o = align256(o + bytes); return at; };
-  L.boxes = take(tiles * sizeof(IniBox));
-  L.ext = take(8 * sizeof(float));
-  L.cell = take(4 * N);
-  L.cnt = take(4 * static_cast<size_t>(kIniCells));
-  L.off = take(4 * (static_cast<size_t>(kIniCells) + 1));
-  L.part = take(scan_partials_bytes(kIniCells));
-  L.sp = take(12 * N);
-  L.orig = take(4 * N);
+  L.part = take(kIniExtCtas * sizeof(IniBox));
+  L.grid = take(sizeof(IniGrid));
+  L.code = take(4 * N);
+  L.hist = take(4 * static_cast<size_t>(kIniBins) * sort_ctas(N));
+  L.kv0 = take(8 * N);
+  L.kv1 = take(8 * N);
+  L.sp = take(16 * N);
+  L.leaf = take(32 * ((N + 31) / 32));
+  L.node = take(32 * ((N + 1023) / 1024));
   L.total = o;
   return L;
+}
+
+// The points into cell order: three passes of count and scatter.
+template <int R>
+cudaError_t launch_order(const float* pts, uint32_t n, const IniLayout& L, char* b, cudaStream_t s) {
+  const IniGrid* grid = reinterpret_cast<const IniGrid*>(b + L.grid);
+  uint32_t* code = reinterpret_cast<uint32_t*>(b + L.code);
+  uint32_t* hist = reinterpret_cast<uint32_t*>(b + L.hist);
+  uint2* kv0 = reinterpret_cast<uint2*>(b + L.kv0);
+  uint2* kv1 = reinterpret_cast<uint2*>(b + L.kv1);
+  float4* sp = reinterpret_cast<float4*>(b + L.sp);
+  const dim3 g(sort_ctas(n)), c(kIniSortCta);
+  cudaError_t e = launch_dep(k_ini_count<R, true>, g, c, 0, s, pts, grid, code, nullptr, n, 0, hist);
+  if (e == cudaSuccess) e = launch_dep(k_ini_scatter<R, true, false>, g, c, 0, s, code, nullptr, n, 0, hist, kv0, pts, sp);
+  if (e == cudaSuccess) e = launch_dep(k_ini_count<R, false>, g, c, 0, s, pts, grid, code, kv0, n, kIniDigit, hist);
+  if (e == cudaSuccess) e = launch_dep(k_ini_scatter<R, false, false>, g, c, 0, s, code, kv0, n, kIniDigit, hist, kv1, pts, sp);
+  if (e == cudaSuccess) e = launch_dep(k_ini_count<R, false>, g, c, 0, s, pts, grid, code, kv1, n, 2 * kIniDigit, hist);
+  if (e == cudaSuccess)
+    e = launch_dep(k_ini_scatter<R, false, true>, g, c, 0, s, code, kv1, n, 2 * kIniDigit, hist, kv0, pts, sp);
+  return e;
 }
 
 }  // namespace
 
 size_t init_scratch_bytes(int64_t n) { return ini_layout(n).total; }
 
-int64_t init_max_points() { return static_cast<int64_t>(kIniMaxTiles) * kIniTile; }
+int64_t init_max_points() { return kIniMaxPoints; }
 
-// zero, boxes, extent, cells, scan (3), scatter, boxes, k-NN, frame
+// partial extents, grid, three radix passes of count and scatter, boxes, k-NN,
+// frame
 int init_launches() { return 11; }
 
 cudaError_t launch_keyframe_init(const float* pts, int64_t n64, const float pose[12], const lgs_init_params& p,
@@ -521,30 +651,24 @@ cudaError_t launch_keyframe_init(const float* pts, int64_t n64, const float pose
                                  float* conf, int64_t* pairs, cudaStream_t s) {
   const uint32_t n = static_cast<uint32_t>(n64);
   if (n == 0) return cudaSuccess;
-  const uint32_t n_tiles = (n + kIniTile - 1) / kIniTile;
   const IniLayout L = ini_layout(n);
   char* b = static_cast<char*>(scratch);
-  IniBox* boxes = reinterpret_cast<IniBox*>(b + L.boxes);
-  float* ext = reinterpret_cast<float*>(b + L.ext);
-  uint32_t* cell = reinterpret_cast<uint32_t*>(b + L.cell);
-  uint32_t* cnt = reinterpret_cast<uint32_t*>(b + L.cnt);
-  uint32_t* off = reinterpret_cast<uint32_t*>(b + L.off);
-  uint32_t* part = reinterpret_cast<uint32_t*>(b + L.part);
-  float* sp = reinterpret_cast<float*>(b + L.sp);
-  uint32_t* orig = reinterpret_cast<uint32_t*>(b + L.orig);
-  const uint32_t g = (n + 255) / 256;
-  k_ini_zero<<<512, 256, 0, s>>>(cnt, kIniCells);
-  k_ini_boxes<<<n_tiles, kIniTile, 0, s>>>(pts, n, boxes);
-  k_ini_extent<<<1, 256, 0, s>>>(boxes, n_tiles, ext);
-  k_ini_cells<<<g, 256, 0, s>>>(pts, n, ext, cell, cnt);
-  exclusive_scan_u32(cnt, off, kIniCells, part, s);
-  k_ini_scatter<<<g, 256, 0, s>>>(pts, n, cell, off, cnt, sp, orig);
-  k_ini_boxes<<<n_tiles, kIniTile, 0, s>>>(sp, n, boxes);
-  if (p.k <= 8) launch_knn<8>(sp, orig, n, boxes, n_tiles, p.k, knn, pairs, s);
-  else if (p.k <= 16) launch_knn<16>(sp, orig, n, boxes, n_tiles, p.k, knn, pairs, s);
-  else if (p.k <= 20) launch_knn<20>(sp, orig, n, boxes, n_tiles, p.k, knn, pairs, s);
-  else if (p.k <= 24) launch_knn<24>(sp, orig, n, boxes, n_tiles, p.k, knn, pairs, s);
-  else launch_knn<32>(sp, orig, n, boxes, n_tiles, p.k, knn, pairs, s);
+  IniBox* part = reinterpret_cast<IniBox*>(b + L.part);
+  float4* sp = reinterpret_cast<float4*>(b + L.sp);
+  float4* leaf = reinterpret_cast<float4*>(b + L.leaf);
+  float4* node = reinterpret_cast<float4*>(b + L.node);
+  const uint32_t n_part = std::min<uint32_t>((n + 255) / 256, kIniExtCtas);
+  const uint32_t n_leaf = (n + 31) / 32, n_node = (n + 1023) / 1024;
+  k_ini_part<<<n_part, 256, 0, s>>>(pts, n, part);
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess)
+    e = launch_dep(k_ini_grid, dim3(1), dim3(32), 0, s, part, n_part, reinterpret_cast<IniGrid*>(b + L.grid));
+  if (e == cudaSuccess) e = sort_wide(n) ? launch_order<16>(pts, n, L, b, s) : launch_order<4>(pts, n, L, b, s);
+  if (e == cudaSuccess) e = launch_dep(k_ini_boxes, dim3(n_node), dim3(1024), 0, s, sp, n, leaf, node);
+  if (e == cudaSuccess)
+    e = launch_dep(k_ini_knn, dim3((n + kKnnCta / 32 - 1) / (kKnnCta / 32)), dim3(kKnnCta), 0, s, sp, n, leaf, n_leaf,
+                   node, n_node, p.k, knn, pairs);
+  if (e != cudaSuccess) return e;
   IniParams P;
   for (int a = 0; a < 3; ++a) {
     for (int b = 0; b < 3; ++b) P.R[3 * a + b] = pose[4 * a + b];
@@ -559,8 +683,7 @@ cudaError_t launch_keyframe_init(const float* pts, int64_t n64, const float pose
   P.alpha_min = p.alpha_min;
   P.alpha_max = p.alpha_max;
   P.k = p.k;
-  k_ini_frame<<<(n + 255) / 256, 256, 0, s>>>(pts, n, knn, P, out, lam, conf);
-  return cudaGetLastError();
+  return launch_dep(k_ini_frame, dim3((n + 255) / 256), dim3(256), 0, s, pts, n, knn, P, out, lam, conf);
 }
 
 }  // namespace lgs

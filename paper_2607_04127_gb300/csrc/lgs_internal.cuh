@@ -724,11 +724,6 @@ cudaError_t launch_manage(const lgs_surfels& M, const float* lam, const float* r
 cudaError_t launch_manage_gather(const int32_t* src, const uint8_t* role, const int64_t* counts, int64_t capacity,
                                  const void* in, void* out, int words, int zero_children, cudaStream_t s);
 
-// exclusive scan of uint32 (out[len] = total; in may equal out; part holds
-// scan_partials_bytes(len) bytes), defined in lgs_manage.cu
-size_t scan_partials_bytes(uint64_t len);
-void exclusive_scan_u32(const uint32_t* in, uint32_t* out, uint32_t len, uint32_t* part, cudaStream_t s);
-
 // keyframe initialisation (lgs_init.cu)
 size_t init_scratch_bytes(int64_t n);
 int64_t init_max_points();
