@@ -120,6 +120,7 @@ lgs_status check_maps(const lgs_surfels* maps, int n_maps, const int32_t* frame_
 
 struct Plan {
   int64_t n_items = 0, n_surf = 0;
+  int64_t max_n = 0;   // surfels of the largest map a frame renders
   uint32_t n_tiles = 0;
   uint32_t table_floats = 0;
   uint32_t tile_pixels = 0;
@@ -171,6 +172,7 @@ lgs_status build_desc(const lgs_surfels* maps, int n_maps, const lgs_frame* fram
     }
     tiles += static_cast<uint64_t>(D.ntr) * D.ntc;
     items += static_cast<uint64_t>(maps[m].n);
+    if (maps[m].n > p.max_n) p.max_n = maps[m].n;
     d.m[m].n_frames += 1;
   }
   if (tiles >= (1ull << 31)) return fail(LGS_ERR_INVALID_ARG, "too many tiles (%llu)", (unsigned long long)tiles);
@@ -225,7 +227,8 @@ Layout make_layout(int64_t items, uint32_t tiles, int64_t pairs_cap, uint32_t ta
   L.ckpt = take(sizeof(float) * lgs::kCkptSlots * static_cast<size_t>(tile_pixels) * static_cast<size_t>(C));
   L.csuf = take(sizeof(float) * static_cast<size_t>(tile_pixels) * static_cast<size_t>(C));
   L.cmask = take(sizeof(uint32_t) * 4 * static_cast<size_t>(tile_pixels) * static_cast<size_t>(C));
-  L.midl = take(4 * T);
+  // a bucket of n > 2048 keys has ceil(n / 1024) < n / 512 groups at most
+  L.groups = take(sizeof(uint2) * (P / 512 + 1));
   // backward queues: class 0 takes at most every (chunk, warp block) item,
   // every other class at most one item per (tile, warp block)
   const size_t blocks = tile_pixels >= 32 ? tile_pixels / 32 : 1;
@@ -444,7 +447,9 @@ lgs_status lgs_session_create(int device, size_t hbm_budget_bytes, lgs_session* 
     return cuda_fail(e, "session create");
   }
   memset(s->h_status, 0, sizeof(Status));
-  if ((e = cudaStreamCreateWithFlags(&s->side.s, cudaStreamNonBlocking)) != cudaSuccess ||
+  int prio_low = 0, prio_high = 0;
+  if ((e = cudaDeviceGetStreamPriorityRange(&prio_low, &prio_high)) != cudaSuccess ||
+      (e = cudaStreamCreateWithPriority(&s->side.s, cudaStreamNonBlocking, prio_high)) != cudaSuccess ||
       (e = cudaEventCreateWithFlags(&s->side.fork, cudaEventDisableTiming)) != cudaSuccess ||
       (e = cudaEventCreateWithFlags(&s->side.join, cudaEventDisableTiming)) != cudaSuccess) {
     lgs_session_destroy(s);
@@ -719,10 +724,10 @@ lgs_status lgs_bin_sort_batch(lgs_session s, const lgs_surfels* maps, int n_maps
     s->g13_zero_off = L.g13;
   }
   if ((e = write_desc(s, *s->desc, w.desc, cs, s->launches)) != cudaSuccess) return cuda_fail(e, "write_desc");
-  if ((e = timed(s, LGS_TIME_BIN, cs, [&] { return lgs::launch_bin(L, w, n_frames, p.n_items, p.n_tiles, s->side, cs); })) !=
+  if ((e = timed(s, LGS_TIME_BIN, cs, [&] { return lgs::launch_bin(L, w, n_frames, p.n_items, p.max_n, p.n_tiles, s->side, cs); })) !=
       cudaSuccess)
     return cuda_fail(e, "bin");
-  s->launches += lgs::bin_kernel_count(p.n_tiles);
+  s->launches += lgs::bin_kernel_count(p.n_tiles, p.max_n);
   s->lay = L;
   s->binned = true;
   s->ckpt_valid = false;

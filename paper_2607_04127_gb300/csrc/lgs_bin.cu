@@ -11,17 +11,15 @@
 //   k_tile_scan   one CTA: exclusive scan of the tile counts -> every tile's
 //                 [start, end) and its fill cursor; capacity check; the
 //                 longest-first tile order of the persistent kernels; the
-//                 lists of tiles longer than kLongList, 2048 and 1024 keys
+//                 list of tiles longer than kLongList
 //   k_emit        every item appends (depth key << 32 | item) to the bucket
 //                 of each tile of its stored set (order inside a bucket
 //                 arbitrary)
-//   k_tile_sort_all
-//                 sort every bucket of up to 2048 keys by the 64-bit key in
-//                 one launch: up to 1024 keys by a merge sort on half a CTA,
-//                 up to 2048 on a whole CTA; then write the item list
-//   k_sort_long   longer buckets, one 1024-thread CTA each, longest first:
-//                 8192-key chunks sorted in shared memory, merged pairwise
-//                 through global memory; then the item list
+//   k_long_split  buckets of more than 2048 keys: partitioned by depth into
+//                 groups of about 1024 keys, one CTA per bucket, longest first
+//   k_tile_sort   sort every shorter bucket and every group by the 64-bit key,
+//                 one CTA each, by distribution in shared memory; write the
+//                 item list
 // The result is the order of the key (tile, depth, item): per tile, by depth,
 // ties by item index.
 #include <cuda_runtime.h>
@@ -75,8 +73,8 @@ __global__ void k_tables(const Desc* __restrict__ D, float* __restrict__ tab, St
     st->count_ticket = 0;
     st->n_long = 0;
     st->n_big = 0;
-    st->n_mid = 0;
     st->long_sort_counter = 0;
+    st->n_groups = 0;
     st->long_counter_fwd = 0;
     st->long_counter_bwd = 0;
     st->long_done_fwd = 0;
@@ -349,19 +347,17 @@ constexpr uint32_t kLenCache = 4096;   // tiles whose list length the scan keeps
 
 // Bucket of a tile list length for the longest-first order: floor(log2(n)) + 1
 // (0 for an empty tile), reversed so that bucket 0 holds the longest lists.
-// Buckets of up to kMergeMax keys take the merge sort (one CTA per tile, all
-// in one launch: a bucket's sort is a long serial chain, so every bucket
-// runs concurrently); longer ones k_sort_long, in this longest-first order.
-constexpr int kMergeMax = 2048;
-constexpr int kMergeSmall = 1024;   // buckets up to this size: the 128-thread merge sort
+// Buckets of up to kSortMax keys are sorted in shared memory by one CTA;
+// longer ones split into groups first (k_long_split), in this longest-first
+// order.
+constexpr uint32_t kSortMax = 2048;
 constexpr int kOrderBuckets = 33;
 __device__ __forceinline__ int order_bucket(uint32_t n) { return kOrderBuckets - 1 - (n ? 32 - __clz(n) : 0); }
 
 __global__ void __launch_bounds__(kScanCta) k_tile_scan(uint32_t* __restrict__ tcur, uint32_t n_tiles,
                                                           uint2* __restrict__ ranges, Status* __restrict__ st,
                                                           int64_t cap, uint32_t* __restrict__ order,
-                                                          uint32_t* __restrict__ longt, uint32_t* __restrict__ cbase,
-                                                          uint32_t* __restrict__ midl) {
+                                                          uint32_t* __restrict__ longt, uint32_t* __restrict__ cbase) {
   pdl_wait();               // (launched after a kernel of this chain: wait for it)
   pdl_launch_dependents();  // the next kernel may be dispatched now
   __shared__ unsigned long long s_w[32];
@@ -496,10 +492,8 @@ __global__ void __launch_bounds__(kScanCta) k_tile_scan(uint32_t* __restrict__ t
     pos = __shfl_sync(0xffffffffu, pos, leader) + __popc(peers & ((1u << lane) - 1u));
     if (b >= 0) order[pos] = t;
     if (len > kLongList) longt[atomicAdd(&st->n_long, 1u)] = t;
-    // buckets beyond the merge sort (k_sort_long's, found through the
-    // order); those beyond the 128-thread merge sort, for its 256-thread form
-    if (len > kMergeMax) atomicAdd(&st->n_big, 1u);
-    if (len > kMergeSmall && len <= kMergeMax) midl[atomicAdd(&st->n_mid, 1u)] = t;
+    // k_long_split's buckets (found through the order)
+    if (len > kSortMax) atomicAdd(&st->n_big, 1u);
   }
 }
 
@@ -587,141 +581,220 @@ __global__ void __launch_bounds__(256) k_emit(const Desc* __restrict__ D, const 
 // ---------------------------------------------------------------------------
 // Per-tile sort
 // ---------------------------------------------------------------------------
-// ---- buckets of at most 2048 keys: merge sort in shared memory -----------
-// Every thread sorts 8 keys in registers (a 19-comparator network), then
-// runs of 8, 16, ... keys are merged pairwise until one run remains: each
-// thread finds where its 8 outputs start in its pair of runs by a binary
-// search along the merge path (ties, which only the padding has, go to the
-// first run) and merges them sequentially.  The bucket is padded with +inf to
-// a whole number N of 8-key rows; a pass's last runs may be shorter than L.
+// ---- up to 2048 keys in shared memory: distribution sort --------------------
+// The depths of a bucket are spread by an estimate of their rank: 256 coarse
+// bins linear in the depth bits are counted, and inside its coarse bin a key
+// takes the linearly interpolated one of as many fine bins as the bin has
+// keys (about one key per fine bin unless the depths cluster far below a
+// coarse bin's width).  Both maps are monotone in the depth, so the keys of
+// one fine bin are adjacent in the result: they are placed together and each
+// finds its rank by comparing the 64-bit keys of its bin.  A bucket with more
+// than kDense keys in one fine bin (mostly equal depths) takes a bitonic sort
+// in place instead.  Bound by issue and by its nine barriers, at about 60
+// instructions per key; a merge sort, one pass per doubling, took 28 us on the
+// street frame (1.27 M keys in 1,916 buckets) and 524 us on 8 keyframes of a
+// 1M map (21.6 M keys in buckets up to 2,048), this 18 and 113 us.
+constexpr int kSortCta = 256;
+constexpr int kSortPer = kSortMax / kSortCta;
+constexpr uint32_t kCoarse = 256;
+constexpr uint32_t kDense = 64;
+static_assert(kCoarse == kSortCta && kSortPer == 8, "one coarse bin per thread, eight fine bins per thread");
 
-__device__ __forceinline__ void cas_reg(unsigned long long& a, unsigned long long& b) {
-  const unsigned long long x = a, y = b;
-  const bool sw = x > y;
-  a = sw ? y : x;
-  b = sw ? x : y;
-}
+struct SortSmem {
+  unsigned long long key[kSortMax];
+  alignas(16) uint32_t fine[kSortMax + 4];
+  uint32_t coarse[kCoarse + 1];
+  uint32_t red[4][kSortCta / 32];
+};
 
-__device__ __forceinline__ void sort8(unsigned long long (&k)[8]) {
-  // Batcher's odd-even merge network for 8 inputs (19 comparators)
-  cas_reg(k[0], k[1]); cas_reg(k[2], k[3]); cas_reg(k[4], k[5]); cas_reg(k[6], k[7]);
-  cas_reg(k[0], k[2]); cas_reg(k[1], k[3]); cas_reg(k[4], k[6]); cas_reg(k[5], k[7]);
-  cas_reg(k[1], k[2]); cas_reg(k[5], k[6]);
-  cas_reg(k[0], k[4]); cas_reg(k[1], k[5]); cas_reg(k[2], k[6]); cas_reg(k[3], k[7]);
-  cas_reg(k[2], k[4]); cas_reg(k[3], k[5]);
-  cas_reg(k[1], k[2]); cas_reg(k[3], k[4]); cas_reg(k[5], k[6]);
-}
-
-// Shared-memory index of key x: one padding slot after every 8 keys, so the
-// 8-key rows of consecutive threads start in different banks.
-__device__ __forceinline__ uint32_t pad8(uint32_t x) { return x + (x >> 3); }
-
-// Barrier of the threads sorting one bucket: the whole CTA (id 0), or one
-// half of it (ids 1, 2 with 128 threads each), so that the two halves of a
-// CTA sort two buckets independently.
-template <int ID>
-__device__ __forceinline__ void part_sync(uint32_t nthr) {
-  if (ID == 0) __syncthreads();
-  else asm volatile("bar.sync %0, %1;" ::"n"(ID), "r"(nthr) : "memory");
-}
-
-// The n <= 8 * nthr keys g[0, n) sorted by threads t = 0 .. nthr - 1 of one
-// part of a CTA (barrier BAR) in sa / sb (pad8 of 8 * nthr keys each);
-// returns the buffer that holds them (key i at pad8(i)), after a barrier.
-template <int BAR>
-__device__ __forceinline__ unsigned long long* smem_merge_sort(const unsigned long long* __restrict__ g, uint32_t n,
-                                                               unsigned long long* sa, unsigned long long* sb,
-                                                               uint32_t t, uint32_t nthr) {
-  const uint32_t N = n > 8 ? (n + 7u) & ~7u : 8u;   // padded to whole 8-key rows only
-  for (uint32_t i = t; i < N; i += nthr) sa[pad8(i)] = i < n ? g[i] : ~0ull;
-  part_sync<BAR>(nthr);
-  const bool act = 8 * t < N;
-  if (act) {
-    unsigned long long k[8];
-#pragma unroll
-    for (int r = 0; r < 8; ++r) k[r] = sa[9 * t + r];
-    sort8(k);
-#pragma unroll
-    for (int r = 0; r < 8; ++r) sa[9 * t + r] = k[r];
+// A depth's coarse bin and its place inside it ([0, 1] up to rounding): the
+// depth bits above `lo`, scaled to the number of bins.
+struct DepthMap {
+  uint32_t lo;
+  float scale;
+  uint32_t last;   // the last bin
+  __device__ __forceinline__ DepthMap(uint32_t lo_, uint32_t hi, uint32_t bins)
+      : lo(lo_), scale(static_cast<float>(bins) / (static_cast<float>(hi - lo_) + 1.0f)), last(bins - 1) {}
+  __device__ __forceinline__ uint32_t bin(uint32_t d, float& frac) const {
+    // (rounded operations: every call gives a depth the same bin)
+    const float x = fmul(static_cast<float>(d - lo), scale);
+    const uint32_t c = min(static_cast<uint32_t>(x), last);
+    frac = fsub(x, static_cast<float>(c));
+    return c;
   }
-  // a pass over runs of L keys reads only the 2 L keys of its thread group's
-  // pair of runs: up to L = 128 those are the 256 keys of the thread's own
-  // warp, so the passes before it need only a warp barrier
-  __syncwarp();
-  unsigned long long *src = sa, *dst = sb;
-  for (uint32_t L = 8; L < N; L <<= 1) {
-    if (act) {
-      const uint32_t tpp = L / 4;                  // threads per pair of runs
-      const uint32_t pair = t / tpp, d = 8 * (t % tpp);
-      // runs A = [a0, a0 + la), B = [b0, b0 + lb): L keys each, the last
-      // ones shorter (B empty when A is the last run)
-      const uint32_t a0 = 2 * L * pair, b0 = a0 + L;
-      const uint32_t la = min(L, N - a0), lb = b0 < N ? min(L, N - b0) : 0u;
-      // i = number of the first d outputs taken from A
-      uint32_t lo = d > lb ? d - lb : 0, hi = d < la ? d : la;
-      while (lo < hi) {
-        const uint32_t mid = (lo + hi) >> 1;
-        if (src[pad8(a0 + mid)] > src[pad8(b0 + d - mid - 1)]) hi = mid;
-        else lo = mid + 1;
-      }
-      uint32_t i = lo, j = d - lo;
-      const uint32_t o = 9 * (a0 / 8 + d / 8);        // pad8 of the 8-aligned output row
+  // Estimated rank from the bins' exclusive counts: monotone in d.
+  __device__ __forceinline__ uint32_t rank(uint32_t d, const uint32_t* start) const {
+    float frac;
+    const uint32_t c = bin(d, frac);
+    const uint32_t b = start[c], m = start[c + 1] - b;
+    return b + min(static_cast<uint32_t>(fmul(frac, static_cast<float>(m))), m - 1u);
+  }
+};
+
+// Exclusive prefix of v over the CTA (kSortCta threads); s_w: a word per
+// warp.  Holds one barrier.
+__device__ __forceinline__ uint32_t cta_exclusive(uint32_t v, uint32_t* s_w) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  uint32_t incl = v;
 #pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        // ties (only the +inf padding) go to A first, as in the search
-        const unsigned long long a = i < la ? src[pad8(a0 + i)] : ~0ull, b = j < lb ? src[pad8(b0 + j)] : ~0ull;
-        const bool takeA = j >= lb || (i < la && a <= b);
-        dst[o + r] = takeA ? a : b;
-        i += takeA;
-        j += !takeA;
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += y;
+  }
+  if (lane == 31) s_w[wid] = incl;
+  __syncthreads();
+  uint32_t base = incl - v;
+#pragma unroll
+  for (int w = 0; w < kSortCta / 32; ++w) base += w < wid ? s_w[w] : 0u;
+  return base;
+}
+
+// Ascending bitonic sort of key[0, n) in shared memory, n <= kSortMax, padded
+// with the largest key.  Every thread of the CTA calls it.
+__device__ __noinline__ void smem_bitonic(unsigned long long* key, uint32_t n) {
+  uint32_t N = 2;
+  while (N < n) N <<= 1;
+  for (uint32_t i = n + threadIdx.x; i < N; i += kSortCta) key[i] = ~0ull;
+  __syncthreads();
+  for (uint32_t w = 2; w <= N; w <<= 1)
+    for (uint32_t j = w >> 1; j; j >>= 1) {
+      for (uint32_t t = threadIdx.x; t < N / 2; t += kSortCta) {
+        const uint32_t i = 2 * t - (t & (j - 1)), o = i + j;   // (bit j of i is clear)
+        const unsigned long long a = key[i], b = key[o];
+        if ((a > b) == ((i & w) == 0)) {
+          key[i] = b;
+          key[o] = a;
+        }
       }
+      __syncthreads();
     }
-    if (2 * L <= 128) __syncwarp();
-    else part_sync<BAR>(nthr);
-    unsigned long long* tmp = src;
-    src = dst;
-    dst = tmp;
+}
+
+// The n <= kSortMax keys get(0) .. get(n - 1) sorted, their items written to
+// out (get may read what out overwrites: every key is read first).  Called by
+// the whole CTA; the caller separates two calls by a barrier.
+template <class Get>
+__device__ __forceinline__ void sort_small(const Get& get, uint32_t n, uint32_t* out, SortSmem& s) {
+  const uint32_t t = threadIdx.x;
+  const int wid = t >> 5;
+  unsigned long long k[kSortPer];
+  uint32_t lo = ~0u, hi = 0u;
+#pragma unroll
+  for (int r = 0; r < kSortPer; ++r) {
+    const uint32_t i = r * kSortCta + t;
+    if (i < n) {
+      k[r] = get(i);
+      lo = min(lo, static_cast<uint32_t>(k[r] >> 32));
+      hi = max(hi, static_cast<uint32_t>(k[r] >> 32));
+    }
   }
-  part_sync<BAR>(nthr);   // the result is read from every warp's keys
-  return src;
+  for (uint32_t i = t; i < n; i += kSortCta) s.fine[i] = 0u;
+  s.coarse[t] = 0u;
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  if ((t & 31) == 0) {
+    s.red[0][wid] = lo;
+    s.red[1][wid] = hi;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kSortCta / 32; ++w) {
+    lo = min(lo, s.red[0][w]);
+    hi = max(hi, s.red[1][w]);
+  }
+  const DepthMap map(lo, hi, kCoarse);
+#pragma unroll
+  for (int r = 0; r < kSortPer; ++r)
+    if (r * kSortCta + t < n) {
+      float frac;
+      atomicAdd(&s.coarse[map.bin(static_cast<uint32_t>(k[r] >> 32), frac)], 1u);
+    }
+  __syncthreads();
+  const uint32_t base = cta_exclusive(s.coarse[t], s.red[2]);
+  s.coarse[t] = base;   // (every thread has read its own count only)
+  if (t == 0) s.coarse[kCoarse] = n;
+  __syncthreads();
+  uint32_t fo[kSortPer];   // fine bin and the key's place among the bin's arrivals
+#pragma unroll
+  for (int r = 0; r < kSortPer; ++r)
+    if (r * kSortCta + t < n) {
+      const uint32_t f = map.rank(static_cast<uint32_t>(k[r] >> 32), s.coarse);
+      fo[r] = f | (atomicAdd(&s.fine[f], 1u) << 16);
+    }
+  __syncthreads();
+  uint32_t v[8], sum = 0u, most = 0u;
+  uint4* f4 = reinterpret_cast<uint4*>(s.fine) + 2 * t;
+  if (8 * t < n) {
+    const uint4 a = f4[0], b = f4[1];
+    const uint32_t x[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      v[j] = 8 * t + j < n ? x[j] : 0u;   // (words past n are not set)
+      sum += v[j];
+      most = max(most, v[j]);
+    }
+  }
+  uint32_t at = cta_exclusive(sum, s.red[3]);
+  if (8 * t < n) {
+    uint32_t e[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      e[j] = at;
+      at += v[j];
+    }
+    f4[0] = make_uint4(e[0], e[1], e[2], e[3]);
+    f4[1] = make_uint4(e[4], e[5], e[6], e[7]);
+    if (8 * t + 8 >= n) s.fine[n] = n;
+  }
+  const bool dense = __syncthreads_or(most > kDense);
+#pragma unroll
+  for (int r = 0; r < kSortPer; ++r)
+    if (r * kSortCta + t < n) s.key[s.fine[fo[r] & 0xffffu] + (fo[r] >> 16)] = k[r];
+  __syncthreads();
+  if (dense) {
+    smem_bitonic(s.key, n);
+    for (uint32_t i = t; i < n; i += kSortCta) out[i] = static_cast<uint32_t>(s.key[i]);
+    return;
+  }
+  for (uint32_t i = t; i < n; i += kSortCta) {
+    const unsigned long long x = s.key[i];
+    const uint32_t f = map.rank(static_cast<uint32_t>(x >> 32), s.coarse);
+    const uint32_t b = s.fine[f], e = s.fine[f + 1];
+    uint32_t pos = b;
+    if (e - b > 1)
+      for (uint32_t j = b; j < e; ++j) pos += s.key[j] < x;
+    out[pos] = static_cast<uint32_t>(x);
+  }
 }
 
-// One bucket of at most 8 * nthr keys: sorted in shared memory, its item list
-// written.
-template <int BAR>
-__device__ __forceinline__ void merge_sort_bucket(uint32_t tile, const uint2* __restrict__ ranges,
-                                                  const unsigned long long* __restrict__ pkey,
-                                                  uint32_t* __restrict__ pv, unsigned long long* sa,
-                                                  unsigned long long* sb, uint32_t t, uint32_t nthr) {
-  const uint2 rg = ranges[tile];
-  const uint32_t n = rg.y - rg.x;
-  const unsigned long long* src = smem_merge_sort<BAR>(pkey + rg.x, n, sa, sb, t, nthr);
-  for (uint32_t i = t; i < n; i += nthr) pv[rg.x + i] = static_cast<uint32_t>(src[pad8(i)]);
-}
+// ---- buckets beyond 2048 keys: partitioned into groups ------------------------
+// k_long_split: one CTA takes a bucket (claimed in the tile scan's
+// longest-first order).  The depth map above with kLongCoarse bins estimates
+// every key's rank, and the keys of one group of 2^sh estimated ranks (1,024,
+// more beyond 2 M keys) are scattered to one range of a second key buffer made
+// of the pair-tile and item arrays (high and low 32 bits; the pair tiles are
+// rewritten on request only).  Then k_tile_sort sorts the groups of all
+// buckets, one CTA each, like short buckets.  The split is a few reads of the keys
+// by 1,024 threads, short even for the longest bucket, and everything after
+// it is spread over the chip; one CTA per bucket, merging chunks through
+// global memory, was bound by the longest bucket's serial passes (6 maps with
+// buckets up to 292 k keys, 28.9 M long keys: 3.49 -> 0.58 + 0.27 ms; 8
+// keyframes of a 1M map, 25.6 M long keys: 1.04 -> 0.18 + 0.25 ms).  A group of more than kSortMax keys (depths
+// that cluster far below a bin's width) is sorted by its CTA with sorted
+// chunks and merge passes through global memory.
+constexpr int kLongCta = 1024;
+constexpr uint32_t kLongCoarse = 2048;
+constexpr uint32_t kMaxGroups = 2048;
+constexpr uint32_t kGroupBits = 10;
+static_assert(kLongCoarse == 2 * kLongCta && kMaxGroups == 2 * kLongCta, "two bins or groups per thread");
 
-// ---- buckets beyond 2048 keys: one CTA each, merged through global memory --
-// A long bucket is sorted by one CTA of kLongSortCta threads: chunks of
-// kLongChunk keys in shared memory (smem_merge_sort), then passes that merge
-// pairs of sorted runs into runs twice as long, ping-ponging between the key
-// array and a second buffer made of the pair-tile and item arrays (high and
-// low 32 bits of each key; the pair tiles are rewritten on request only, and
-// the item list is the keys' low half, so a result left there is already the
-// list).  A pass writes its output in tiles of kLongChunk keys: the tile's
-// first and last merge-path diagonals are found by binary searches in global
-// memory (one per thread, for up to kLongSortCta tiles at once), its two input
-// ranges loaded into shared memory, and every thread merges its 8 outputs.
-// O(n log n) per bucket instead of the bitonic network's O(n log^2 n).
-constexpr int kLongSortCta = 1024;
-constexpr uint32_t kLongChunk = 8 * kLongSortCta;   // 8192 keys
-constexpr size_t kLongSortSmem = 2 * sizeof(unsigned long long) * (kLongChunk + kLongChunk / 8) +
-                                 sizeof(uint32_t) * (kLongSortCta + 1);   // two key buffers, the diagonals
-
-// A bucket's keys: 64-bit words, or split into high and low 32-bit halves.
+// A bucket's keys: 64-bit words, or split into high and low 32-bit halves
+// (read from L2: the CTA rewrites them).
 struct KeyBuf {
   unsigned long long* k;
   uint32_t *hi, *lo;
   __device__ __forceinline__ unsigned long long get(uint32_t i) const {
-    return k ? k[i] : (static_cast<unsigned long long>(hi[i]) << 32) | lo[i];
+    return k ? __ldcg(k + i) : (static_cast<unsigned long long>(__ldcg(hi + i)) << 32) | __ldcg(lo + i);
   }
   __device__ __forceinline__ void put(uint32_t i, unsigned long long v) const {
     if (k) {
@@ -746,139 +819,224 @@ __device__ __forceinline__ uint32_t path_split(const KeyBuf& X, uint32_t a0, uin
   return lo;
 }
 
-__global__ void __launch_bounds__(kLongSortCta) k_sort_long(const uint2* __restrict__ ranges,
-                                                             Status* __restrict__ st,
-                                                             const uint32_t* __restrict__ order,
-                                                             uint32_t n_tiles, unsigned long long* __restrict__ pkey,
-                                                             uint32_t* __restrict__ ptile, uint32_t* __restrict__ pv) {
-  extern __shared__ __align__(16) unsigned long long s_long[];
-  unsigned long long* sa = s_long;
-  unsigned long long* sb = s_long + kLongChunk + kLongChunk / 8;
-  uint32_t* s_split = reinterpret_cast<uint32_t*>(sb + kLongChunk + kLongChunk / 8);
-  __shared__ uint32_t s_claim;
+// The n keys of Y sorted by one CTA, their items left in Y.lo: chunks of
+// kSortMax keys sorted in shared memory into X, then passes that merge pairs
+// of runs, ping-ponging between X and Y, in output tiles of kSortMax keys (the
+// tiles' first merge-path diagonals found by binary searches, one per thread,
+// their two input ranges loaded into shared memory, eight outputs merged per
+// thread).
+__device__ __noinline__ void merge_sort_global(const KeyBuf& X, const KeyBuf& Y, uint32_t n, SortSmem& s) {
+  const uint32_t t = threadIdx.x;
+  unsigned long long* sa = s.key;
+  uint32_t* s_split = s.fine;   // kSortCta + 1 words
+  for (uint32_t c0 = 0; c0 < n; c0 += kSortMax) {
+    const uint32_t m = min(kSortMax, n - c0);
+    for (uint32_t i = t; i < m; i += kSortCta) sa[i] = Y.get(c0 + i);
+    __syncthreads();
+    smem_bitonic(sa, m);
+    for (uint32_t i = t; i < m; i += kSortCta) X.put(c0 + i, sa[i]);
+    __syncthreads();
+  }
+  bool in_x = true;
+  for (uint32_t R = kSortMax; R < n; R <<= 1) {
+    const KeyBuf& S = in_x ? X : Y;
+    const KeyBuf& Dst = in_x ? Y : X;
+    const uint32_t n_out = (n + kSortMax - 1) / kSortMax;   // output tiles (a run pair holds whole tiles)
+    for (uint32_t q0 = 0; q0 < n_out; q0 += kSortCta) {
+      // first diagonal of output tiles q0 + t (and the end of the last one)
+      __syncthreads();
+      for (uint32_t q = q0 + t; q <= min(q0 + kSortCta, n_out); q += kSortCta) {
+        const uint32_t o = min(q * kSortMax, n);
+        uint32_t p = o / (2 * R);
+        if (o == n && o % (2 * R) == 0 && o > 0) --p;   // the end diagonal of the last pair
+        const uint32_t a0 = 2 * R * p, la = min(R, n - a0), b0 = a0 + R;
+        const uint32_t lb = b0 < n ? min(R, n - b0) : 0u;
+        s_split[q - q0] = path_split(S, a0, la, b0, lb, o - a0);
+      }
+      __syncthreads();
+      const uint32_t q1 = min(q0 + kSortCta, n_out);
+      for (uint32_t q = q0; q < q1; ++q) {
+        const uint32_t o = q * kSortMax, oe = min(o + kSortMax, n);
+        const uint32_t p = o / (2 * R);
+        const uint32_t a0 = 2 * R * p, la = min(R, n - a0), b0 = a0 + R;
+        const uint32_t d0 = o - a0, d1 = oe - a0;
+        const uint32_t i0 = s_split[q - q0];
+        // the tile's end diagonal: the next tile's first one, or the whole
+        // pair when the tile closes it
+        const uint32_t i1 = d1 == la + (b0 < n ? min(R, n - b0) : 0u) ? la : s_split[q + 1 - q0];
+        const uint32_t j0 = d0 - i0, j1 = d1 - i1;
+        const uint32_t na = i1 - i0, nb = j1 - j0;
+        // A's part then B's part, in shared memory
+        for (uint32_t i = t; i < na; i += kSortCta) sa[i] = S.get(a0 + i0 + i);
+        for (uint32_t i = t; i < nb; i += kSortCta) sa[na + i] = S.get(b0 + j0 + i);
+        __syncthreads();
+        const uint32_t d = 8 * t;
+        if (d < na + nb) {
+          uint32_t lo = d > nb ? d - nb : 0u, hi = d < na ? d : na;
+          while (lo < hi) {
+            const uint32_t mid = (lo + hi) >> 1;
+            if (sa[mid] > sa[na + d - mid - 1]) hi = mid;
+            else lo = mid + 1;
+          }
+          uint32_t i = lo, j = d - lo;
+          const uint32_t cnt = min(8u, na + nb - d);
+          for (uint32_t r = 0; r < cnt; ++r) {
+            const unsigned long long a = i < na ? sa[i] : ~0ull, b = j < nb ? sa[na + j] : ~0ull;
+            const bool takeA = j >= nb || (i < na && a < b);
+            Dst.put(o + d + r, takeA ? a : b);
+            i += takeA;
+            j += !takeA;
+          }
+        }
+        __syncthreads();
+      }
+    }
+    in_x = !in_x;
+  }
+  // the item list: the keys' low halves (already in place when the result is
+  // in the split buffer)
+  if (in_x)
+    for (uint32_t i = t; i < n; i += kSortCta) Y.lo[i] = static_cast<uint32_t>(X.get(i));
+}
+
+// fn(key) for the n keys X[0, n) in turn, four loads in flight per thread.
+template <class Fn>
+__device__ __forceinline__ void for_keys(const unsigned long long* __restrict__ X, uint32_t n, Fn fn) {
+  for (uint32_t i0 = threadIdx.x; i0 < n; i0 += 4 * kLongCta) {
+    unsigned long long x[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) x[u] = i0 + u * kLongCta < n ? __ldg(X + i0 + u * kLongCta) : 0ull;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (i0 + u * kLongCta < n) fn(x[u]);
+  }
+}
+
+// Exclusive prefix over the CTA's 2 * kLongCta words, two per thread (c[2t],
+// c[2t + 1]).  Holds two barriers.
+__device__ __forceinline__ uint2 long_exclusive(uint2 c, uint32_t* s_w) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  uint32_t incl = c.x + c.y;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += y;
+  }
+  if (lane == 31) s_w[wid] = incl;
+  __syncthreads();
+  uint32_t w = s_w[lane];
+  w = __reduce_add_sync(0xffffffffu, lane < wid ? w : 0u);
+  __syncthreads();   // s_w is rewritten by the next call
+  const uint32_t b = w + incl - c.x - c.y;
+  return make_uint2(b, b + c.x);
+}
+
+__global__ void __launch_bounds__(kLongCta, 2)
+    k_long_split(const uint2* __restrict__ ranges, Status* __restrict__ st, const uint32_t* __restrict__ order,
+                 uint32_t n_tiles, const unsigned long long* __restrict__ pkey, uint32_t* __restrict__ ptile,
+                 uint32_t* __restrict__ pv, uint2* __restrict__ groups) {
+  pdl_launch_dependents();  // the next kernel may be dispatched now
+  __shared__ uint32_t s_hist[2 * kLongCta];     // counts per bin, then per group, then group cursors
+  __shared__ uint32_t s_start[kLongCoarse + 2]; // the bucket's keys before each bin
+  __shared__ uint32_t s_w[32], s_mm[2], s_claim, s_at;
   if (st->overflow || st->n_big == 0) return;
   const uint32_t t = threadIdx.x;
   while (true) {
     // buckets in the tile scan's longest-first order; the long ones come
-    // first, so the first list of at most kMergeMax keys ends the work
+    // first, so the first list of a shorter class ends the work
     __syncthreads();
-    if (t == 0) s_claim = atomicAdd(&st->long_sort_counter, 1u);
+    if (t == 0) {
+      s_claim = atomicAdd(&st->long_sort_counter, 1u);
+      s_mm[0] = ~0u;
+      s_mm[1] = 0u;
+    }
+    s_hist[2 * t] = s_hist[2 * t + 1] = 0u;
     __syncthreads();
     const uint32_t k = s_claim;
     if (k >= n_tiles) return;
-    const uint32_t tile = order[k];
-    const uint2 rg = ranges[tile];
+    const uint2 rg = ranges[order[k]];
     const uint32_t n = rg.y - rg.x;
-    if (order_bucket(n) > order_bucket(kMergeMax + 1)) return;   // a shorter class: no long list follows
-    if (n <= kMergeMax) continue;
-    KeyBuf X{pkey + rg.x, nullptr, nullptr}, Y{nullptr, ptile + rg.x, pv + rg.x};
-    // sorted chunks, in place
-    for (uint32_t c0 = 0; c0 < n; c0 += kLongChunk) {
-      const uint32_t m = min(kLongChunk, n - c0);
-      const unsigned long long* res = smem_merge_sort<0>(X.k + c0, m, sa, sb, t, kLongSortCta);
-      for (uint32_t i = t; i < m; i += kLongSortCta) X.k[c0 + i] = res[pad8(i)];
-      __syncthreads();
+    if (order_bucket(n) > order_bucket(kSortMax + 1)) return;   // a shorter class: no long list follows
+    if (n <= kSortMax) continue;
+    uint32_t sh = kGroupBits;
+    while (((n - 1) >> sh) >= kMaxGroups) ++sh;
+    const uint32_t n_groups = ((n - 1) >> sh) + 1;
+    const unsigned long long* X = pkey + rg.x;
+    // the bucket's depth range
+    uint32_t lo = ~0u, hi = 0u;
+    for_keys(X, n, [&](unsigned long long x) {
+      lo = min(lo, static_cast<uint32_t>(x >> 32));
+      hi = max(hi, static_cast<uint32_t>(x >> 32));
+    });
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if ((t & 31) == 0) {
+      atomicMin(&s_mm[0], lo);
+      atomicMax(&s_mm[1], hi);
     }
-    // merge passes: runs of R keys into runs of 2 R
-    bool in_x = true;
-    for (uint32_t R = kLongChunk; R < n; R <<= 1) {
-      const KeyBuf& S = in_x ? X : Y;
-      const KeyBuf& Dst = in_x ? Y : X;
-      const uint32_t n_out = (n + kLongChunk - 1) / kLongChunk;   // output tiles (a run pair holds whole tiles)
-      for (uint32_t q0 = 0; q0 < n_out; q0 += kLongSortCta) {
-        // first diagonal of output tiles q0 + t (and the end of the last one)
-        __syncthreads();
-        for (uint32_t q = q0 + t; q <= min(q0 + kLongSortCta, n_out); q += kLongSortCta) {
-          const uint32_t o = min(q * kLongChunk, n);
-          uint32_t p = o / (2 * R);
-          if (o == n && o % (2 * R) == 0 && o > 0) --p;   // the end diagonal of the last pair
-          const uint32_t a0 = 2 * R * p, la = min(R, n - a0), b0 = a0 + R;
-          const uint32_t lb = b0 < n ? min(R, n - b0) : 0u;
-          s_split[q - q0] = path_split(S, a0, la, b0, lb, o - a0);
-        }
-        __syncthreads();
-        const uint32_t q1 = min(q0 + kLongSortCta, n_out);
-        for (uint32_t q = q0; q < q1; ++q) {
-          const uint32_t o = q * kLongChunk, oe = min(o + kLongChunk, n);
-          const uint32_t p = o / (2 * R);
-          const uint32_t a0 = 2 * R * p, la = min(R, n - a0), b0 = a0 + R;
-          const uint32_t d0 = o - a0, d1 = oe - a0;
-          const uint32_t i0 = s_split[q - q0];
-          // the tile's end diagonal: the next tile's first one, or the whole
-          // pair when the tile closes it
-          const uint32_t i1 = d1 == la + (b0 < n ? min(R, n - b0) : 0u) ? la : s_split[q + 1 - q0];
-          const uint32_t j0 = d0 - i0, j1 = d1 - i1;
-          const uint32_t na = i1 - i0, nb = j1 - j0;
-          // A's part then B's part, in shared memory
-          for (uint32_t i = t; i < na; i += kLongSortCta) sa[i] = S.get(a0 + i0 + i);
-          for (uint32_t i = t; i < nb; i += kLongSortCta) sa[na + i] = S.get(b0 + j0 + i);
-          __syncthreads();
-          const uint32_t d = 8 * t;
-          if (d < na + nb) {
-            uint32_t lo = d > nb ? d - nb : 0u, hi = d < na ? d : na;
-            while (lo < hi) {
-              const uint32_t mid = (lo + hi) >> 1;
-              if (sa[mid] > sa[na + d - mid - 1]) hi = mid;
-              else lo = mid + 1;
-            }
-            uint32_t i = lo, j = d - lo;
-            const uint32_t cnt = min(8u, na + nb - d);
-            for (uint32_t r = 0; r < cnt; ++r) {
-              const unsigned long long a = i < na ? sa[i] : ~0ull, b = j < nb ? sa[na + j] : ~0ull;
-              const bool takeA = j >= nb || (i < na && a < b);
-              Dst.put(o + d + r, takeA ? a : b);
-              i += takeA;
-              j += !takeA;
-            }
-          }
-          __syncthreads();
-        }
-      }
-      in_x = !in_x;
-    }
-    // the item list: the keys' low halves (already in place when the result
-    // is in the split buffer)
-    if (in_x)
-      for (uint32_t i = t; i < n; i += kLongSortCta) pv[rg.x + i] = static_cast<uint32_t>(X.k[i]);
+    __syncthreads();
+    const DepthMap map(s_mm[0], s_mm[1], kLongCoarse);
+    for_keys(X, n, [&](unsigned long long x) {
+      float frac;
+      atomicAdd(&s_hist[map.bin(static_cast<uint32_t>(x >> 32), frac)], 1u);
+    });
+    __syncthreads();
+    const uint2 first = long_exclusive(make_uint2(s_hist[2 * t], s_hist[2 * t + 1]), s_w);
+    s_start[2 * t] = first.x;
+    s_start[2 * t + 1] = first.y;
+    if (t == 0) s_start[kLongCoarse] = n;
+    s_hist[2 * t] = s_hist[2 * t + 1] = 0u;   // (every thread has read its own counts only)
+    __syncthreads();
+    for_keys(X, n, [&](unsigned long long x) {
+      atomicAdd(&s_hist[map.rank(static_cast<uint32_t>(x >> 32), s_start) >> sh], 1u);
+    });
+    __syncthreads();
+    const uint2 c = make_uint2(s_hist[2 * t], s_hist[2 * t + 1]);
+    const uint2 at = long_exclusive(c, s_w);
+    s_hist[2 * t] = at.x;
+    s_hist[2 * t + 1] = at.y;
+    if (t == 0) s_at = atomicAdd(&st->n_groups, n_groups);
+    __syncthreads();
+    if (2 * t < n_groups) groups[s_at + 2 * t] = make_uint2(rg.x + at.x, rg.x + at.x + c.x);
+    if (2 * t + 1 < n_groups) groups[s_at + 2 * t + 1] = make_uint2(rg.x + at.y, rg.x + at.y + c.y);
+    for_keys(X, n, [&](unsigned long long x) {
+      const uint32_t pos = rg.x + atomicAdd(&s_hist[map.rank(static_cast<uint32_t>(x >> 32), s_start) >> sh], 1u);
+      ptile[pos] = static_cast<uint32_t>(x >> 32);
+      pv[pos] = static_cast<uint32_t>(x);
+    });
   }
 }
 
-// ---- every bucket of at most 2048 keys in one launch ------------------------
-// The first n_lead CTAs take the buckets of 1025..2048 keys from the tile
-// scan's list (the merge sort over the whole CTA), looping until it is done;
-// every other CTA sorts two buckets of at most 1024 keys, one per half (128
-// threads, its own named barrier).  Shared memory: two halves of two
-// 1152-key buffers, or one pair of 2304-key buffers.  Longer buckets are
-// k_sort_long's.
-constexpr int kSortAllCta = 256;
-constexpr int kSortAllSmem = 2 * (kMergeMax + kMergeMax / 8);   // 4608 keys, 36 KB
-static_assert(kSortAllCta == kMergeMax / 8 && kSortAllCta == 2 * (kMergeSmall / 8), "thread counts");
-
-__global__ void __launch_bounds__(kSortAllCta) k_tile_sort_all(const uint2* __restrict__ ranges,
-                                                                const Status* __restrict__ st,
-                                                                const uint32_t* __restrict__ midl,
-                                                                uint32_t n_tiles, uint32_t n_lead,
-                                                                unsigned long long* __restrict__ pkey,
-                                                                uint32_t* __restrict__ pv) {
-  __shared__ unsigned long long s[kSortAllSmem];
+// TILES: CTAs below n_tiles take the bucket of their tile, if it has at most
+// kSortMax keys.  GROUPS: the CTAs after them take the long buckets' groups
+// (their keys in the split buffer) in turn.  (One kernel for both needs more
+// registers than the tiles alone: street frame 18 against 28 us.)
+template <bool TILES, bool GROUPS>
+__global__ void __launch_bounds__(kSortCta) k_tile_sort(const uint2* __restrict__ ranges,
+                                                         const Status* __restrict__ st, uint32_t n_tiles,
+                                                         unsigned long long* pkey, uint32_t* ptile, uint32_t* pv,
+                                                         const uint2* __restrict__ groups) {
+  if (GROUPS) pdl_wait();   // (launched after k_long_split: wait for it)
+  __shared__ SortSmem s;
   if (st->overflow) return;
-  if (blockIdx.x < n_lead) {
-    for (uint32_t k = blockIdx.x; k < st->n_mid; k += n_lead) {
-      __syncthreads();
-      merge_sort_bucket<0>(midl[k], ranges, pkey, pv, s, s + kMergeMax + kMergeMax / 8, threadIdx.x, kSortAllCta);
-    }
+  if (TILES && (!GROUPS || blockIdx.x < n_tiles)) {
+    const uint2 rg = ranges[blockIdx.x];
+    const uint32_t n = rg.y - rg.x;
+    if (n == 0 || n > kSortMax) return;   // empty, or k_long_split's
+    sort_small([&](uint32_t i) { return pkey[rg.x + i]; }, n, pv + rg.x, s);
     return;
   }
-  const uint32_t half = threadIdx.x >> 7;
-  const uint32_t tile = 2 * (blockIdx.x - n_lead) + half;
-  if (tile >= n_tiles) return;
-  const uint2 rg = ranges[tile];
-  const uint32_t n = rg.y - rg.x;
-  if (n == 0 || n > kMergeSmall) return;   // empty, or a list of the lead CTAs
-  unsigned long long* sa = s + half * 2 * (kMergeSmall + kMergeSmall / 8);
-  unsigned long long* sb = sa + kMergeSmall + kMergeSmall / 8;
-  if (half == 0) merge_sort_bucket<1>(tile, ranges, pkey, pv, sa, sb, threadIdx.x & 127u, 128);
-  else merge_sort_bucket<2>(tile, ranges, pkey, pv, sa, sb, threadIdx.x & 127u, 128);
+  if (!GROUPS) return;
+  const uint32_t first = TILES ? n_tiles : 0u, n_groups = st->n_groups;
+  for (uint32_t g = blockIdx.x - first; g < n_groups; g += gridDim.x - first) {
+    const uint2 rg = groups[g];
+    const uint32_t n = rg.y - rg.x;
+    const KeyBuf Y{nullptr, ptile + rg.x, pv + rg.x};
+    __syncthreads();   // the previous group's shared memory is no longer read
+    if (n == 0) continue;
+    if (n <= kSortMax) sort_small([&](uint32_t i) { return Y.get(i); }, n, Y.lo, s);
+    else merge_sort_global(KeyBuf{pkey + rg.x, nullptr, nullptr}, Y, n, s);
+  }
 }
 
 // The tile of every pair (sorted order), written only when a caller asks for
@@ -898,11 +1056,29 @@ cudaError_t launch_fill_tile_of_pair(const WsPtrs& w, uint32_t n_tiles, cudaStre
 // ---------------------------------------------------------------------------
 // Orchestration
 // ---------------------------------------------------------------------------
-// kernels launch_bin enqueues (memsets not counted)
-int bin_kernel_count(uint32_t) { return 5; }
+// How the long buckets (more than kSortMax keys) are sorted, by the largest
+// map of the call.  None can arise up to kSortMax surfels.  From kSideItems
+// surfels on, k_long_split and the groups' sort run on the side stream
+// alongside the short buckets' sort (1M surfels, 8 keyframes: 0.43 ms beside
+// 0.11); below, long buckets are few and the fork and join would cost a small
+// frame, which the host's launches bound, more (2,000-surfel room, bin and
+// forward: 53 us with them, 37 to 43 us without).
+constexpr int64_t kSideItems = 32768;
+enum LongPath { kLongNone, kLongInline, kLongSide };
+static LongPath long_path(int64_t max_n) {
+  return max_n <= static_cast<int64_t>(kSortMax) ? kLongNone : (max_n < kSideItems ? kLongInline : kLongSide);
+}
 
-cudaError_t launch_bin(const Layout& L, const WsPtrs& w, int n_frames, int64_t n_items, uint32_t n_tiles,
-                       const SideStream& side, cudaStream_t s) {
+// kernels launch_bin enqueues (memsets not counted); max_n: surfels of the
+// largest map that a frame renders
+int bin_kernel_count(uint32_t n_tiles, int64_t max_n) {
+  if (n_tiles == 0) return 4;
+  const LongPath p = long_path(max_n);
+  return p == kLongNone ? 5 : (p == kLongInline ? 6 : 7);
+}
+
+cudaError_t launch_bin(const Layout& L, const WsPtrs& w, int n_frames, int64_t n_items, int64_t max_n,
+                       uint32_t n_tiles, const SideStream& side, cudaStream_t s) {
   k_tables<<<n_frames, 256, 0, s>>>(w.desc, w.tables, w.st, reinterpret_cast<uint32_t*>(w.loss_part),
                                     static_cast<uint32_t>(loss_part_bytes() / 4), w.tcur, n_tiles);
   const int64_t ni = n_items > 0 ? n_items : 1;
@@ -913,7 +1089,7 @@ cudaError_t launch_bin(const Layout& L, const WsPtrs& w, int n_frames, int64_t n
                               w.tset, w.tcur, w.st);
   if (e0 == cudaSuccess)
     e0 = launch_dep(k_tile_scan, dim3(1), dim3(kScanCta), 0, s, w.tcur, n_tiles, w.ranges, w.st, L.pairs_cap, w.work,
-                    w.longt, w.cbase, w.midl);
+                    w.longt, w.cbase);
   if (e0 == cudaSuccess)
     e0 = launch_dep(k_emit, dim3(gi), dim3(256), 0, s, w.desc, w.tables, w.key, w.cnt, w.tset, w.tcur, w.ranges, w.st,
                     w.pkey);
@@ -922,26 +1098,30 @@ cudaError_t launch_bin(const Layout& L, const WsPtrs& w, int n_frames, int64_t n
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const unsigned few = static_cast<unsigned>(sms) < n_tiles ? static_cast<unsigned>(sms) : n_tiles;
-    const unsigned grid = few + (n_tiles + 1) / 2;
-    // the long buckets: one CTA each, longest first (an early exit when the
-    // tile scan found none), on the side stream alongside the short buckets
-    static bool smem_set[64] = {false};
-    if (dev < 64 && !smem_set[dev]) {
-      const cudaError_t e = cudaFuncSetAttribute(k_sort_long, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 static_cast<int>(kLongSortSmem));
-      if (e != cudaSuccess) return e;
-      smem_set[dev] = true;
+    // the short buckets, and the long ones: longest first (an early exit when
+    // the tile scan found none), then the CTAs that sort their groups
+    const LongPath path = long_path(max_n);
+    const unsigned group_ctas = 4 * sms;
+    cudaError_t e = cudaSuccess;
+    if (path == kLongInline) {
+      k_long_split<<<2 * sms, kLongCta, 0, s>>>(w.ranges, w.st, w.work, n_tiles, w.pkey, w.ptile, w.pv, w.groups);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      return launch_dep(k_tile_sort<true, true>, dim3(n_tiles + group_ctas), dim3(kSortCta), 0, s, w.ranges, w.st,
+                        n_tiles, w.pkey, w.ptile, w.pv, w.groups);
     }
-    cudaError_t e = cudaEventRecord(side.fork, s);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(side.s, side.fork, 0);
+    if (path == kLongSide && (e = cudaEventRecord(side.fork, s)) != cudaSuccess) return e;
+    k_tile_sort<true, false><<<n_tiles, kSortCta, 0, s>>>(w.ranges, w.st, n_tiles, w.pkey, w.ptile, w.pv, w.groups);
+    if ((e = cudaGetLastError()) != cudaSuccess || path == kLongNone) return e;
+    // (the side stream has the higher priority: its CTAs take the slots that
+    // short buckets free, and the launches do not delay the short buckets)
+    if ((e = cudaStreamWaitEvent(side.s, side.fork, 0)) != cudaSuccess) return e;
+    k_long_split<<<2 * sms, kLongCta, 0, side.s>>>(w.ranges, w.st, w.work, n_tiles, w.pkey, w.ptile, w.pv, w.groups);
+    if ((e = cudaGetLastError()) == cudaSuccess)
+      e = launch_dep(k_tile_sort<false, true>, dim3(group_ctas), dim3(kSortCta), 0, side.s, w.ranges, w.st, 0u,
+                     w.pkey, w.ptile, w.pv, w.groups);
+    if (e == cudaSuccess) e = cudaEventRecord(side.join, side.s);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, side.join, 0);
     if (e != cudaSuccess) return e;
-    k_sort_long<<<sms, kLongSortCta, kLongSortSmem, side.s>>>(w.ranges, w.st, w.work, n_tiles, w.pkey, w.ptile,
-                                                               w.pv);
-    if ((e = cudaGetLastError()) != cudaSuccess || (e = cudaEventRecord(side.join, side.s)) != cudaSuccess) return e;
-    k_tile_sort_all<<<grid, kSortAllCta, 0, s>>>(w.ranges, w.st, w.midl, n_tiles, few, w.pkey, w.pv);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = cudaStreamWaitEvent(s, side.join, 0)) != cudaSuccess) return e;
   }
   return cudaGetLastError();
 }

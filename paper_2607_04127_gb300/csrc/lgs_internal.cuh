@@ -112,14 +112,14 @@ struct Status {
   unsigned int loss_ticket;           // loss CTAs finished (the last one reduces; self-resetting)
   unsigned int n_chunks;              // backward chunks of the last binning (kChunk list entries each)
   unsigned int count_ticket;          // mask-count CTAs finished (the last one adds up; self-resetting)
-  unsigned int n_big;                 // buckets of more than 2048 keys (the bitonic sort)
-  unsigned int n_mid;                 // buckets of 1025..2048 keys (the wide merge sort)
+  unsigned int n_big;                 // buckets of more than 2048 keys (split into groups)
+  unsigned int n_groups;              // groups of these buckets
   unsigned int long_sort_counter;     // tile order positions claimed by the long-bucket sort
 };
 
 struct Layout {
   size_t desc, status, tables, rec, box, key, cnt, tset, tcur, pkey, ptile, pv, ranges, g13, work, longt, loss_part,
-      cbase, ckpt, csuf, cmask, midl, bwm, bq, total;
+      cbase, ckpt, csuf, cmask, groups, bwm, bq, total;
   int64_t items_cap, pairs_cap, chunks_cap;
   uint32_t bq_cap0, bq_capk;  // capacity of the backward queue of class 0 and of each other class
   uint32_t tiles_cap;
@@ -149,7 +149,7 @@ struct WsPtrs {
   float* ckpt;             // [chunks][kCkptSlots][tile pixels] forward checkpoint at every chunk end
   float* csuf;             // [chunks][tile pixels] long lists: the suffix of the later chunks (backward)
   uint32_t* cmask;         // [chunks][4 windows][tile pixels] entries each pixel composited, one bit per entry
-  uint32_t* midl;          // [tiles] tiles whose bucket takes the wide merge sort (st->n_mid of them)
+  uint2* groups;           // [pairs / 512 + 1] ranges of the long buckets' groups (st->n_groups of them)
   uint32_t* bwm;           // [tiles][warp blocks] the block's largest n_contrib (short lists; written by k_fwd_s)
   uint2* bq;               // backward work queues: (chunk * blocks per tile + block, tile); class 0 first
   uint32_t bq_cap0, bq_capk;
@@ -179,7 +179,7 @@ inline WsPtrs ws_ptrs(void* base, const Layout& L) {
   p.ckpt = reinterpret_cast<float*>(b + L.ckpt);
   p.csuf = reinterpret_cast<float*>(b + L.csuf);
   p.cmask = reinterpret_cast<uint32_t*>(b + L.cmask);
-  p.midl = reinterpret_cast<uint32_t*>(b + L.midl);
+  p.groups = reinterpret_cast<uint2*>(b + L.groups);
   p.bwm = reinterpret_cast<uint32_t*>(b + L.bwm);
   p.bq = reinterpret_cast<uint2*>(b + L.bq);
   p.bq_cap0 = L.bq_cap0;
@@ -694,9 +694,9 @@ struct SideStream {
   cudaStream_t s;
   cudaEvent_t fork, join;
 };
-cudaError_t launch_bin(const Layout& L, const WsPtrs& w, int n_frames, int64_t n_items, uint32_t n_tiles,
-                       const SideStream& side, cudaStream_t s);
-int bin_kernel_count(uint32_t n_tiles);
+cudaError_t launch_bin(const Layout& L, const WsPtrs& w, int n_frames, int64_t n_items, int64_t max_n,
+                       uint32_t n_tiles, const SideStream& side, cudaStream_t s);
+int bin_kernel_count(uint32_t n_tiles, int64_t max_n);
 // the tile of every pair of the last binning into w.ptile (on request only)
 cudaError_t launch_fill_tile_of_pair(const WsPtrs& w, uint32_t n_tiles, cudaStream_t s);
 cudaError_t launch_raster_fwd(const Layout& L, const WsPtrs& w, const Desc& h, const uint32_t* pv, int batch, int group,
