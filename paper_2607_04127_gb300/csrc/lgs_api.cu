@@ -2,6 +2,7 @@
 // argument validation and the launch sequence of every entry point.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstddef>
 
 #include <vector>
@@ -225,10 +226,16 @@ Layout make_layout(int64_t items, uint32_t tiles, int64_t pairs_cap, uint32_t ta
   const int64_t C = chunk_cap(pairs_cap, tiles);
   L.cbase = take(4 * T);
   L.ckpt = take(sizeof(float) * lgs::kCkptSlots * static_cast<size_t>(tile_pixels) * static_cast<size_t>(C));
-  L.csuf = take(sizeof(float) * static_cast<size_t>(tile_pixels) * static_cast<size_t>(C));
   L.cmask = take(sizeof(uint32_t) * 4 * static_cast<size_t>(tile_pixels) * static_cast<size_t>(C));
   // a bucket of n > 2048 keys has ceil(n / 1024) < n / 512 groups at most
   L.groups = take(sizeof(uint2) * (P / 512 + 1));
+  // a list of n > kLongList entries has ceil(n / kSeg) <= n / kSeg + n / kLongList segments
+  const size_t SG = P / lgs::kSeg + P / lgs::kLongList + 1, LL = std::min(T, P / lgs::kLongList + 1);
+  L.segs = take(sizeof(uint2) * SG);
+  L.sbase = take(4 * T);
+  L.segsum = take(sizeof(float) * 5 * static_cast<size_t>(tile_pixels) * SG);
+  L.ssuf = take(sizeof(float) * static_cast<size_t>(tile_pixels) * SG);
+  L.dead = take(sizeof(uint32_t) * static_cast<size_t>(tile_pixels) * LL);
   // backward queues: class 0 takes at most every (chunk, warp block) item,
   // every other class at most one item per (tile, warp block)
   const size_t blocks = tile_pixels >= 32 ? tile_pixels / 32 : 1;
@@ -724,7 +731,7 @@ lgs_status lgs_bin_sort_batch(lgs_session s, const lgs_surfels* maps, int n_maps
     s->g13_zero_off = L.g13;
   }
   if ((e = write_desc(s, *s->desc, w.desc, cs, s->launches)) != cudaSuccess) return cuda_fail(e, "write_desc");
-  if ((e = timed(s, LGS_TIME_BIN, cs, [&] { return lgs::launch_bin(L, w, n_frames, p.n_items, p.max_n, p.n_tiles, s->side, cs); })) !=
+  if ((e = timed(s, LGS_TIME_BIN, cs, [&] { return lgs::launch_bin(L, w, n_frames, p.n_items, p.max_n, p.n_tiles, p.tile_pixels / 32, s->side, cs); })) !=
       cudaSuccess)
     return cuda_fail(e, "bin");
   s->launches += lgs::bin_kernel_count(p.n_tiles, p.max_n);
@@ -939,7 +946,7 @@ lgs_status lgs_render_fwd_loss_batch(lgs_session s, const lgs_surfels* maps, int
          return lgs::launch_raster_fwd_loss(w, d, w.pv, s->tune.persistent, *params, loss_out, cs);
        })) != cudaSuccess)
     return cuda_fail(e, "raster_fwd_loss");
-  s->launches += 3;   // counts and regulariser, per-tile forward, long-list forward (which writes the loss vector)
+  s->launches += 1 + lgs::raster_fwd_kernel_count(d);   // counts and regulariser, forward
   s->last_stream = cs;
   s->ckpt_valid = true;
   return LGS_OK;
@@ -970,7 +977,7 @@ lgs_status lgs_render_fwd_batch(lgs_session s, const lgs_surfels* maps, int n_ma
          return lgs::launch_raster_fwd(s->lay, w, d, pv, s->tune.fwd_batch, s->tune.group, s->tune.persistent, cs);
        })) != cudaSuccess)
     return cuda_fail(e, "raster_fwd");
-  s->launches += 2;   // per-tile and long-list kernels
+  s->launches += lgs::raster_fwd_kernel_count(d);
   s->last_stream = cs;
   s->ckpt_valid = s->tune.fwd_batch == 0 && s->tune.group == 16;
   return LGS_OK;

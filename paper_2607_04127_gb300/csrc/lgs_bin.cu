@@ -72,6 +72,9 @@ __global__ void k_tables(const Desc* __restrict__ D, float* __restrict__ tab, St
     st->loss_ticket = 0;
     st->count_ticket = 0;
     st->n_long = 0;
+    st->n_segs = 0;
+    st->seg_counter = 0;
+    st->seg_done = 0;
     st->n_big = 0;
     st->long_sort_counter = 0;
     st->n_groups = 0;
@@ -899,6 +902,15 @@ __device__ __noinline__ void merge_sort_global(const KeyBuf& X, const KeyBuf& Y,
     for (uint32_t i = t; i < n; i += kSortCta) Y.lo[i] = static_cast<uint32_t>(X.get(i));
 }
 
+// What k_long_split writes for the forward's long lists (SegBuf).
+struct SegPlan {
+  const uint32_t* longt;
+  uint32_t* sbase;
+  uint2* segs;
+  uint32_t* dead;
+  uint32_t blocks;   // warp blocks per tile
+};
+
 // fn(key) for the n keys X[0, n) in turn, four loads in flight per thread.
 template <class Fn>
 __device__ __forceinline__ void for_keys(const unsigned long long* __restrict__ X, uint32_t n, Fn fn) {
@@ -931,16 +943,58 @@ __device__ __forceinline__ uint2 long_exclusive(uint2 c, uint32_t* s_w) {
   return make_uint2(b, b + c.x);
 }
 
+// The segments of the forward's long lists (one CTA): every list's first
+// segment and the (list, segment) items ordered by segment (up to kSegClass;
+// the later ones together).
+constexpr uint32_t kSegClass = 2 * kLongCta - 1;
+
+__device__ void plan_segments(const uint2* __restrict__ ranges, Status* __restrict__ st, const SegPlan& P,
+                              uint32_t* s_cnt, uint32_t* s_w) {
+  const uint32_t t = threadIdx.x, n_long = st->n_long;
+  const auto segments = [&](uint32_t l) {
+    const uint2 rg = ranges[P.longt[l]];
+    return (rg.y - rg.x + kSeg - 1) / kSeg;
+  };
+  s_cnt[2 * t] = s_cnt[2 * t + 1] = 0u;
+  __syncthreads();
+  uint32_t carry = 0;
+  for (uint32_t l0 = 0; l0 < n_long; l0 += kLongCta) {
+    const uint32_t l = l0 + t;
+    const uint32_t n = l < n_long ? segments(l) : 0u;
+    const uint32_t at = long_exclusive(make_uint2(n, 0u), s_w).x;
+    if (n) {
+      P.sbase[P.longt[l]] = carry + at;
+      for (uint32_t s = 0; s < n; ++s) atomicAdd(&s_cnt[min(s, kSegClass)], 1u);
+    }
+    if (t == kLongCta - 1) s_w[0] = at + n;
+    __syncthreads();
+    carry += s_w[0];
+    __syncthreads();
+  }
+  const uint2 first = long_exclusive(make_uint2(s_cnt[2 * t], s_cnt[2 * t + 1]), s_w);
+  s_cnt[2 * t] = first.x;
+  s_cnt[2 * t + 1] = first.y;
+  __syncthreads();
+  for (uint32_t l = t; l < n_long; l += kLongCta) {
+    const uint32_t n = segments(l);
+    for (uint32_t s = 0; s < n; ++s) P.segs[atomicAdd(&s_cnt[min(s, kSegClass)], 1u)] = make_uint2(l, s);
+  }
+  for (uint32_t i = t; i < n_long * P.blocks * 32; i += kLongCta) P.dead[i] = ~0u;
+  if (t == 0) st->n_segs = carry;
+  __syncthreads();
+}
+
 __global__ void __launch_bounds__(kLongCta, 2)
     k_long_split(const uint2* __restrict__ ranges, Status* __restrict__ st, const uint32_t* __restrict__ order,
                  uint32_t n_tiles, const unsigned long long* __restrict__ pkey, uint32_t* __restrict__ ptile,
-                 uint32_t* __restrict__ pv, uint2* __restrict__ groups) {
+                 uint32_t* __restrict__ pv, uint2* __restrict__ groups, SegPlan plan) {
   pdl_launch_dependents();  // the next kernel may be dispatched now
   __shared__ uint32_t s_hist[2 * kLongCta];     // counts per bin, then per group, then group cursors
   __shared__ uint32_t s_start[kLongCoarse + 2]; // the bucket's keys before each bin
   __shared__ uint32_t s_w[32], s_mm[2], s_claim, s_at;
   if (st->overflow || st->n_big == 0) return;
   const uint32_t t = threadIdx.x;
+  if (blockIdx.x == gridDim.x - 1 && st->n_long) plan_segments(ranges, st, plan, s_hist, s_w);
   while (true) {
     // buckets in the tile scan's longest-first order; the long ones come
     // first, so the first list of a shorter class ends the work
@@ -1078,7 +1132,7 @@ int bin_kernel_count(uint32_t n_tiles, int64_t max_n) {
 }
 
 cudaError_t launch_bin(const Layout& L, const WsPtrs& w, int n_frames, int64_t n_items, int64_t max_n,
-                       uint32_t n_tiles, const SideStream& side, cudaStream_t s) {
+                       uint32_t n_tiles, uint32_t blocks, const SideStream& side, cudaStream_t s) {
   k_tables<<<n_frames, 256, 0, s>>>(w.desc, w.tables, w.st, reinterpret_cast<uint32_t*>(w.loss_part),
                                     static_cast<uint32_t>(loss_part_bytes() / 4), w.tcur, n_tiles);
   const int64_t ni = n_items > 0 ? n_items : 1;
@@ -1102,9 +1156,11 @@ cudaError_t launch_bin(const Layout& L, const WsPtrs& w, int n_frames, int64_t n
     // the tile scan found none), then the CTAs that sort their groups
     const LongPath path = long_path(max_n);
     const unsigned group_ctas = 4 * sms;
+    const SegPlan plan{w.longt, w.sbase, w.segs, w.dead, blocks};
     cudaError_t e = cudaSuccess;
     if (path == kLongInline) {
-      k_long_split<<<2 * sms, kLongCta, 0, s>>>(w.ranges, w.st, w.work, n_tiles, w.pkey, w.ptile, w.pv, w.groups);
+      k_long_split<<<2 * sms, kLongCta, 0, s>>>(w.ranges, w.st, w.work, n_tiles, w.pkey, w.ptile, w.pv, w.groups,
+                                                  plan);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
       return launch_dep(k_tile_sort<true, true>, dim3(n_tiles + group_ctas), dim3(kSortCta), 0, s, w.ranges, w.st,
                         n_tiles, w.pkey, w.ptile, w.pv, w.groups);
@@ -1115,7 +1171,8 @@ cudaError_t launch_bin(const Layout& L, const WsPtrs& w, int n_frames, int64_t n
     // (the side stream has the higher priority: its CTAs take the slots that
     // short buckets free, and the launches do not delay the short buckets)
     if ((e = cudaStreamWaitEvent(side.s, side.fork, 0)) != cudaSuccess) return e;
-    k_long_split<<<2 * sms, kLongCta, 0, side.s>>>(w.ranges, w.st, w.work, n_tiles, w.pkey, w.ptile, w.pv, w.groups);
+    k_long_split<<<2 * sms, kLongCta, 0, side.s>>>(w.ranges, w.st, w.work, n_tiles, w.pkey, w.ptile, w.pv, w.groups,
+                                                   plan);
     if ((e = cudaGetLastError()) == cudaSuccess)
       e = launch_dep(k_tile_sort<false, true>, dim3(group_ctas), dim3(kSortCta), 0, side.s, w.ranges, w.st, 0u,
                      w.pkey, w.ptile, w.pv, w.groups);

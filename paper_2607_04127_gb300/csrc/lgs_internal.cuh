@@ -100,6 +100,8 @@ struct Status {
   unsigned int work_counter2;
   unsigned int bq_count[kBwdClasses]; // backward items queued per class (zero between backwards)
   unsigned int n_long;                // tiles whose list is longer than kLongList
+  unsigned int n_segs;                // their segments
+  unsigned int seg_counter, seg_done; // work counter of their masks, warps that have finished (self-resetting)
   unsigned int long_counter_fwd;      // work counters of the long-list kernels (self-resetting)
   unsigned int long_counter_bwd;
   unsigned int long_done_fwd;         // warps of the long-list kernels that have finished
@@ -119,7 +121,7 @@ struct Status {
 
 struct Layout {
   size_t desc, status, tables, rec, box, key, cnt, tset, tcur, pkey, ptile, pv, ranges, g13, work, longt, loss_part,
-      cbase, ckpt, csuf, cmask, groups, bwm, bq, total;
+      cbase, ckpt, cmask, groups, segs, sbase, segsum, ssuf, dead, bwm, bq, total;
   int64_t items_cap, pairs_cap, chunks_cap;
   uint32_t bq_cap0, bq_capk;  // capacity of the backward queue of class 0 and of each other class
   uint32_t tiles_cap;
@@ -147,7 +149,11 @@ struct WsPtrs {
   double* loss_part;       // loss partial sums and mask counts
   uint32_t* cbase;         // [tiles] first backward chunk of every tile
   float* ckpt;             // [chunks][kCkptSlots][tile pixels] forward checkpoint at every chunk end
-  float* csuf;             // [chunks][tile pixels] long lists: the suffix of the later chunks (backward)
+  uint2* segs;             // [segments] segments of the long lists: (long list, segment), segment by segment
+  uint32_t* sbase;         // [tiles] first segment of a long list
+  float* segsum;           // [segments][5][tile pixels] a segment's sums (SegBuf)
+  float* ssuf;             // [segments][tile pixels] the suffix of the later segments (backward)
+  uint32_t* dead;          // [long lists][tile pixels] first segment known to stop the pixel (~0 between forwards)
   uint32_t* cmask;         // [chunks][4 windows][tile pixels] entries each pixel composited, one bit per entry
   uint2* groups;           // [pairs / 512 + 1] ranges of the long buckets' groups (st->n_groups of them)
   uint32_t* bwm;           // [tiles][warp blocks] the block's largest n_contrib (short lists; written by k_fwd_s)
@@ -177,7 +183,11 @@ inline WsPtrs ws_ptrs(void* base, const Layout& L) {
   p.loss_part = reinterpret_cast<double*>(b + L.loss_part);
   p.cbase = reinterpret_cast<uint32_t*>(b + L.cbase);
   p.ckpt = reinterpret_cast<float*>(b + L.ckpt);
-  p.csuf = reinterpret_cast<float*>(b + L.csuf);
+  p.segs = reinterpret_cast<uint2*>(b + L.segs);
+  p.sbase = reinterpret_cast<uint32_t*>(b + L.sbase);
+  p.segsum = reinterpret_cast<float*>(b + L.segsum);
+  p.ssuf = reinterpret_cast<float*>(b + L.ssuf);
+  p.dead = reinterpret_cast<uint32_t*>(b + L.dead);
   p.cmask = reinterpret_cast<uint32_t*>(b + L.cmask);
   p.groups = reinterpret_cast<uint2*>(b + L.groups);
   p.bwm = reinterpret_cast<uint32_t*>(b + L.bwm);
@@ -476,16 +486,21 @@ __device__ __forceinline__ bool box_hits(const float4& b, const WarpBox& w) {
 // Then for a unit ray d: den = n.d, t = h/den, u = t (a_u.d) - b_u,
 // v = t (a_v.d) - b_v.
 // ---------------------------------------------------------------------------
-// Tiles whose list is longer than this are composited by the entry-parallel
-// per-pixel kernels instead of the per-tile ones (their pixels would walk the
-// whole list one entry at a time).
+// Tiles whose list is longer than this get their window masks in segments of
+// kSeg entries, one warp per (segment, pixel block), and are composited by one
+// warp per pixel, instead of by the per-tile kernels (whose warps would walk the
+// whole list alone).  (Lists of 2,049 to 4,096 entries measured 1 to 2 % slower
+// this way; segments of 1,024 and 2,048 entries 2 and 7 % slower.)
 constexpr uint32_t kLongList = 4096;
+constexpr uint32_t kSeg = 512;
 
 // Backward work unit of the chunked walk: kChunk consecutive entries of a
 // tile list.  The forward records, per pixel, at the end of every chunk the
 // transmittance and the chunk's own sums of w, w t and w n' (a checkpoint of
 // six floats), so every chunk's reverse walk can start on its own.
 constexpr uint32_t kChunk = 128;
+constexpr uint32_t kSegChunks = kSeg / kChunk;
+static_assert(kSeg % kChunk == 0 && kLongList >= kSeg, "a segment holds whole chunks, a long list more than one segment");
 // Floats of a checkpoint per (chunk, pixel): T at the chunk end and the
 // chunk's own sums of w, w t and w n.
 constexpr int kCkptSlots = 6;
@@ -567,8 +582,10 @@ __device__ __forceinline__ float fix_mean(long long sum, float grid, int n) {
 // term, Eq. totalloss weights): masked L1 depth, positive BCE opacity,
 // cosine normal against N_gicp.  Adds the terms' fixed-point values to ld,
 // la, ln and returns dL/d(A, S_t, S_n) (scaled by `scale` = 1 / frames of the
-// map) in g.  Every loss path (the loss kernel, the forward epilogues, the
-// allocation-free loss) calls this one function, so their bits agree.
+// map) in g.  Every loss path (the loss kernel, the forward's epilogue, the
+// allocation-free loss) calls this one function, and every sum of products is
+// written with its rounding (no contraction left to the compiler), so their
+// bits agree.
 __device__ __forceinline__ void pixel_image_loss(float Dm, float A, float St, float nx, float ny, float nz, float sx,
                                                  float sy, float sz, float scale, float ind, float inn,
                                                  const lgs_loss_params& P, float (&g)[5], long long& ld,
@@ -582,22 +599,21 @@ __device__ __forceinline__ void pixel_image_loss(float Dm, float A, float St, fl
   const float sgn = diff > 0.f ? 1.f : (diff < 0.f ? -1.f : 0.f);
   const float gDh = sgn * ind;
   g[1] = scale * gDh / a;
-  g[0] = scale * (-gDh * St / (a * a));
   // log(A + 1e-6): for A >= 1/2 as log1p((A - 1) + 1e-6), where A - 1 is
   // exact, so opacities near 1 keep their precision; below 1/2 directly,
   // where A + 1e-6 is exact to half an ulp
   la += to_fix(-(A >= 0.5f ? log1pf((A - 1.0f) + 1e-6f) : logf(A + 1e-6f)), kFixU);
-  g[0] -= scale * P.lambda_alpha * ind / (A + 1e-6f);
-  if (nx * nx + ny * ny + nz * nz > 0.f) {
-    const float m = sqrtf(sx * sx + sy * sy + sz * sz + 1e-12f);
+  g[0] = __fsub_rn(__fmul_rn(scale, -gDh * St / (a * a)), scale * P.lambda_alpha * ind / a);
+  if (__fmaf_rn(nz, nz, __fmaf_rn(ny, ny, __fmul_rn(nx, nx))) > 0.f) {
+    const float m = sqrtf(__fadd_rn(__fmaf_rn(sz, sz, __fmaf_rn(sy, sy, __fmul_rn(sx, sx))), 1e-12f));
     const float im = 1.f / m;
-    ln += to_fix(1.0f - (sx * nx + sy * ny + sz * nz) * im, kFixU);
+    ln += to_fix(__fmaf_rn(-__fmaf_rn(sz, nz, __fmaf_rn(sy, ny, __fmul_rn(sx, nx))), im, 1.0f), kFixU);
     const float k = -P.lambda_n * P.lambda_ng * inn;
     const float g0 = k * nx, g1 = k * ny, g2 = k * nz;
-    const float sg = (sx * g0 + sy * g1 + sz * g2) * im * im * im;
-    g[2] = scale * (g0 * im - sx * sg);
-    g[3] = scale * (g1 * im - sy * sg);
-    g[4] = scale * (g2 * im - sz * sg);
+    const float sg = __fmul_rn(__fmaf_rn(sz, g2, __fmaf_rn(sy, g1, __fmul_rn(sx, g0))), im) * im * im;
+    g[2] = scale * __fmaf_rn(g0, im, -__fmul_rn(sx, sg));
+    g[3] = scale * __fmaf_rn(g1, im, -__fmul_rn(sy, sg));
+    g[4] = scale * __fmaf_rn(g2, im, -__fmul_rn(sz, sg));
   }
 }
 
@@ -695,10 +711,12 @@ struct SideStream {
   cudaEvent_t fork, join;
 };
 cudaError_t launch_bin(const Layout& L, const WsPtrs& w, int n_frames, int64_t n_items, int64_t max_n,
-                       uint32_t n_tiles, const SideStream& side, cudaStream_t s);
+                       uint32_t n_tiles, uint32_t blocks, const SideStream& side, cudaStream_t s);
 int bin_kernel_count(uint32_t n_tiles, int64_t max_n);
 // the tile of every pair of the last binning into w.ptile (on request only)
 cudaError_t launch_fill_tile_of_pair(const WsPtrs& w, uint32_t n_tiles, cudaStream_t s);
+// kernels launch_raster_fwd enqueues
+int raster_fwd_kernel_count(const Desc& h);
 cudaError_t launch_raster_fwd(const Layout& L, const WsPtrs& w, const Desc& h, const uint32_t* pv, int batch, int group,
                               int persistent, cudaStream_t s);
 // chunked: the forward was the shared-memory walk, which wrote the chunk

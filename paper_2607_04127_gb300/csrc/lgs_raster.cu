@@ -101,14 +101,15 @@ struct TileCtx {
   int HW;
 };
 
-__device__ __forceinline__ TileCtx tile_ctx(const Desc& D, uint32_t tile, const uint2* __restrict__ ranges) {
+__device__ __forceinline__ TileCtx tile_ctx(const Desc& D, uint32_t tile, const uint2* __restrict__ ranges,
+                                            int vt) {
   TileCtx t;
   t.f = frame_of_tile(D, tile);
   const FrameDev& F = D.f[t.f];
   const int lt = static_cast<int>(tile - F.tile_base);
   const int ti = lt / F.ntc, tj = lt - ti * F.ntc;
   int lr, lc;
-  pixel_of_thread(F, static_cast<int>(threadIdx.x), lr, lc);
+  pixel_of_thread(F, vt, lr, lc);
   t.r = ti * F.th + lr;
   t.c = tj * F.tw + lc;
   t.inside = t.r < F.H && t.c < F.W;
@@ -172,7 +173,7 @@ __global__ void __launch_bounds__(kMaxTileThreads)
   uint32_t tile;
   uint32_t evals = 0, contrib = 0, alg = 0;
   for (int iter = 0; next_tile(persistent, order, D->n_tiles, &st->work_counter, tile, iter); ++iter) {
-    const TileCtx tc = tile_ctx(*D, tile, ranges);
+    const TileCtx tc = tile_ctx(*D, tile, ranges, static_cast<int>(threadIdx.x));
     if (tc.end - tc.start > kLongList) continue;   // the long-list kernels' tile
     const FrameDev& F = D->f[tc.f];
     const WarpBox wb = warp_box(tc.inside, tc.r, tc.c, F.W);
@@ -306,7 +307,7 @@ __global__ void __launch_bounds__(kMaxTileThreads)
   uint32_t tile;
   uint32_t evals = 0, contrib = 0;
   for (int iter = 0; next_tile(persistent, order, D->n_tiles, &st->work_counter2, tile, iter); ++iter) {
-    const TileCtx tc = tile_ctx(*D, tile, ranges);
+    const TileCtx tc = tile_ctx(*D, tile, ranges, static_cast<int>(threadIdx.x));
     if (tc.end - tc.start > kLongList) continue;   // the long-list kernels' tile
     const FrameDev& F = D->f[tc.f];
     const WarpBox wb = warp_box(tc.inside, tc.r, tc.c, F.W);
@@ -431,7 +432,7 @@ __global__ void __launch_bounds__(kMaxTileThreads)
   uint32_t tile;
   uint32_t evals = 0, contrib = 0, alg = 0;
   for (int iter = 0; next_tile(persistent, order, D->n_tiles, &st->work_counter, tile, iter); ++iter) {
-    const TileCtx tc = tile_ctx(*D, tile, ranges);
+    const TileCtx tc = tile_ctx(*D, tile, ranges, static_cast<int>(threadIdx.x));
     if (tc.end - tc.start > kLongList) continue;   // the long-list kernels' tile
     const FrameDev& F = D->f[tc.f];
     const WarpBox wb = warp_box(tc.inside, tc.r, tc.c, F.W);
@@ -529,7 +530,7 @@ __global__ void __launch_bounds__(kMaxTileThreads)
   uint32_t tile;
   uint32_t evals = 0, contrib = 0;
   for (int iter = 0; next_tile(persistent, order, D->n_tiles, &st->work_counter2, tile, iter); ++iter) {
-    const TileCtx tc = tile_ctx(*D, tile, ranges);
+    const TileCtx tc = tile_ctx(*D, tile, ranges, static_cast<int>(threadIdx.x));
     if (tc.end - tc.start > kLongList) continue;   // the long-list kernels' tile
     const FrameDev& F = D->f[tc.f];
     const WarpBox wb = warp_box(tc.inside, tc.r, tc.c, F.W);
@@ -682,7 +683,7 @@ struct LossEpi {
   lgs_loss_params P;
   int* ctot;                     // mask counts [frame][2], complete before the forward
   unsigned long long* acc;       // fixed-point sums [frame][4], then [maps] of the regulariser
-  float* out;                    // loss vector, written by the long-list forward's last CTA
+  float* out;                    // loss vector, written by the forward's last CTA
 };
 
 __device__ __forceinline__ void loss_epilogue(const Desc& D, const LossEpi& L, int f, bool inside, int64_t pix,
@@ -715,14 +716,252 @@ __device__ __forceinline__ void loss_epilogue(const Desc& D, const LossEpi& L, i
   }
 }
 
-// hits evaluated together per step of the shared-memory forward (3 measured
-// fastest on the street frame: 2 leaves latency exposed, 4 costs registers)
-constexpr int FWD_HITS = 3;
+__device__ __forceinline__ uint32_t warp_claim(unsigned int* counter) {
+  uint32_t id = 0;
+  if ((threadIdx.x & 31) == 0) id = atomicAdd(counter, 1u);
+  return __shfl_sync(0xffffffffu, id, 0);
+}
 
+// A warp that finds no work left counts itself done; the last of `total` resets
+// the work and done counters to zero for the next launch on the stream.
+__device__ __forceinline__ void long_finish(unsigned int* counter, unsigned int* done, unsigned int total) {
+  if ((threadIdx.x & 31) == 0) {
+    __threadfence();
+    if (atomicAdd(done, 1u) == total - 1) {
+      *counter = 0u;
+      *done = 0u;
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Long lists (more than kLongList entries) in the forward
+// ---------------------------------------------------------------------------
+// A tile with a very long list (a far horizon seen along a street: tens of
+// thousands of entries, few of which any pixel composites) would make its
+// warps walk the list alone while the rest of the frame is done.  Two steps:
+//  (1) k_long_masks: the list is cut into segments of kSeg entries, and warps
+//      claim (segment, pixel block) items: the warp finds which entries are
+//      valid at which of its 32 pixels and writes the window masks.  Items are
+//      claimed segment by segment over all long lists, so that a pixel's first
+//      segments are usually done before its later ones start: a segment behind
+//      one whose entries alone stop the pixel is skipped.
+//  (2) k_fwd_long, one warp per pixel: the 32 lanes take the entries of a
+//      window that the masks name; the transmittance before each is T times a
+//      multiplicative scan of (1 - a) over the lanes, the early stop is the
+//      first lane whose T (1 - a) falls below 1e-4, and the composited sums
+//      are warp reductions.  Windows without a valid entry are skipped.
+// The lists' box tests and evaluations, shared by 32 pixels in (1), were the
+// bulk of (2) when it walked every window of the list itself with a box test
+// per (pixel, entry): 8 keyframes of a 1M map (17.9 M long entries) 3.5 ms, now
+// 0.53 + 0.87; 6 maps (26.8 M) 4.8 ms, now 0.52 + 0.60.
+// The products and sums associate differently from the per-tile walk (same
+// values to a few ulps), and exactly as they did without step (1).
+constexpr int kSegSlots = 5;   // a segment's sums of w, w t, w n'(3)
+
+struct SegBuf {
+  const uint2* item;       // [segments] (long list, segment), segment by segment
+  const uint32_t* longt;   // [long lists] tile
+  const uint32_t* sbase;   // [tiles] first segment of a long list
+  float* sum;              // [segments][kSegSlots][tile pixels]
+  uint32_t* dead;          // [long lists][tile pixels] first segment known to stop the pixel (~0: none)
+};
+
+// Step (1) takes a pixel for stopped a little below the threshold: its product
+// of (1 - a) associates differently from step (2)'s.
+constexpr float kSurelyStopped = 0.99e-4f;
+
+// The pixels of a 4 x 8 block (rows r0 .. r0 + 3, columns cmid - 3.5 .. cmid +
+// 3.5, one bit each in lane order) inside a culling box.  A box that nearly
+// wraps around the frame takes every column (its distance is formed for the
+// block's centre, so a pixel of the block could be nearer the other way round).
+__device__ __forceinline__ uint32_t block_cover(const float4& b, float r0, float cmid, float W, float inv_W) {
+  const int lo = max(static_cast<int>(ceilf(b.x - r0)), 0), hi = min(static_cast<int>(floorf(b.y - r0)), 3);
+  if (lo > hi) return 0u;
+  uint32_t cols = 0xffu;
+  if (b.w < 0.5f * W - 8.0f) {
+    float d = b.z - cmid;
+    d -= W * rintf(d * inv_W);
+    const int cl = max(static_cast<int>(ceilf(fmaxf(d - b.w, -4.0f) + 3.5f)), 0);
+    const int ch = min(static_cast<int>(floorf(fminf(d + b.w, 4.0f) + 3.5f)), 7);
+    if (cl > ch) return 0u;
+    cols = (2u << ch) - (1u << cl);
+  }
+  const uint32_t rows = 0x01010101u & (0xffffffffu << (8 * lo)) & (0xffffffffu >> (8 * (3 - hi)));
+  return cols * rows;
+}
+
+// Transpose of a 32 x 32 bit matrix, one row per lane: bit j of lane i becomes
+// bit i of lane j.
+__device__ __forceinline__ uint32_t warp_transpose(uint32_t x, int lane) {
+  uint32_t m = 0x0000ffffu;
+#pragma unroll
+  for (int k = 16; k; k >>= 1) {
+    const uint32_t y = __shfl_xor_sync(0xffffffffu, x, k);
+    x = (lane & k) ? (x & ~m) | ((y & ~m) >> k) : (x & m) | ((y & m) << k);
+    m ^= m << (k >> 1);
+  }
+  return x;
+}
+
+// The pixels of a warp and the entries whose culling box holds them.  Lane i
+// holds entry i of a window (box b; ok: there is one); candidates() returns the
+// entries whose box holds the lane's pixel, one bit each, and sets hit where
+// the lane's entry is one of some pixel's.
+template <bool BLOCK48>
+struct WarpPixels;
+
+// 4 x 8 blocks (pixel_of_thread): every lane finds the pixels inside its
+// entry's box, and a transpose gives every pixel its entries.
+template <>
+struct WarpPixels<true> {
+  float r0, cmid, W, inv_W;
+  __device__ __forceinline__ WarpPixels(const FrameDev& F, const TileCtx& tc, int lane)
+      : r0(static_cast<float>(tc.r - (lane >> 3))),
+        cmid(static_cast<float>(tc.c - (lane & 7)) + 3.5f),
+        W(static_cast<float>(F.W)),
+        inv_W(1.0f / static_cast<float>(F.W)) {}
+  __device__ __forceinline__ uint32_t candidates(const float4& b, bool ok, int lane, bool& hit) const {
+    const uint32_t cover = ok ? block_cover(b, r0, cmid, W, inv_W) : 0u;
+    hit = cover != 0u;
+    return warp_transpose(cover, lane);
+  }
+};
+
+// Any other shape: the boxes that meet the warp's pixels, tested one by one.
+template <>
+struct WarpPixels<false> {
+  WarpBox wb, px;
+  __device__ __forceinline__ WarpPixels(const FrameDev& F, const TileCtx& tc, int)
+      : wb(warp_box(tc.inside, tc.r, tc.c, F.W)),
+        px{static_cast<float>(tc.r), static_cast<float>(tc.r), static_cast<float>(tc.c), 0.f,
+           static_cast<float>(F.W)} {}
+  __device__ __forceinline__ uint32_t candidates(const float4& b, bool ok, int, bool& hit) const {
+    hit = ok && box_hits(b, wb);
+    uint32_t m = 0u;
+    for (uint32_t h = __ballot_sync(0xffffffffu, hit); h; h &= h - 1) {
+      const int q = __ffs(h) - 1;
+      const float4 x = make_float4(__shfl_sync(0xffffffffu, b.x, q), __shfl_sync(0xffffffffu, b.y, q),
+                                   __shfl_sync(0xffffffffu, b.z, q), __shfl_sync(0xffffffffu, b.w, q));
+      if (box_hits(x, px)) m |= 1u << q;
+    }
+    return m;
+  }
+};
+
+// Candidates a lane evaluates together per step of the shared-memory forward
+// (street frame, bin and forward: 1 169.9 us, 2 167.3, 3 165.6; its step and
+// 8 keyframes of a 1M map: 357.8, 347.0, 350.2 us and 6.31, 6.13, 6.10 ms).
+// Every lane takes its own next candidates (street frame: 17 per window and
+// warp at most over the lanes, where the warp took all 21 hits together; the
+// forward 115 -> 111 us).
+constexpr int FWD_HITS = 2;
+
+// Step (1) of the long lists: warps claim (segment, block) items.
+template <bool BLOCK48>
+__global__ void __launch_bounds__(256, 3)
+    k_long_masks(const Desc* __restrict__ Dp, const uint2* __restrict__ ranges, const uint32_t* __restrict__ pv,
+                 const float4* __restrict__ rec, const float4* __restrict__ box, Status* __restrict__ st,
+                 const uint32_t* __restrict__ cbase, float* __restrict__ ckpt, uint32_t* __restrict__ cmask,
+                 uint32_t* __restrict__ bwm, SegBuf seg) {
+  pdl_wait();               // (launched after a kernel of this chain: wait for it)
+  pdl_launch_dependents();  // the next kernel may be dispatched now
+  __shared__ WarpRecs s_w[8];
+  const Desc& D = *Dp;
+  const int lane = threadIdx.x & 31;
+  WarpRecs& sw = s_w[threadIdx.x >> 5];
+  const int npx = D.th * D.tw;
+  const uint32_t blocks = static_cast<uint32_t>(npx) >> 5;
+  const uint32_t n_items = st->n_segs * blocks;
+  if (n_items == 0) return;
+  uint32_t evals = 0;
+  while (true) {
+    const uint32_t id = warp_claim(&st->seg_counter);
+    if (id >= n_items) break;
+    const uint2 it = __ldg(seg.item + id / blocks);
+    const uint32_t li = it.x, sg = it.y, tile = __ldg(seg.longt + li);
+    const int vt = static_cast<int>(id % blocks) * 32 + lane;
+    const TileCtx tc = tile_ctx(D, tile, ranges, vt);
+    uint32_t* dead = seg.dead + static_cast<int64_t>(li) * npx + vt;
+    bool done = !tc.inside || __ldcg(dead) < sg;
+    if (__all_sync(0xffffffffu, done)) continue;
+    const FrameDev& F = D.f[tc.f];
+    const WarpPixels<BLOCK48> bb(F, tc, lane);
+    float dx = 0.f, dy = 0.f, dz = 0.f;
+    if (tc.inside) pixel_ray(F, tc.r, tc.c, dx, dy, dz);
+    const uint32_t first = tc.start + sg * kSeg, end = min(first + kSeg, tc.end);
+    // the checkpoints and the segment's sums start empty (step (2) writes the
+    // chunks and segments in which the pixel composites something)
+    const int64_t cb = static_cast<int64_t>(cbase[tile]);
+    if (sg == 0 && lane == 0) bwm[tile * blocks + id % blocks] = 0u;   // (step (2) takes the maximum)
+    for (uint32_t c = sg * kSegChunks; c * kChunk < end - tc.start; ++c)
+#pragma unroll
+      for (int k = 0; k < kCkptSlots; ++k) ckpt[((cb + c) * kCkptSlots + k) * npx + vt] = 0.f;
+#pragma unroll
+    for (int k = 0; k < kSegSlots; ++k)
+      seg.sum[((static_cast<int64_t>(__ldg(seg.sbase + tile)) + sg) * kSegSlots + k) * npx + vt] = 0.f;
+    float T = 1.0f;
+    uint32_t item_nx = first + 32 + lane < end ? __ldg(pv + first + 32 + lane) : 0u;
+    uint32_t item_cur = first + lane < end ? __ldg(pv + first + lane) : 0u;
+    float4 box_cur = first + lane < end ? __ldg(box + item_cur) : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (uint32_t base = first; base < end; base += 32) {
+      if (__all_sync(0xffffffffu, done)) break;
+      uint32_t* mword = cmask + (cb * 4 + (base - tc.start) / 32) * npx + vt;
+      const uint32_t j = base + lane;
+      const uint32_t item = item_cur;
+      const float4 bx = box_cur;
+      item_cur = item_nx;
+      box_cur = j + 32 < end ? __ldg(box + item_nx) : make_float4(0.f, 0.f, 0.f, 0.f);
+      item_nx = j + 64 < end ? __ldg(pv + j + 64) : 0u;
+      bool hit;
+      uint32_t m = bb.candidates(bx, j < end, lane, hit);
+      if (done) m = 0u;
+      uint32_t cbits = 0;
+      if (__any_sync(0xffffffffu, m)) {
+        evals += __popc(m);
+        const int idle = __ffs(__ballot_sync(0xffffffffu, hit)) - 1;
+        __syncwarp();
+        if (hit) stage_hit(rec, item, sw, lane);
+        __syncwarp();
+        do {
+          int bq[FWD_HITS];
+          bool on[FWD_HITS];
+          Eval e[FWD_HITS];
+#pragma unroll
+          for (int q = 0; q < FWD_HITS; ++q) {
+            on[q] = m != 0u;
+            bq[q] = on[q] ? __ffs(m) - 1 : idle;
+            m &= m - 1;
+            eval_pair(sw.r0[bq[q]], sw.r1[bq[q]], sw.r2[bq[q]], sw.al[bq[q]], dx, dy, dz, e[q]);
+          }
+#pragma unroll
+          for (int q = 0; q < FWD_HITS; ++q) {
+            const bool ok = on[q] && e[q].valid;
+            cbits |= ok ? 1u << bq[q] : 0u;
+            T *= ok ? 1.0f - e[q].a : 1.0f;
+          }
+        } while (__any_sync(0xffffffffu, m));
+        if (!done && T < kSurelyStopped) {
+          done = true;
+          atomicMin(dead, sg);
+        }
+      }
+      *mword = cbits;
+    }
+  }
+  long_finish(&st->seg_counter, &st->seg_done, gridDim.x * (blockDim.x >> 5));
+  unsigned long long ev = evals;
+  for (int o = 16; o > 0; o >>= 1) ev += __shfl_xor_sync(0xffffffffu, ev, o);
+  if (lane == 0 && ev) atomicAdd(&st->evals_fwd, ev);
+}
+
+// The tiles with short lists: every CTA its own, or persistent ones claiming
+// them.  The long lists were composited before; with LOSS the CTA that finishes
+// last writes the loss vector.
 // At most 72 registers: 14 CTAs of an 8 x 8 tile (64 threads) per SM, so
 // the 2048 tiles of a 128 x 1024 frame fit in one wave on 152 SMs (75
 // registers leave 72 tiles for a second wave).
-template <bool LOSS>
+template <bool LOSS, bool BLOCK48>
 __global__ void __maxnreg__(72)
     k_fwd_s(const Desc* __restrict__ D, const uint2* __restrict__ ranges, const uint32_t* __restrict__ pv,
             const float4* __restrict__ rec, const float4* __restrict__ box, const uint32_t* __restrict__ order,
@@ -736,10 +975,10 @@ __global__ void __maxnreg__(72)
   uint32_t tile;
   uint32_t evals = 0, contrib = 0, alg = 0;
   for (int iter = 0; next_tile(persistent, order, D->n_tiles, &st->work_counter, tile, iter); ++iter) {
-    const TileCtx tc = tile_ctx(*D, tile, ranges);
-    if (tc.end - tc.start > kLongList) continue;   // the long-list kernels' tile
+    const TileCtx tc = tile_ctx(*D, tile, ranges, static_cast<int>(threadIdx.x));
+    if (tc.end - tc.start > kLongList) continue;   // k_fwd_long's tile
     const FrameDev& F = D->f[tc.f];
-    const WarpBox wb = warp_box(tc.inside, tc.r, tc.c, F.W);
+    const WarpPixels<BLOCK48> bb(F, tc, lane);
     float dx = 0.f, dy = 0.f, dz = 0.f;
     if (tc.inside) pixel_ray(F, tc.r, tc.c, dx, dy, dz);
     float T = 1.0f, A = 0.0f, St = 0.0f, Sx = 0.0f, Sy = 0.0f, Sz = 0.0f;
@@ -782,15 +1021,18 @@ __global__ void __maxnreg__(72)
       item_cur = item_nx;
       box_cur = j + 32 < tc.end ? __ldg(box + item_nx) : make_float4(0.f, 0.f, 0.f, 0.f);
       item_nx = j + 64 < tc.end ? __ldg(pv + j + 64) : 0u;
-      bool hit = false;
-      if (j < tc.end) hit = box_hits(bx, wb);
-      uint32_t m = __ballot_sync(0xffffffffu, hit);
-      if (!m) {
+      // the pixel's candidates of the window, one bit per entry
+      bool hit;
+      uint32_t m = bb.candidates(bx, j < tc.end, lane, hit);
+      if (done) m = 0u;
+      if (!__any_sync(0xffffffffu, m)) {
         *mword = 0u;
         continue;
       }
-      const uint32_t m_hits = m;
-      const bool done_before = done;
+      const uint32_t m_cand = m;
+      // a lane without a candidate evaluates a staged one with weight 0 (its
+      // record is finite; an unused slot may hold anything)
+      const int idle = __ffs(__ballot_sync(0xffffffffu, hit)) - 1;
       __syncwarp();
       if (hit) stage_hit(rec, item, sw, lane);
       __syncwarp();
@@ -822,38 +1064,34 @@ __global__ void __maxnreg__(72)
         stop_at = stop ? k0 + bq : stop_at;
         done = done || stop;
       };
-      // FWD_HITS hits per step: their evaluations are independent
-      // (instruction-level parallelism), the composites follow in list order
+      // every lane takes its own next FWD_HITS candidates: their evaluations
+      // are independent (instruction-level parallelism), the composites
+      // follow in list order
       do {
         int bq[FWD_HITS];
-        bq[0] = __ffs(m) - 1;
-        m &= m - 1;
-#pragma unroll
-        for (int q = 1; q < FWD_HITS; ++q) {
-          bq[q] = m ? __ffs(m) - 1 : -1;
-          m &= m - 1;
-        }
+        bool on[FWD_HITS];
         float4 r0q[FWD_HITS];
         Eval eq[FWD_HITS];
 #pragma unroll
         for (int q = 0; q < FWD_HITS; ++q) {
-          const int b = bq[q] >= 0 ? bq[q] : bq[0];
-          r0q[q] = sw.r0[b];
-          eval_pair(r0q[q], sw.r1[b], sw.r2[b], sw.al[b], dx, dy, dz, eq[q]);
+          on[q] = m != 0u;
+          bq[q] = on[q] ? __ffs(m) - 1 : idle;
+          m &= m - 1;
+          r0q[q] = sw.r0[bq[q]];
+          eval_pair(r0q[q], sw.r1[bq[q]], sw.r2[bq[q]], sw.al[bq[q]], dx, dy, dz, eq[q]);
+          eq[q].valid = eq[q].valid && on[q];
         }
 #pragma unroll
-        for (int q = 0; q < FWD_HITS; ++q)
-          if (bq[q] >= 0) composite(eq[q], r0q[q], bq[q]);
-        if (__all_sync(0xffffffffu, done)) break;
-      } while (m);
+        for (int q = 0; q < FWD_HITS; ++q) composite(eq[q], r0q[q], bq[q]);
+        if (done) m = 0u;
+      } while (__any_sync(0xffffffffu, m));
       *mword = cbits;
       // the window's statistics from its bits: composited pairs, the last
-      // one, and the hits evaluated before the pixel stopped (through the
-      // stop entry when it stopped in this window)
+      // one, and the candidates evaluated before the pixel stopped (through
+      // the stop entry when it stopped in this window)
       if (cbits) last = k0 + (31 - __clz(cbits));
       contrib += __popc(cbits);
-      if (!done_before)
-        evals += __popc(stop_at >= k0 ? m_hits & (0xffffffffu >> (31 - (stop_at - k0))) : m_hits);
+      evals += __popc(stop_at >= k0 ? m_cand & (0xffffffffu >> (31 - (stop_at - k0))) : m_cand);
     }
     if (tc.end > tc.start) checkpoint();
     if (tc.inside) {
@@ -881,6 +1119,251 @@ __global__ void __maxnreg__(72)
   if (lane == 0 && ev) atomicAdd(&st->evals_fwd, ev);
   if (lane == 0 && co) atomicAdd(&st->contrib_fwd, co);
   if (lane == 0 && al) atomicAdd(&st->alg_fwd, al);
+  if (LOSS) {
+    // every pixel's epilogue has added its terms when the last CTA is done
+    // (the regulariser was summed and the long lists composited before): it
+    // writes the loss vector
+    __shared__ bool s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&st->loss_ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (s_last && threadIdx.x < 32) finish_loss_vector(*D, loss.P, loss.ctot, loss.acc, loss.out, st);
+  }
+}
+
+// Thread of the per-tile forward that holds tile pixel (lr, lc) (the inverse
+// of pixel_of_thread): the chunk checkpoints and window masks are laid out by
+// it.
+__device__ __forceinline__ int thread_of_pixel(const FrameDev& F, int lr, int lc) {
+  if ((F.tw & 7) == 0 && (F.th & 3) == 0) {
+    const int wpr = F.tw >> 3;
+    return ((((lr >> 2) * wpr) + (lc >> 3)) << 5) | ((lr & 3) << 3) | (lc & 7);
+  }
+  return lr * F.tw + lc;
+}
+
+struct LongPix {
+  const FrameDev* F;
+  int r, c;
+  bool inside;
+  uint32_t start, end, tile, li;
+  int64_t pix;
+  int HW;
+  int vt;   // the pixel's thread in the per-tile layout (checkpoints, masks)
+};
+
+__device__ __forceinline__ bool long_item(const Desc& D, const uint2* __restrict__ ranges,
+                                          const uint32_t* __restrict__ longt, uint32_t n_long, uint32_t id,
+                                          LongPix& p) {
+  const uint32_t tp = static_cast<uint32_t>(D.th * D.tw);
+  const uint32_t gi = id / tp, k = id - gi * tp;
+  if (gi >= n_long) return false;
+  const uint32_t tile = longt[gi];
+  const int f = frame_of_tile(D, tile);
+  const FrameDev& F = D.f[f];
+  const int lt = static_cast<int>(tile - F.tile_base);
+  const int ti = lt / F.ntc, tj = lt - ti * F.ntc;
+  p.F = &F;
+  p.tile = tile;
+  p.li = gi;
+  p.vt = thread_of_pixel(F, static_cast<int>(k) / F.tw, static_cast<int>(k) % F.tw);
+  p.r = ti * F.th + static_cast<int>(k) / F.tw;
+  p.c = tj * F.tw + static_cast<int>(k) % F.tw;
+  p.inside = p.r < F.H && p.c < F.W;
+  p.pix = static_cast<int64_t>(p.r) * F.W + p.c;
+  p.HW = F.H * F.W;
+  const uint2 rg = ranges[tile];
+  p.start = rg.x;
+  p.end = rg.y;
+  return true;
+}
+
+__device__ __forceinline__ float warp_sum(float x) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  return x;
+}
+
+// Step (2) of the long lists: one warp per pixel (see above).  Software
+// pipeline over the non-empty windows: the entries two ahead and the records
+// one ahead are loaded while a window is composited.
+template <bool LOSS>
+__global__ void __launch_bounds__(256, 3) k_fwd_long(const Desc* __restrict__ D, const uint2* __restrict__ ranges,
+                                                  const uint32_t* __restrict__ pv, const float4* __restrict__ rec,
+                                                  Status* __restrict__ st, const uint32_t* __restrict__ cbase,
+                                                  float* __restrict__ ckpt, const uint32_t* __restrict__ cmask,
+                                                  uint32_t* __restrict__ bwm, LossEpi loss, SegBuf seg) {
+  pdl_wait();               // (launched after a kernel of this chain: wait for it)
+  pdl_launch_dependents();  // the next kernel may be dispatched now
+  const int lane = threadIdx.x & 31;
+  const uint32_t n_long = st->n_long;
+  if (n_long == 0) return;
+  const int npx = D->th * D->tw;
+  uint32_t contrib = 0, alg = 0;
+  LongPix P;
+  while (long_item(*D, ranges, seg.longt, n_long, warp_claim(&st->long_counter_fwd), P)) {
+    if (!P.inside) continue;
+    const FrameDev& F = *P.F;
+    float dx, dy, dz;
+    pixel_ray(F, P.r, P.c, dx, dy, dz);
+    float T = 1.f, A = 0.f, St = 0.f, Sx = 0.f, Sy = 0.f, Sz = 0.f;
+    int last = 0, stop_at = -1;
+    const int64_t cb = static_cast<int64_t>(cbase[P.tile]), sb = static_cast<int64_t>(seg.sbase[P.tile]);
+    const uint32_t* words = cmask + cb * 4 * npx + P.vt;
+    const uint32_t n_win = (P.end - P.start + 31) / 32;
+    // the chunked backward's inputs: T and the chunk's own sums at the end of
+    // every chunk in which the pixel composites something, and the segments'
+    // sums (the others are zero: step (1))
+    float cA = 0.f, cSt = 0.f, cSx = 0.f, cSy = 0.f, cSz = 0.f;
+    float g[kSegSlots] = {0.f, 0.f, 0.f, 0.f, 0.f};
+    uint32_t chunk = ~0u;   // the chunk being composited
+    const auto close_chunk = [&](uint32_t next) {
+      if (chunk == ~0u) return;
+      const float v[kSegSlots] = {warp_sum(cA), warp_sum(cSt), warp_sum(cSx), warp_sum(cSy), warp_sum(cSz)};
+      if (lane == 0) {
+        float* o = ckpt + ((cb + chunk) * kCkptSlots) * npx + P.vt;
+        o[0] = T;
+#pragma unroll
+        for (int q = 0; q < kSegSlots; ++q) o[(q + 1) * npx] = v[q];
+      }
+      cA = cSt = cSx = cSy = cSz = 0.f;
+#pragma unroll
+      for (int q = 0; q < kSegSlots; ++q) g[q] += v[q];
+      const uint32_t sg = chunk / kSegChunks;
+      if (next != ~0u && next / kSegChunks == sg) return;
+#pragma unroll
+      for (int q = 0; q < kSegSlots; ++q) {
+        if (lane == 0) seg.sum[((sb + sg) * kSegSlots + q) * npx + P.vt] = g[q];
+        g[q] = 0.f;
+      }
+    };
+    // the non-empty windows in order, found 32 mask words at a time (words
+    // past the pixel's stop are not set; the walk ends before it uses them)
+    uint32_t w0 = 0, word = static_cast<uint32_t>(lane) < n_win ? __ldg(words + static_cast<int64_t>(lane) * npx) : 0u;
+    uint32_t word_nx = 32u + lane < n_win ? __ldg(words + static_cast<int64_t>(32 + lane) * npx) : 0u;
+    uint32_t nz = __ballot_sync(0xffffffffu, word != 0u);
+    const auto advance = [&](uint32_t& win, uint32_t& bits) -> bool {
+      while (!nz) {
+        w0 += 32;
+        if (w0 >= n_win) return false;
+        word = word_nx;
+        word_nx = w0 + 32 + lane < n_win ? __ldg(words + static_cast<int64_t>(w0 + 32 + lane) * npx) : 0u;
+        nz = __ballot_sync(0xffffffffu, word != 0u);
+      }
+      const int b = __ffs(nz) - 1;
+      nz &= nz - 1;
+      bits = __shfl_sync(0xffffffffu, word, b);
+      win = w0 + b;
+      return true;
+    };
+    const auto entry = [&](bool on, uint32_t win, uint32_t bits) -> uint32_t {
+      const uint32_t j = P.start + 32 * win + lane;
+      return on && ((bits >> lane) & 1u) && j < P.end ? __ldg(pv + j) : ~0u;
+    };
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    const auto load = [&](uint32_t item, float4& r0, float4& r1, float4& r2, float& al) {
+      const float4* rp = rec + 4 * static_cast<int64_t>(item);
+      const bool on = item != ~0u;
+      r0 = on ? __ldg(rp) : zero;
+      r1 = on ? __ldg(rp + 1) : zero;
+      r2 = on ? __ldg(rp + 2) : zero;
+      al = on ? __ldg(reinterpret_cast<const float*>(rp + 3)) : 0.f;
+    };
+    uint32_t win = 0, bits = 0, win1 = 0, bits1 = 0, win2 = 0, bits2 = 0;
+    bool on = advance(win, bits);
+    uint32_t item = entry(on, win, bits);
+    bool on1 = on && advance(win1, bits1);
+    uint32_t item1 = entry(on1, win1, bits1);
+    float4 r0, r1, r2;
+    float al;
+    load(item, r0, r1, r2, al);
+    while (on) {
+      const bool on2 = on1 && advance(win2, bits2);
+      const uint32_t item2 = entry(on2, win2, bits2);
+      float4 q0, q1, q2;
+      float ql;
+      load(item1, q0, q1, q2, ql);
+      if (win / 4 != chunk) {
+        close_chunk(win / 4);
+        chunk = win / 4;
+      }
+      const bool valid = item != ~0u;
+      Eval e;
+      eval_pair(r0, r1, r2, al, dx, dy, dz, e);
+      // P_j = prod_{i <= j} (1 - a_i) over the valid lanes
+      float Pj = valid ? __fsub_rn(1.0f, e.a) : 1.0f;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const float y = __shfl_up_sync(0xffffffffu, Pj, o);
+        if (lane >= o) Pj *= y;
+      }
+      float Pex = __shfl_up_sync(0xffffffffu, Pj, 1);
+      if (lane == 0) Pex = 1.0f;
+      const uint32_t sm = __ballot_sync(0xffffffffu, valid && T * Pj < 1e-4f);
+      const int fs = sm ? __ffs(sm) - 1 : 32;
+      const bool inc = valid && lane < fs;
+      const float w = inc ? e.a * (T * Pex) : 0.f;
+      const float ws = valid && e.den > 0.f ? -w : w;
+      // every lane sums its own entries' terms; the pixel's totals are the
+      // warp sums of these after the walk
+      A += w;
+      if (inc) St = fmaf(w, e.t, St);
+      Sx = fmaf(ws, r0.x, Sx);
+      Sy = fmaf(ws, r0.y, Sy);
+      Sz = fmaf(ws, r0.z, Sz);
+      cA += w;
+      if (inc) cSt = fmaf(w, e.t, cSt);
+      cSx = fmaf(ws, r0.x, cSx);
+      cSy = fmaf(ws, r0.y, cSy);
+      cSz = fmaf(ws, r0.z, cSz);
+      contrib += inc;
+      const uint32_t im = __ballot_sync(0xffffffffu, inc);
+      if (im) last = static_cast<int>(32 * win) + (31 - __clz(im)) + 1;
+      T *= __shfl_sync(0xffffffffu, fs < 32 ? Pex : Pj, fs < 32 ? fs : 31);
+      if (sm) {
+        stop_at = static_cast<int>(32 * win) + fs + 1;
+        break;
+      }
+      on = on1;
+      win = win1;
+      bits = bits1;
+      item = item1;
+      on1 = on2;
+      win1 = win2;
+      bits1 = bits2;
+      item1 = item2;
+      r0 = q0;
+      r1 = q1;
+      r2 = q2;
+      al = ql;
+    }
+    close_chunk(~0u);
+    A = warp_sum(A);
+    St = warp_sum(St);
+    Sx = warp_sum(Sx);
+    Sy = warp_sum(Sy);
+    Sz = warp_sum(Sz);
+    if (lane == 0) {
+      F.A[P.pix] = A;
+      F.St[P.pix] = St;
+      F.Sn[P.pix] = Sx;
+      F.Sn[P.HW + P.pix] = Sy;
+      F.Sn[2 * static_cast<int64_t>(P.HW) + P.pix] = Sz;
+      F.Tf[P.pix] = T;
+      F.nc[P.pix] = last;
+      alg += stop_at >= 0 ? static_cast<uint32_t>(stop_at) : P.end - P.start;
+      seg.dead[static_cast<int64_t>(P.li) * npx + P.vt] = ~0u;   // for the next forward
+      if (last) atomicMax(bwm + (static_cast<int64_t>(P.tile) * npx + P.vt) / 32, static_cast<uint32_t>(last));
+    }
+    // the warp holds one pixel: lane 0 alone takes its loss terms
+    if (LOSS) loss_epilogue(*D, loss, static_cast<int>(P.F - D->f), lane == 0, P.pix, P.HW, A, St, Sx, Sy, Sz);
+  }
+  long_finish(&st->long_counter_fwd, &st->long_done_fwd, gridDim.x * (blockDim.x >> 5));
+  unsigned long long co = contrib, al64 = alg;
+  for (int o = 16; o > 0; o >>= 1) co += __shfl_xor_sync(0xffffffffu, co, o);
+  if (lane == 0 && co) atomicAdd(&st->contrib_fwd, co);
+  if (lane == 0 && al64) atomicAdd(&st->alg_fwd, al64);
 }
 
 __global__ void __launch_bounds__(kMaxTileThreads)
@@ -895,7 +1378,7 @@ __global__ void __launch_bounds__(kMaxTileThreads)
   uint32_t tile;
   uint32_t evals = 0, contrib = 0;
   for (int iter = 0; next_tile(persistent, order, D->n_tiles, &st->work_counter2, tile, iter); ++iter) {
-    const TileCtx tc = tile_ctx(*D, tile, ranges);
+    const TileCtx tc = tile_ctx(*D, tile, ranges, static_cast<int>(threadIdx.x));
     if (tc.end - tc.start > kLongList) continue;   // the long-list kernels' tile
     const FrameDev& F = D->f[tc.f];
     const WarpBox wb = warp_box(tc.inside, tc.r, tc.c, F.W);
@@ -1010,8 +1493,8 @@ __global__ void __launch_bounds__(kBwdChunkCta)
     k_bwd_c(const Desc* __restrict__ D, const uint2* __restrict__ ranges, const uint32_t* __restrict__ pv,
             const float4* __restrict__ rec, const float4* __restrict__ box, float* __restrict__ g13,
             const uint32_t* __restrict__ cbase, const float* __restrict__ ckpt, const uint32_t* __restrict__ cmask,
-            const float* __restrict__ csuf, const uint2* __restrict__ bq, uint32_t bq_cap0, uint32_t bq_capk,
-            Status* __restrict__ st) {
+            SegBuf seg, const float* __restrict__ ssuf, const uint2* __restrict__ bq, uint32_t bq_cap0,
+            uint32_t bq_capk, Status* __restrict__ st) {
   pdl_wait();               // (launched after a kernel of this chain: wait for it)
   pdl_launch_dependents();  // the next kernel may be dispatched now
   __shared__ WarpRecs s_w[kBwdChunkCta / 32];
@@ -1066,14 +1549,16 @@ __global__ void __launch_bounds__(kBwdChunkCta)
       gSz = F.gSn[2 * static_cast<int64_t>(HW) + pix];
       const float* o = ckpt + (static_cast<int64_t>(cbase[tile] + c) * kCkptSlots) * npx + vt;
       T = o[0];
+      uint32_t c_last = static_cast<uint32_t>(nc - 1) / kChunk;
       if (rg.y - rg.x > kLongList) {
-        S = csuf[static_cast<int64_t>(cbase[tile] + c) * npx + vt];   // the suffix k_bwd_prep wrote
-      } else {
-        const uint32_t c_last = static_cast<uint32_t>(nc - 1) / kChunk;
-        for (uint32_t c2 = c + 1; c2 <= c_last; ++c2) {
-          const float* q = ckpt + (static_cast<int64_t>(cbase[tile] + c2) * kCkptSlots) * npx + vt;
-          S += gA * q[npx] + gSt * q[2 * npx] + gSx * q[3 * npx] + gSy * q[4 * npx] + gSz * q[5 * npx];
-        }
+        // a long list: the segments after the chunk's are in the suffix that
+        // k_bwd_prep wrote
+        S = ssuf[static_cast<int64_t>(__ldg(seg.sbase + tile) + c / kSegChunks) * npx + vt];
+        c_last = min(c_last, c / kSegChunks * kSegChunks + kSegChunks - 1);
+      }
+      for (uint32_t c2 = c + 1; c2 <= c_last; ++c2) {
+        const float* q = ckpt + (static_cast<int64_t>(cbase[tile] + c2) * kCkptSlots) * npx + vt;
+        S += gA * q[npx] + gSt * q[2 * npx] + gSx * q[3 * npx] + gSy * q[4 * npx] + gSz * q[5 * npx];
       }
     }
     // entries [k_lo, k_hi) of the list, walked down in 32-entry steps: a
@@ -1154,263 +1639,12 @@ __global__ void __launch_bounds__(kBwdChunkCta)
   // composited pairs, counted there)
 }
 
-// ---------------------------------------------------------------------------
-// Long lists (more than kLongList entries): one warp per pixel
-// ---------------------------------------------------------------------------
-// A tile with a very long list (a far horizon seen along a street: tens of
-// thousands of entries, few of which any pixel composites) would make its
-// CTA walk the list one entry at a time while the rest of the frame is done.
-// Here a work item is one (long tile, pixel), claimed through an atomic
-// counter; the 32 lanes take 32 consecutive entries of the list for the
-// warp's pixel.  Forward: the transmittance before each entry is T times a
-// multiplicative scan of (1 - a) over the lanes, the early stop is the first
-// lane whose T (1 - a) falls below 1e-4, and the composited sums are warp
-// reductions.  Backward: from T_final, the transmittance before each entry
-// is T divided by the suffix product of (1 - a), the suffix S a suffix sum;
-// every valid lane adds its own entry's 12 moments with atomics.  The products
-// and sums associate differently from the per-tile kernels (same values to a
-// few ulps).
-// Thread of the per-tile forward that holds tile pixel (lr, lc) (the inverse
-// of pixel_of_thread): the chunk checkpoints and window masks are laid out by
-// it.
-__device__ __forceinline__ int thread_of_pixel(const FrameDev& F, int lr, int lc) {
-  if ((F.tw & 7) == 0 && (F.th & 3) == 0) {
-    const int wpr = F.tw >> 3;
-    return ((((lr >> 2) * wpr) + (lc >> 3)) << 5) | ((lr & 3) << 3) | (lc & 7);
-  }
-  return lr * F.tw + lc;
-}
-
-struct LongPix {
-  const FrameDev* F;
-  int r, c;
-  bool inside;
-  uint32_t start, end, tile;
-  int64_t pix;
-  int HW;
-  int vt;   // the pixel's thread in the per-tile layout (checkpoints, masks)
-};
-
-__device__ __forceinline__ bool long_item(const Desc& D, const uint2* __restrict__ ranges,
-                                          const uint32_t* __restrict__ longt, uint32_t n_long, uint32_t id,
-                                          LongPix& p) {
-  const uint32_t tp = static_cast<uint32_t>(D.th * D.tw);
-  const uint32_t gi = id / tp, k = id - gi * tp;
-  if (gi >= n_long) return false;
-  const uint32_t tile = longt[gi];
-  const int f = frame_of_tile(D, tile);
-  const FrameDev& F = D.f[f];
-  const int lt = static_cast<int>(tile - F.tile_base);
-  const int ti = lt / F.ntc, tj = lt - ti * F.ntc;
-  p.F = &F;
-  p.tile = tile;
-  p.vt = thread_of_pixel(F, static_cast<int>(k) / F.tw, static_cast<int>(k) % F.tw);
-  p.r = ti * F.th + static_cast<int>(k) / F.tw;
-  p.c = tj * F.tw + static_cast<int>(k) % F.tw;
-  p.inside = p.r < F.H && p.c < F.W;
-  p.pix = static_cast<int64_t>(p.r) * F.W + p.c;
-  p.HW = F.H * F.W;
-  const uint2 rg = ranges[tile];
-  p.start = rg.x;
-  p.end = rg.y;
-  return true;
-}
-
-__device__ __forceinline__ uint32_t warp_claim(unsigned int* counter) {
-  uint32_t id = 0;
-  if ((threadIdx.x & 31) == 0) id = atomicAdd(counter, 1u);
-  return __shfl_sync(0xffffffffu, id, 0);
-}
-
-// A warp that finds no work left counts itself done; the last one resets the
-// work and done counters to zero for the next launch on the stream.
-__device__ __forceinline__ void long_finish(unsigned int* counter, unsigned int* done) {
-  if ((threadIdx.x & 31) == 0) {
-    __threadfence();
-    const unsigned int total = gridDim.x * (blockDim.x >> 5);
-    if (atomicAdd(done, 1u) == total - 1) {
-      *counter = 0u;
-      *done = 0u;
-    }
-  }
-}
-
-__device__ __forceinline__ float warp_sum(float x) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-  return x;
-}
-
-// Four CTAs per SM (64 registers): with the loads pipelined below, 32 warps
-// per SM measured faster than 24 at 72 registers (batched forward 8.0 against
-// 8.5 ms).
-template <bool LOSS>
-__global__ void __launch_bounds__(256, 4) k_fwd_long(const Desc* __restrict__ D, const uint2* __restrict__ ranges,
-                                                  const uint32_t* __restrict__ pv, const float4* __restrict__ rec,
-                                                  const float4* __restrict__ box,
-                                                  const uint32_t* __restrict__ longt, Status* __restrict__ st,
-                                                  const uint32_t* __restrict__ cbase, float* __restrict__ ckpt,
-                                                  uint32_t* __restrict__ cmask, LossEpi loss) {
-  pdl_wait();               // (launched after a kernel of this chain: wait for it)
-  pdl_launch_dependents();  // the next kernel may be dispatched now
-  const int lane = threadIdx.x & 31;
-  const uint32_t n_long = st->n_long;
-  if (n_long == 0) {
-    // no long list: the per-tile forward before it on the stream has added
-    // every pixel's loss terms, so one warp writes the loss vector at once
-    // (no ticket over the grid)
-    if (LOSS && blockIdx.x == 0 && threadIdx.x < 32)
-      finish_loss_vector(*D, loss.P, loss.ctot, loss.acc, loss.out, st);
-    return;
-  }
-  uint32_t evals = 0, contrib = 0, alg = 0;
-  LongPix P;
-  while (long_item(*D, ranges, longt, n_long, warp_claim(&st->long_counter_fwd), P)) {
-    if (!P.inside) continue;
-    const FrameDev& F = *P.F;
-    float dx, dy, dz;
-    pixel_ray(F, P.r, P.c, dx, dy, dz);
-    WarpBox pb;
-    pb.r0 = pb.r1 = static_cast<float>(P.r);
-    pb.cmid = static_cast<float>(P.c);
-    pb.chalf = 0.f;
-    pb.W = static_cast<float>(F.W);
-    float T = 1.f, A = 0.f, St = 0.f, Sx = 0.f, Sy = 0.f, Sz = 0.f;
-    int last = 0, stop_at = -1;
-    // the chunked backward's inputs, laid out as the per-tile forward's: the
-    // pixel's composited entries of every window it walks (one bit each) and,
-    // at the end of every chunk it walks, T and the chunk's own sums
-    const int npx = D->th * D->tw;
-    const int64_t cb = static_cast<int64_t>(cbase[P.tile]);
-    float cA = 0.f, cSt = 0.f, cSx = 0.f, cSy = 0.f, cSz = 0.f;
-    const auto checkpoint = [&](uint32_t chunk) {
-      const float a = warp_sum(cA), b = warp_sum(cSt), x = warp_sum(cSx), y = warp_sum(cSy), z = warp_sum(cSz);
-      if (lane == 0) {
-        float* o = ckpt + ((cb + chunk) * kCkptSlots) * npx + P.vt;
-        o[0] = T;
-        o[npx] = a;
-        o[2 * npx] = b;
-        o[3 * npx] = x;
-        o[4 * npx] = y;
-        o[5 * npx] = z;
-      }
-      cA = cSt = cSx = cSy = cSz = 0.f;
-    };
-    uint32_t win = 0;
-    // software pipeline over the windows: the list entry two windows ahead
-    // and the culling box one window ahead are loaded while this window is
-    // composited (each window's loads would otherwise form a chain of
-    // dependent round trips: entry, then box, then record)
-    uint32_t item_next = P.start + 32 + lane < P.end ? __ldg(pv + P.start + 32 + lane) : 0u;
-    uint32_t item_cur = P.start + lane < P.end ? __ldg(pv + P.start + lane) : 0u;
-    float4 box_cur = P.start + lane < P.end ? __ldg(box + item_cur) : make_float4(0.f, 0.f, 0.f, 0.f);
-    for (uint32_t base = P.start; base < P.end; base += 32, ++win) {
-      if (win > 0 && win % 4 == 0) checkpoint(win / 4 - 1);
-      uint32_t* mword = cmask + (cb * 4 + win) * npx + P.vt;
-      const uint32_t j = base + lane;
-      const uint32_t item = item_cur;
-      const float4 bx = box_cur;
-      item_cur = item_next;
-      box_cur = j + 32 < P.end ? __ldg(box + item_next) : make_float4(0.f, 0.f, 0.f, 0.f);
-      item_next = j + 64 < P.end ? __ldg(pv + j + 64) : 0u;
-      bool valid = false;
-      Eval e;
-      float nx = 0.f, ny = 0.f, nz = 0.f;
-      if (j < P.end) {
-        if (box_hits(bx, pb)) {
-          const float4* rp = rec + 4 * static_cast<int64_t>(item);
-          const float4 r0 = __ldg(rp);
-          eval_pair(r0, __ldg(rp + 1), __ldg(rp + 2), __ldg(reinterpret_cast<const float*>(rp + 3)), dx, dy, dz, e);
-          valid = e.valid;
-          nx = r0.x; ny = r0.y; nz = r0.z;
-          ++evals;
-        }
-      }
-      // a window without a valid pair leaves T and the sums as they are
-      if (!__any_sync(0xffffffffu, valid)) {
-        if (lane == 0) *mword = 0u;
-        continue;
-      }
-      // P_j = prod_{i <= j} (1 - a_i) over the valid lanes
-      float Pj = valid ? __fsub_rn(1.0f, e.a) : 1.0f;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const float y = __shfl_up_sync(0xffffffffu, Pj, o);
-        if (lane >= o) Pj *= y;
-      }
-      float Pex = __shfl_up_sync(0xffffffffu, Pj, 1);
-      if (lane == 0) Pex = 1.0f;
-      const uint32_t sm = __ballot_sync(0xffffffffu, valid && T * Pj < 1e-4f);
-      const int fs = sm ? __ffs(sm) - 1 : 32;
-      const bool inc = valid && lane < fs;
-      const float w = inc ? e.a * (T * Pex) : 0.f;
-      const float ws = valid && e.den > 0.f ? -w : w;
-      // every lane sums its own entries' terms; the pixel's totals are the
-      // warp sums of these after the walk
-      A += w;
-      if (inc) St = fmaf(w, e.t, St);   // (e is unset on lanes without a box hit)
-      Sx = fmaf(ws, nx, Sx);
-      Sy = fmaf(ws, ny, Sy);
-      Sz = fmaf(ws, nz, Sz);
-      cA += w;
-      if (inc) cSt = fmaf(w, e.t, cSt);
-      cSx = fmaf(ws, nx, cSx);
-      cSy = fmaf(ws, ny, cSy);
-      cSz = fmaf(ws, nz, cSz);
-      contrib += inc;
-      const uint32_t im = __ballot_sync(0xffffffffu, inc);
-      if (lane == 0) *mword = im;
-      if (im) last = static_cast<int>(base - P.start) + (31 - __clz(im)) + 1;
-      T *= __shfl_sync(0xffffffffu, fs < 32 ? Pex : Pj, fs < 32 ? fs : 31);
-      if (sm) {
-        stop_at = static_cast<int>(base - P.start) + fs + 1;
-        break;
-      }
-    }
-    // the chunk holding the walk's last window (the list end or the stop)
-    if (P.end > P.start) checkpoint((win > 0 && stop_at < 0 ? win - 1 : win) / 4);
-    A = warp_sum(A);
-    St = warp_sum(St);
-    Sx = warp_sum(Sx);
-    Sy = warp_sum(Sy);
-    Sz = warp_sum(Sz);
-    if (lane == 0) {
-      F.A[P.pix] = A;
-      F.St[P.pix] = St;
-      F.Sn[P.pix] = Sx;
-      F.Sn[P.HW + P.pix] = Sy;
-      F.Sn[2 * static_cast<int64_t>(P.HW) + P.pix] = Sz;
-      F.Tf[P.pix] = T;
-      F.nc[P.pix] = last;
-      alg += stop_at >= 0 ? static_cast<uint32_t>(stop_at) : P.end - P.start;
-    }
-    // the warp holds one pixel: lane 0 alone takes its loss terms
-    if (LOSS) loss_epilogue(*D, loss, static_cast<int>(P.F - D->f), lane == 0, P.pix, P.HW, A, St, Sx, Sy, Sz);
-  }
-  long_finish(&st->long_counter_fwd, &st->long_done_fwd);
-  unsigned long long ev = evals, co = contrib, al = alg;
-  for (int o = 16; o > 0; o >>= 1) {
-    ev += __shfl_xor_sync(0xffffffffu, ev, o);
-    co += __shfl_xor_sync(0xffffffffu, co, o);
-  }
-  if (lane == 0 && ev) atomicAdd(&st->evals_fwd, ev);
-  if (lane == 0 && co) atomicAdd(&st->contrib_fwd, co);
-  if (lane == 0 && al) atomicAdd(&st->alg_fwd, al);
-  if (LOSS) {
-    // this launch follows the per-tile forward on the stream, so when its
-    // last CTA is done every pixel's epilogue has added its terms: that CTA
-    // writes the loss vector (the regulariser was summed before the forward)
-    __shared__ bool s_last;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      __threadfence();
-      s_last = atomicAdd(&st->loss_ticket, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (s_last && threadIdx.x < 32) finish_loss_vector(*D, loss.P, loss.ctot, loss.acc, loss.out, st);
-  }
-}
-
+// Long lists in the backward of the tunings without chunks: a work item is one
+// (long tile, pixel), claimed through an atomic counter; the 32 lanes take 32
+// consecutive entries of the list for the warp's pixel.  From T_final, the
+// transmittance before each entry is T divided by the suffix product of (1 - a)
+// over the lanes, the suffix S a suffix sum; every valid lane adds its own
+// entry's 12 moments with atomics.
 __global__ void __launch_bounds__(256) k_bwd_long(const Desc* __restrict__ D, const uint2* __restrict__ ranges,
                                                   const uint32_t* __restrict__ pv, const float4* __restrict__ rec,
                                                   const float4* __restrict__ box, float* __restrict__ g13,
@@ -1492,7 +1726,7 @@ __global__ void __launch_bounds__(256) k_bwd_long(const Desc* __restrict__ D, co
       S += __shfl_sync(0xffffffffu, Cs, 0);
     }
   }
-  long_finish(&st->long_counter_bwd, &st->long_done_bwd);
+  long_finish(&st->long_counter_bwd, &st->long_done_bwd, gridDim.x * (blockDim.x >> 5));
   unsigned long long ev = evals, co = contrib;
   for (int o = 16; o > 0; o >>= 1) {
     ev += __shfl_xor_sync(0xffffffffu, ev, o);
@@ -1504,31 +1738,30 @@ __global__ void __launch_bounds__(256) k_bwd_long(const Desc* __restrict__ D, co
 
 // Before the chunked backward (one launch):
 // (1) its work queues, from the forward's largest n_contrib of every (tile,
-//     warp block) (a long list: its length): one thread per tile, warp-
+//     warp block): one thread per tile, warp-
 //     aggregated reservations (one atomic per warp for class 0, one per
 //     class present and block for the others).  A tile's full chunks are
 //     queued chunk by chunk, its blocks side by side: they read the same
 //     list entries, so warps that claim them together share those loads in
 //     L2.  The queue sizes are zero on entry (cleared with the claim
 //     counter).
-// (2) over the long lists: the suffix S of every chunk (the sum over the
-//     pixel's later chunks c' of gA dA_c' + gSt dSt_c' + gS . dSn_c'),
-//     written to a buffer of its own (the checkpoints stay as the forward
-//     wrote them, for any further backward), so that k_bwd_c reads it
-//     instead of summing, per work item, up to thousands of later chunks.
-//     One CTA per (long tile, warp block): its eight warps split the
-//     block's chunks into segments (lane = pixel), sum their segment while
-//     parking every chunk's term in the suffix buffer, add up the later
-//     segments' sums in shared memory, then walk their segment down.  A
-//     list of 2,000 chunks is eight chains of 250, not one of 2,000.
+// (2) over the long lists: the suffix S of every segment (the sum over the
+//     pixel's later segments s' of gA dA_s' + gSt dSt_s' + gS . dSn_s'), so
+//     that k_bwd_c sums the later chunks of one segment only instead of, per
+//     work item, up to thousands of them.  One CTA per (long tile, warp
+//     block): its eight warps split the block's segments into parts (lane =
+//     pixel), sum their part while parking every segment's term in the suffix
+//     buffer, add up the later parts' sums in shared memory, then walk their
+//     part down.
 constexpr int kMaxBlocks = kMaxTileThreads / 32;
+constexpr uint32_t kPrepChunks = 16;   // full chunks that one lane queues
 
 __global__ void __launch_bounds__(256) k_bwd_prep(const Desc* __restrict__ D, const uint2* __restrict__ ranges,
-                                                  const uint32_t* __restrict__ longt, Status* __restrict__ st,
+                                                  Status* __restrict__ st,
                                                   const uint32_t* __restrict__ cbase,
                                                   const uint32_t* __restrict__ bwm, uint2* __restrict__ bq,
-                                                  uint32_t cap0, uint32_t capk,
-                                                  const float* __restrict__ ckpt, float* __restrict__ csuf) {
+                                                  uint32_t cap0, uint32_t capk, SegBuf seg,
+                                                  float* __restrict__ ssuf) {
   pdl_wait();               // (launched after a kernel of this chain: wait for it)
   pdl_launch_dependents();  // the next kernel may be dispatched now
   const int lane = threadIdx.x & 31;
@@ -1538,14 +1771,11 @@ __global__ void __launch_bounds__(256) k_bwd_prep(const Desc* __restrict__ D, co
   for (uint32_t t0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); t0 < n_tiles; t0 += gridDim.x * blockDim.x) {
     const uint32_t tile = t0 + static_cast<uint32_t>(lane);
     const bool ok = tile < n_tiles;
-    // a long list's blocks take every chunk (its pixels' walks end in
-    // k_fwd_long, which keeps no per-block maximum)
-    const uint32_t len = ok ? ranges[tile].y - ranges[tile].x : 0u;
     uint32_t wm[kMaxBlocks];
     uint32_t nfull = 0, nf_max = 0;
 #pragma unroll
     for (int b = 0; b < kMaxBlocks; ++b) {
-      wm[b] = ok && static_cast<uint32_t>(b) < blocks ? (len > kLongList ? len : bwm[tile * blocks + b]) : 0u;
+      wm[b] = ok && static_cast<uint32_t>(b) < blocks ? bwm[tile * blocks + b] : 0u;
       nfull += wm[b] / kChunk;
       nf_max = max(nf_max, wm[b] / kChunk);
     }
@@ -1560,13 +1790,44 @@ __global__ void __launch_bounds__(256) k_bwd_prep(const Desc* __restrict__ D, co
     uint32_t pos = 0;
     if (lane == 31 && incl) pos = atomicAdd(&st->bq_count[0], incl);
     pos = __shfl_sync(0xffffffffu, pos, 31) + incl - nfull;
-    for (uint32_t c = 0; c < nf_max; ++c) {
+    // (a tile with more than a few full chunks is queued by the whole warp:
+    // one lane writing a long list's thousands of items took 0.4 ms)
+    const bool many = nf_max > kPrepChunks;
+    for (uint32_t c = 0; c < (many ? 0u : nf_max); ++c) {
 #pragma unroll
       for (int b = 0; b < kMaxBlocks; ++b) {
         if (c < wm[b] / kChunk) {
           if (pos < cap0) bq[pos] = make_uint2((c0 + c) * blocks + static_cast<uint32_t>(b), tile);
           ++pos;
         }
+      }
+    }
+    for (uint32_t big = __ballot_sync(0xffffffffu, many); big; big &= big - 1) {
+      const int src = __ffs(big) - 1;
+      uint32_t full[kMaxBlocks];
+#pragma unroll
+      for (int b = 0; b < kMaxBlocks; ++b) full[b] = __shfl_sync(0xffffffffu, wm[b] / kChunk, src);
+      const uint32_t nc = __shfl_sync(0xffffffffu, nf_max, src), cb = __shfl_sync(0xffffffffu, c0, src);
+      uint32_t at = __shfl_sync(0xffffffffu, pos, src);
+      for (uint32_t cc = 0; cc < nc; cc += 32) {
+        const uint32_t c = cc + static_cast<uint32_t>(lane);
+        uint32_t n = 0;
+#pragma unroll
+        for (int b = 0; b < kMaxBlocks; ++b) n += c < full[b];
+        uint32_t o = n;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+          const uint32_t x = __shfl_up_sync(0xffffffffu, o, d);
+          if (lane >= d) o += x;
+        }
+        uint32_t k = at + o - n;
+#pragma unroll
+        for (int b = 0; b < kMaxBlocks; ++b)
+          if (c < full[b]) {
+            if (k < cap0) bq[k] = make_uint2((cb + c) * blocks + static_cast<uint32_t>(b), t0 + static_cast<uint32_t>(src));
+            ++k;
+          }
+        at += __shfl_sync(0xffffffffu, o, 31);
       }
     }
     // every block's chunk holding its last entry: the class of its walked
@@ -1585,100 +1846,117 @@ __global__ void __launch_bounds__(256) k_bwd_prep(const Desc* __restrict__ D, co
         bq[cap0 + (cls - 1) * capk + bk] = make_uint2((c0 + wm[b] / kChunk) * blocks + static_cast<uint32_t>(b), tile);
     }
   }
-  // (2) requires 256 threads (eight segments); CTA-uniform loop
-  __shared__ float s_seg[8][32];
+  // (2) requires 256 threads (eight parts); CTA-uniform loop
+  __shared__ float s_part[8][32];
   const uint32_t n_long = st->n_long;
   const int npx = static_cast<int>(blocks) * 32;
-  const int wseg = threadIdx.x >> 5;
+  const int part = threadIdx.x >> 5;
   for (uint32_t it = blockIdx.x; it < n_long * blocks; it += gridDim.x) {
     const uint32_t lt = it / blocks, blk = it - lt * blocks;
-    const uint32_t tile = longt[lt];
-    const FrameDev& F = D->f[frame_of_tile(*D, tile)];
-    const int ltile = static_cast<int>(tile - F.tile_base);
-    const int ti = ltile / F.ntc, tj = ltile - ti * F.ntc;
+    const uint32_t tile = seg.longt[lt];
     const int vt = static_cast<int>(blk) * 32 + lane;
-    int lr, lc;
-    pixel_of_thread(F, vt, lr, lc);
-    const int r = ti * F.th + lr, col = tj * F.tw + lc;
-    const int64_t pix = static_cast<int64_t>(r) * F.W + col;
-    const int HW = F.H * F.W;
-    const int nc = r < F.H && col < F.W ? F.nc[pix] : 0;
-    const int cl = nc > 0 ? (nc - 1) / static_cast<int>(kChunk) + 1 : 0;   // the pixel's chunks
-    const int seg = (__reduce_max_sync(0xffffffffu, static_cast<uint32_t>(cl)) + 7) / 8;
-    const int lo = wseg * seg, hi = min(lo + seg, cl);
+    const TileCtx tc = tile_ctx(*D, tile, ranges, vt);
+    const FrameDev& F = D->f[tc.f];
+    const int nc = tc.inside ? F.nc[tc.pix] : 0;
+    const int ns = nc > 0 ? (nc - 1) / static_cast<int>(kSeg) + 1 : 0;   // the pixel's segments
+    const int per = (__reduce_max_sync(0xffffffffu, ns) + 7) / 8;
+    const int lo = part * per, hi = min(lo + per, ns);
     float gA = 0.f, gSt = 0.f, gSx = 0.f, gSy = 0.f, gSz = 0.f;
     if (hi > lo) {
-      gA = F.gA[pix];
-      gSt = F.gSt[pix];
-      gSx = F.gSn[pix];
-      gSy = F.gSn[HW + pix];
-      gSz = F.gSn[2 * static_cast<int64_t>(HW) + pix];
+      gA = F.gA[tc.pix];
+      gSt = F.gSt[tc.pix];
+      gSx = F.gSn[tc.pix];
+      gSy = F.gSn[tc.HW + tc.pix];
+      gSz = F.gSn[2 * static_cast<int64_t>(tc.HW) + tc.pix];
     }
-    const int64_t cb = static_cast<int64_t>(cbase[tile]);
-    // pass 1: every chunk's term (parked in csuf) and the segment's sum
+    const int64_t s0 = static_cast<int64_t>(seg.sbase[tile]);
+    // pass 1: every segment's term (parked in ssuf) and the part's sum
     float tot = 0.f;
-    for (int c = hi - 1; c >= lo; c -= 8) {
-      float v[8];
+    for (int s = hi - 1; s >= lo; s -= 4) {
+      float v[4];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
+      for (int u = 0; u < 4; ++u) {
         v[u] = 0.f;
-        if (c - u >= lo) {
-          const float* q = ckpt + (cb + c - u) * kCkptSlots * npx + vt;
-          v[u] = gA * q[npx] + gSt * q[2 * npx] + gSx * q[3 * npx] + gSy * q[4 * npx] + gSz * q[5 * npx];
+        if (s - u >= lo) {
+          const float* q = seg.sum + (s0 + s - u) * kSegSlots * npx + vt;
+          v[u] = gA * q[0] + gSt * q[npx] + gSx * q[2 * npx] + gSy * q[3 * npx] + gSz * q[4 * npx];
         }
       }
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        if (c - u >= lo) {
-          csuf[(cb + c - u) * npx + vt] = v[u];
+      for (int u = 0; u < 4; ++u) {
+        if (s - u >= lo) {
+          ssuf[(s0 + s - u) * npx + vt] = v[u];
           tot += v[u];
         }
       }
     }
-    s_seg[wseg][lane] = tot;
+    s_part[part][lane] = tot;
     __syncthreads();
     float S = 0.f;
-    for (int w2 = 7; w2 > wseg; --w2) S += s_seg[w2][lane];
-    // pass 2: the suffix before every chunk of the segment, walking down
-    for (int c = hi - 1; c >= lo; c -= 8) {
+    for (int w2 = 7; w2 > part; --w2) S += s_part[w2][lane];
+    // pass 2: the suffix after every segment of the part, walking down
+    for (int s = hi - 1; s >= lo; s -= 8) {
       float v[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) v[u] = c - u >= lo ? csuf[(cb + c - u) * npx + vt] : 0.f;
+      for (int u = 0; u < 8; ++u) v[u] = s - u >= lo ? ssuf[(s0 + s - u) * npx + vt] : 0.f;
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
-        if (c - u >= lo) {
-          csuf[(cb + c - u) * npx + vt] = S;
+        if (s - u >= lo) {
+          ssuf[(s0 + s - u) * npx + vt] = S;
           S += v[u];
         }
       }
     }
-    __syncthreads();   // s_seg is rewritten by the next item
+    __syncthreads();   // s_part is rewritten by the next item
   }
 }
 
 // The work counters start at zero (reset at binning and by the last warp of
 // every launch), so no memset precedes the launch.
-static cudaError_t launch_long(bool fwd, const WsPtrs& w, const uint32_t* pv, cudaStream_t s,
-                               const LossEpi* loss = nullptr) {
+static cudaError_t launch_bwd_long(const WsPtrs& w, const uint32_t* pv, cudaStream_t s) {
   int dev = 0, sms = 152, per_sm = 2;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   // as many CTAs as fit (the walks are bound by load latency); warps claim
   // (tile, pixel) items until none are left
-  if (fwd && loss) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fwd_long<true>, 256, 0);
-  else if (fwd) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fwd_long<false>, 256, 0);
-  else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bwd_long, 256, 0);
-  const int grid = sms * (per_sm > 0 ? per_sm : 1);
-  // (a plain launch: dispatched during the shared-memory forward, its CTAs
-  // made the 16-map batch's long-list forward 7.9 -> 14.7 ms)
-  if (fwd && loss)
-    k_fwd_long<true><<<grid, 256, 0, s>>>(w.desc, w.ranges, pv, w.rec, w.box, w.longt, w.st, w.cbase, w.ckpt, w.cmask,
-                                          *loss);
-  else if (fwd)
-    k_fwd_long<false><<<grid, 256, 0, s>>>(w.desc, w.ranges, pv, w.rec, w.box, w.longt, w.st, w.cbase, w.ckpt,
-                                           w.cmask, LossEpi{});
-  else k_bwd_long<<<grid, 256, 0, s>>>(w.desc, w.ranges, pv, w.rec, w.box, w.g13, w.longt, w.st);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bwd_long, 256, 0);
+  k_bwd_long<<<sms * (per_sm > 0 ? per_sm : 1), 256, 0, s>>>(w.desc, w.ranges, pv, w.rec, w.box, w.g13, w.longt, w.st);
   return cudaGetLastError();
+}
+
+static SegBuf seg_buf(const WsPtrs& w) { return SegBuf{w.segs, w.longt, w.sbase, w.segsum, w.dead}; }
+
+// Whether a map is large enough for a list to be long.
+static bool may_be_long(const Desc& h) {
+  int64_t most = 0;
+  for (int f = 0; f < h.n_frames; ++f) most = h.f[f].n > most ? h.f[f].n : most;
+  return most > static_cast<int64_t>(kLongList);
+}
+
+// 4 x 8 pixel blocks per warp (pixel_of_thread)
+static bool block48(const Desc& h) { return (h.tw & 7) == 0 && (h.th & 3) == 0; }
+
+// The long lists, before the tiles with short ones; `after_kernel`: they follow
+// a kernel of this call.  Without long lists both are early exits whose launch
+// overlaps the kernel before.
+static cudaError_t launch_fwd_long(const WsPtrs& w, const Desc& h, const uint32_t* pv, cudaStream_t s,
+                                   bool after_kernel, const LossEpi* loss) {
+  int dev = 0, sms = 152;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const auto masks = block48(h) ? k_long_masks<true> : k_long_masks<false>;
+  cudaError_t e;
+  if (after_kernel) {
+    e = launch_dep(masks, dim3(3 * sms), dim3(256), 0, s, w.desc, w.ranges, pv, w.rec, w.box, w.st, w.cbase, w.ckpt,
+                   w.cmask, w.bwm, seg_buf(w));
+  } else {
+    masks<<<3 * sms, 256, 0, s>>>(w.desc, w.ranges, pv, w.rec, w.box, w.st, w.cbase, w.ckpt, w.cmask, w.bwm,
+                                  seg_buf(w));
+    e = cudaGetLastError();
+  }
+  if (e != cudaSuccess) return e;
+  return launch_dep(loss ? k_fwd_long<true> : k_fwd_long<false>, dim3(3 * sms), dim3(256), 0, s, w.desc, w.ranges, pv,
+                    w.rec, w.st, w.cbase, w.ckpt, w.cmask, w.bwm, loss ? *loss : LossEpi{}, seg_buf(w));
 }
 
 // ---------------------------------------------------------------------------
@@ -1717,8 +1995,8 @@ static cudaError_t launch_raster_fwd_tiles(const WsPtrs& w, const Desc& h, const
   switch (batch) {
     case 0:
       if (group == 16)
-        k_fwd_s<false><<<grid, h.th * h.tw, 0, s>>>(w.desc, w.ranges, pv, w.rec, w.box, ord, w.st, persistent,
-                                                    w.cbase, w.ckpt, w.cmask, w.bwm, LossEpi{});
+        (block48(h) ? k_fwd_s<false, true> : k_fwd_s<false, false>)<<<grid, h.th * h.tw, 0, s>>>(
+            w.desc, w.ranges, pv, w.rec, w.box, ord, w.st, persistent, w.cbase, w.ckpt, w.cmask, w.bwm, LossEpi{});
       else if (group == 1) k_fwd_w<1><<<grid, h.th * h.tw, 0, s>>>(w.desc, w.ranges, pv, w.rec, w.box, ord, w.st, persistent);
       else if (group == 2) k_fwd_w<2><<<grid, h.th * h.tw, 0, s>>>(w.desc, w.ranges, pv, w.rec, w.box, ord, w.st, persistent);
       else k_fwd_w<4><<<grid, h.th * h.tw, 0, s>>>(w.desc, w.ranges, pv, w.rec, w.box, ord, w.st, persistent);
@@ -1751,13 +2029,17 @@ static cudaError_t launch_raster_bwd_tiles(const WsPtrs& w, const Desc& h, const
   }
 }
 
-// The per-tile kernel, then the long-list kernel for the tiles it skipped.
+// The long lists, then the per-tile kernel.
 cudaError_t launch_raster_fwd(const Layout&, const WsPtrs& w, const Desc& h, const uint32_t* pv, int batch,
                               int group, int persistent, cudaStream_t s) {
-  cudaError_t e = launch_raster_fwd_tiles(w, h, pv, batch, group, persistent, s);
-  if (e != cudaSuccess) return e;
-  return launch_long(true, w, pv, s);
+  if (may_be_long(h)) {
+    const cudaError_t e = launch_fwd_long(w, h, pv, s, false, nullptr);
+    if (e != cudaSuccess) return e;
+  }
+  return launch_raster_fwd_tiles(w, h, pv, batch, group, persistent, s);
 }
+
+int raster_fwd_kernel_count(const Desc& h) { return may_be_long(h) ? 3 : 1; }
 
 // Chunked backward: as many resident CTAs as fit, warps claim (chunk, pixel
 // block) items from the queues k_bwd_prep built until none are left.
@@ -1767,21 +2049,25 @@ static cudaError_t launch_raster_bwd_chunks(const WsPtrs& w, const uint32_t* pv,
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bwd_c, kBwdChunkCta, 0);
   return launch_dep(k_bwd_c, dim3(sms * (per_sm > 0 ? per_sm : 1)), dim3(kBwdChunkCta), 0, s, w.desc, w.ranges, pv,
-                    w.rec, w.box, w.g13, w.cbase, w.ckpt, w.cmask, w.csuf, w.bq, w.bq_cap0, w.bq_capk, w.st);
+                    w.rec, w.box, w.g13, w.cbase, w.ckpt, w.cmask, seg_buf(w), w.ssuf, w.bq, w.bq_cap0, w.bq_capk,
+                    w.st);
 }
 
-// The shared-memory forward with the image-loss epilogue (and the long-list
-// forward with the same epilogue).  Follows launch_loss_counts on the same
-// stream, which zeroed the tile counter.
+// The shared-memory forward with the image-loss epilogue.  Follows
+// launch_loss_counts on the same stream, which zeroed the tile counter.
 cudaError_t launch_raster_fwd_loss(const WsPtrs& w, const Desc& h, const uint32_t* pv, int persistent,
                                    const lgs_loss_params& p, float* loss_out, cudaStream_t s) {
   LossEpi loss{p, loss_counts_ptr(w), reinterpret_cast<unsigned long long*>(w.loss_part), loss_out};
   const int grid = persistent ? persistent_grid(h.th * h.tw) : static_cast<int>(h.n_tiles);
-  // (follows k_loss_count on the stream: dispatched while it runs)
-  cudaError_t e = launch_dep(k_fwd_s<true>, dim3(grid), dim3(h.th * h.tw), 0, s, w.desc, w.ranges, pv, w.rec, w.box,
-                             persistent ? w.work : nullptr, w.st, persistent, w.cbase, w.ckpt, w.cmask, w.bwm, loss);
-  if (e != cudaSuccess) return e;
-  return launch_long(true, w, pv, s, &loss);
+  // (each follows a kernel of this call, k_loss_count first: dispatched while
+  // it runs)
+  if (may_be_long(h)) {
+    const cudaError_t e = launch_fwd_long(w, h, pv, s, true, &loss);
+    if (e != cudaSuccess) return e;
+  }
+  return launch_dep(block48(h) ? k_fwd_s<true, true> : k_fwd_s<true, false>, dim3(grid), dim3(h.th * h.tw), 0, s, w.desc,
+                    w.ranges, pv, w.rec, w.box, persistent ? w.work : nullptr, w.st, persistent, w.cbase, w.ckpt,
+                    w.cmask, w.bwm, loss);
 }
 
 cudaError_t launch_raster_bwd(const Layout&, const WsPtrs& w, const Desc& h, const uint32_t* pv, int batch,
@@ -1793,15 +2079,15 @@ cudaError_t launch_raster_bwd(const Layout&, const WsPtrs& w, const Desc& h, con
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    k_bwd_prep<<<4 * sms, 256, 0, s>>>(w.desc, w.ranges, w.longt, w.st, w.cbase, w.bwm, w.bq, w.bq_cap0, w.bq_capk,
-                                       w.ckpt, w.csuf);
+    k_bwd_prep<<<4 * sms, 256, 0, s>>>(w.desc, w.ranges, w.st, w.cbase, w.bwm, w.bq, w.bq_cap0, w.bq_capk,
+                                       seg_buf(w), w.ssuf);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return launch_raster_bwd_chunks(w, pv, s);
   }
   cudaError_t e = launch_raster_bwd_tiles(w, h, pv, batch, group, persistent, s);
   if (e != cudaSuccess) return e;
-  return launch_long(false, w, pv, s);
+  return launch_bwd_long(w, pv, s);
 }
 
 }  // namespace lgs
