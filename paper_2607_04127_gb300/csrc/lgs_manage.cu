@@ -32,6 +32,7 @@
 // split cap select, weights, output scan, write.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 
 #include "lgs_internal.cuh"
@@ -262,6 +263,8 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* s
 
 __global__ void __launch_bounds__(kScanCta) k_scan_blocks(const uint32_t* in, uint32_t* out, uint32_t len,
                                                           uint32_t* __restrict__ part) {
+  pdl_wait();               // (launched after a kernel of this chain: wait for it)
+  pdl_launch_dependents();  // the next kernel may be dispatched now
   __shared__ uint32_t s_warp[32];
   const uint64_t base = static_cast<uint64_t>(blockIdx.x) * kScanBlock + static_cast<uint64_t>(threadIdx.x) * kScanItems;
   uint32_t v[kScanItems], sum = 0;
@@ -282,6 +285,8 @@ __global__ void __launch_bounds__(kScanCta) k_scan_blocks(const uint32_t* in, ui
 
 __global__ void __launch_bounds__(kScanCta) k_scan_top(uint32_t* __restrict__ part, uint32_t nb,
                                                        uint32_t* __restrict__ out, uint32_t len) {
+  pdl_wait();               // (launched after a kernel of this chain: wait for it)
+  pdl_launch_dependents();  // the next kernel may be dispatched now
   __shared__ uint32_t s_warp[32];
   uint32_t carry = 0;
   for (uint32_t b0 = 0; b0 < nb; b0 += kScanCta) {
@@ -297,17 +302,22 @@ __global__ void __launch_bounds__(kScanCta) k_scan_top(uint32_t* __restrict__ pa
 
 __global__ void __launch_bounds__(kScanCta) k_scan_add(uint32_t* __restrict__ out, uint32_t len,
                                                        const uint32_t* __restrict__ part) {
+  pdl_wait();               // (launched after a kernel of this chain: wait for it)
+  pdl_launch_dependents();  // the next kernel may be dispatched now
   const uint32_t add = part[blockIdx.x];
   const uint64_t base = static_cast<uint64_t>(blockIdx.x) * kScanBlock;
   for (uint32_t j = threadIdx.x; j < kScanBlock; j += kScanCta)
     if (base + j < len) out[base + j] += add;
 }
 
-void launch_scan(const uint32_t* in, uint32_t* out, uint32_t len, uint32_t* part, cudaStream_t s) {
+// (each launch follows a kernel of the call: dispatched while it runs)
+cudaError_t launch_scan(const uint32_t* in, uint32_t* out, uint32_t len, uint32_t* part, cudaStream_t s) {
   const uint32_t nb = scan_blocks(len);
-  if (nb) k_scan_blocks<<<nb, kScanCta, 0, s>>>(in, out, len, part);
-  k_scan_top<<<1, kScanCta, 0, s>>>(part, nb, out, len);
-  if (nb) k_scan_add<<<nb, kScanCta, 0, s>>>(out, len, part);
+  cudaError_t e = cudaSuccess;
+  if (nb) e = launch_dep(k_scan_blocks, dim3(nb), dim3(kScanCta), 0, s, in, out, len, part);
+  if (e == cudaSuccess) e = launch_dep(k_scan_top, dim3(1), dim3(kScanCta), 0, s, part, nb, out, len);
+  if (e == cudaSuccess && nb) e = launch_dep(k_scan_add, dim3(nb), dim3(kScanCta), 0, s, out, len, part);
+  return e;
 }
 
 // ---------------------------------------------------------------------------
@@ -375,11 +385,35 @@ __global__ void __launch_bounds__(kMgCta) k_sel_digit(const unsigned long long* 
                                                       Sel* __restrict__ sel, unsigned long long* cbuf0,
                                                       unsigned long long* cbuf1, int d, int last, int shift,
                                                       int width, int mode, float q) {
+  pdl_wait();               // (launched after a kernel of this chain: wait for it)
+  pdl_launch_dependents();  // the next kernel may be dispatched now
   __shared__ uint32_t h[kBins];
   __shared__ uint32_t s_warp[32];
   __shared__ uint32_t s_kind, s_k, s_base, s_last;
   __shared__ unsigned long long s_pre;
   __shared__ unsigned long long s_stage[kMgCta / 32][kStage];
+  // the CTAs that take part: as many as the keys to read need (digits from the
+  // third on read what the one before left, usually a few hundred keys; a CTA
+  // without any would only add to the ticket)
+  constexpr int kUnroll = 8;
+  const uint32_t len = d >= 2 ? sel->ccount[(d - 2) & 1] : n;
+  const uint32_t parts = max(1u, min(gridDim.x, (len + kMgCta * kUnroll - 1) / (kMgCta * kUnroll)));
+  if (blockIdx.x >= parts) return;
+  // digit d >= 2 reads the buffer digit d - 1 wrote; digit d >= 1 writes the
+  // other one (unless it is the last digit).  kUnroll keys per thread per round
+  // in flight, the first round's loads ahead of the set-up: the digit is bound
+  // by latency (1M keys, a quantile's three digits: 35 us with 4 keys per round
+  // and every CTA on the ticket, now 31; 16 keys per round measured slower)
+  const unsigned long long* src = d >= 2 ? (((d - 2) & 1) ? cbuf1 : cbuf0) : key;
+  unsigned long long kk[kUnroll];
+  const auto fetch = [&](uint32_t i0) {
+#pragma unroll
+    for (int u = 0; u < kUnroll; ++u) {
+      const uint32_t i = i0 + u * blockDim.x + threadIdx.x;
+      kk[u] = i < len ? src[i] : kNoKey;
+    }
+  };
+  fetch(blockIdx.x * blockDim.x * kUnroll);
   if (threadIdx.x == 0) {
     if (mode != kSetupNone) {
       sel_setup(sel, mode, q, s_kind, s_k, s_base);
@@ -394,14 +428,6 @@ __global__ void __launch_bounds__(kMgCta) k_sel_digit(const unsigned long long* 
   __syncthreads();
   const bool active = s_kind == kSelKth;
   if (active) {
-    // digit d >= 2 reads the buffer digit d - 1 wrote; digit d >= 1 writes
-    // the other one (unless it is the last digit)
-    const unsigned long long* src = key;
-    uint32_t len = n;
-    if (d >= 2) {
-      src = ((d - 2) & 1) ? cbuf1 : cbuf0;
-      len = sel->ccount[(d - 2) & 1];
-    }
     unsigned long long* dst = ((d - 1) & 1) ? cbuf1 : cbuf0;
     uint32_t* dcount = &sel->ccount[(d - 1) & 1];
     const bool compact = d >= 1 && !last;
@@ -411,19 +437,12 @@ __global__ void __launch_bounds__(kMgCta) k_sel_digit(const unsigned long long* 
     const unsigned long long hi = shift + width >= 64 ? 0ull : (~0ull << (shift + width));
     const uint32_t dmask = (1u << width) - 1u;
     const int lane = threadIdx.x & 31;
-    // kUnroll keys per thread per round, loaded before use (the loop is
-    // latency-bound otherwise); warp-uniform rounds
-    constexpr int kUnroll = 4;
-    const uint32_t step = gridDim.x * blockDim.x * kUnroll;
+    // warp-uniform rounds
+    const uint32_t step = parts * blockDim.x * kUnroll;
     for (uint32_t i0 = blockIdx.x * blockDim.x * kUnroll; i0 < len; i0 += step) {
-      unsigned long long kk[kUnroll];
 #pragma unroll
       for (int u = 0; u < kUnroll; ++u) {
-        const uint32_t i = i0 + u * blockDim.x + threadIdx.x;
-        kk[u] = i < len ? src[i] : kNoKey;
-      }
-#pragma unroll
-      for (int u = 0; u < kUnroll; ++u) {
+        if (i0 + u * blockDim.x >= len) break;   // (uniform)
         const unsigned long long k = kk[u];
         const uint32_t bin =
             (k != kNoKey && !((k ^ pre) & hi)) ? (static_cast<uint32_t>(k >> shift) & dmask) : kBins;
@@ -446,21 +465,25 @@ __global__ void __launch_bounds__(kMgCta) k_sel_digit(const unsigned long long* 
           }
         }
       }
+      if (i0 + step < len) fetch(i0 + step);
     }
     if (compact && sc) {
       __syncwarp();
       flush_stage(stage, sc, dst, dcount, lane);
     }
     __syncthreads();
-    for (uint32_t t = threadIdx.x; t < kBins; t += blockDim.x)
-      if (h[t]) atomicAdd(&sel->hist[t], h[t]);
+    if (parts > 1)
+      for (uint32_t t = threadIdx.x; t < kBins; t += blockDim.x)
+        if (h[t]) atomicAdd(&sel->hist[t], h[t]);
   }
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(&sel->ticket, 1u) == gridDim.x - 1 ? 1u : 0u;
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
+  if (parts > 1) {
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&sel->ticket, 1u) == parts - 1 ? 1u : 0u;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+  }
   if (threadIdx.x == 0) {
     sel->ticket = 0;
     sel->ccount[d & 1] = 0;   // the buffer digit d + 1 writes (digit d read it, or nobody did)
@@ -475,21 +498,21 @@ __global__ void __launch_bounds__(kMgCta) k_sel_digit(const unsigned long long* 
   if (!active) return;
   // pick: each of the 256 threads owns 8 consecutive bins
   constexpr int kPer = kBins / kMgCta;
-  volatile uint32_t* vh = sel->hist;
+  volatile uint32_t* vh = parts > 1 ? sel->hist : h;
   uint32_t v[kPer], sum = 0;
 #pragma unroll
   for (int j = 0; j < kPer; ++j) {
     v[j] = vh[threadIdx.x * kPer + j];
     sum += v[j];
   }
-  const uint32_t kk = s_k;
+  const uint32_t rank = s_k;
   uint32_t total;
   uint32_t ex = block_exclusive_scan(sum, s_warp, total);
 #pragma unroll
   for (int j = 0; j < kPer; ++j) {
-    if (ex <= kk && kk < ex + v[j]) {
+    if (ex <= rank && rank < ex + v[j]) {
       sel->prefix = s_pre | (static_cast<unsigned long long>(threadIdx.x * kPer + j) << shift);
-      sel->k = kk - ex;
+      sel->k = rank - ex;
     }
     ex += v[j];
     vh[threadIdx.x * kPer + j] = 0u;
@@ -497,11 +520,13 @@ __global__ void __launch_bounds__(kMgCta) k_sel_digit(const unsigned long long* 
 }
 
 template <int D>
-void launch_select(const unsigned long long* key, uint32_t n, Sel* sel, unsigned long long* const (&cbuf)[2],
+cudaError_t launch_select(const unsigned long long* key, uint32_t n, Sel* sel, unsigned long long* const (&cbuf)[2],
                    const Digit (&digits)[D], int mode, float q, int grid, cudaStream_t s) {
-  for (int d = 0; d < D; ++d)
-    k_sel_digit<<<grid, kMgCta, 0, s>>>(key, n, sel, cbuf[0], cbuf[1], d, d == D - 1 ? 1 : 0, digits[d].shift,
-                                        digits[d].width, d == 0 ? mode : kSetupNone, q);
+  cudaError_t e = cudaSuccess;
+  for (int d = 0; d < D && e == cudaSuccess; ++d)
+    e = launch_dep(k_sel_digit, dim3(grid), dim3(kMgCta), 0, s, key, n, sel, cbuf[0], cbuf[1], d, d == D - 1 ? 1 : 0,
+                   digits[d].shift, digits[d].width, d == 0 ? mode : static_cast<int>(kSetupNone), q);
+  return e;
 }
 
 // selected if the select takes every key, or the key is at most the k-th
@@ -516,6 +541,7 @@ __device__ __forceinline__ bool sel_takes(uint32_t kind, unsigned long long pref
 __global__ void __launch_bounds__(kMgCta) k_mg_res_keys(const float* __restrict__ res, uint32_t n,
                                                         unsigned long long* __restrict__ key, Sel* __restrict__ sel,
                                                         int64_t* __restrict__ counts) {
+  pdl_launch_dependents();  // the next kernel may be dispatched now
   if (blockIdx.x == 0) {
     for (uint32_t t = threadIdx.x; t < kBins; t += blockDim.x) sel->hist[t] = 0;
     if (threadIdx.x == 0) {
@@ -555,6 +581,8 @@ __global__ void __launch_bounds__(kMgCta) k_mg_score(const float* __restrict__ l
                                                      const float* __restrict__ logit, uint32_t n, MgParams P,
                                                      float* __restrict__ score, MgScratch S,
                                                      int64_t* __restrict__ counts) {
+  pdl_wait();               // (launched after a kernel of this chain: wait for it)
+  pdl_launch_dependents();  // the next kernel may be dispatched now
   const float rq = okey_inv(static_cast<uint32_t>(S.sel->prefix >> 32));
   const uint32_t stride = gridDim.x * blockDim.x;
   uint32_t n_dead = 0, n_alive = 0;
@@ -597,6 +625,8 @@ __global__ void __launch_bounds__(kMgCta) k_mg_insert(const float* __restrict__ 
                                                       const float* __restrict__ score, uint32_t n,
                                                       const Sel* __restrict__ sel, MgParams P, int ax, int bx,
                                                       MgScratch S) {
+  pdl_wait();               // (launched after a kernel of this chain: wait for it)
+  pdl_launch_dependents();  // the next kernel may be dispatched now
   const bool any = sel->kind != kSelNone;
   const float qp = __uint_as_float(static_cast<uint32_t>(sel->prefix >> 32));
   const uint32_t mask = S.T - 1;
@@ -648,6 +678,8 @@ __global__ void __launch_bounds__(kMgCta) k_mg_insert(const float* __restrict__ 
 __global__ void __launch_bounds__(kMgCta) k_mg_measure(const float* __restrict__ mean, const float* __restrict__ quat,
                                                        const float* __restrict__ log_scale, uint32_t n, MgParams P,
                                                        MgScratch S) {
+  pdl_wait();               // (launched after a kernel of this chain: wait for it)
+  pdl_launch_dependents();  // the next kernel may be dispatched now
   const int lane = threadIdx.x & 31;
   for (uint32_t i0 = blockIdx.x * blockDim.x; i0 < n; i0 += gridDim.x * blockDim.x) {
     const uint32_t i = i0 + threadIdx.x;
@@ -676,6 +708,8 @@ __global__ void __launch_bounds__(kMgCta) k_mg_measure(const float* __restrict__
 }
 
 __global__ void __launch_bounds__(kMgCta) k_mg_scatter(uint32_t n, MgScratch S) {
+  pdl_wait();               // (launched after a kernel of this chain: wait for it)
+  pdl_launch_dependents();  // the next kernel may be dispatched now
   const int lane = threadIdx.x & 31;
   for (uint32_t i0 = blockIdx.x * blockDim.x; i0 < n; i0 += gridDim.x * blockDim.x) {
     const uint32_t i = i0 + threadIdx.x;
@@ -711,6 +745,8 @@ __device__ __forceinline__ void cover(const float* __restrict__ score, const MgS
 // radii in shared memory and each member counts the strictly smaller ones
 // (fewer than k: covered).
 __global__ void __launch_bounds__(kMgCta) k_mg_decide(const float* __restrict__ score, MgParams P, MgScratch S) {
+  pdl_wait();               // (launched after a kernel of this chain: wait for it)
+  pdl_launch_dependents();  // the next kernel may be dispatched now
   __shared__ uint32_t h[kBins];
   __shared__ uint32_t s_warp[32];
   __shared__ uint32_t s_pre, s_k, s_cov;
@@ -822,6 +858,8 @@ __global__ void __launch_bounds__(kMgCta) k_mg_decide(const float* __restrict__ 
 // keys for the next quantile (counted into the select) and clears the table.
 __global__ void __launch_bounds__(kMgCta) k_mg_apply_prune(const float* __restrict__ score, uint32_t n, MgScratch S,
                                                            int64_t* __restrict__ removed) {
+  pdl_wait();               // (launched after a kernel of this chain: wait for it)
+  pdl_launch_dependents();  // the next kernel may be dispatched now
   const uint32_t kind = S.sel->kind;
   const unsigned long long prefix = S.sel->prefix;
   const uint32_t stride = gridDim.x * blockDim.x;
@@ -853,6 +891,8 @@ __global__ void __launch_bounds__(kMgCta) k_mg_apply_prune(const float* __restri
 __global__ void __launch_bounds__(kMgCta) k_mg_split_keys(const float* __restrict__ logit,
                                                           const float* __restrict__ score, uint32_t n, MgParams P,
                                                           MgScratch S) {
+  pdl_wait();               // (launched after a kernel of this chain: wait for it)
+  pdl_launch_dependents();  // the next kernel may be dispatched now
   const bool any = S.sel->kind != kSelNone;
   const float qs = __uint_as_float(static_cast<uint32_t>(S.sel->prefix >> 32));
   const uint32_t stride = gridDim.x * blockDim.x;
@@ -871,6 +911,8 @@ __global__ void __launch_bounds__(kMgCta) k_mg_split_keys(const float* __restric
 }
 
 __global__ void __launch_bounds__(kMgCta) k_mg_weights(uint32_t n, MgScratch S) {
+  pdl_wait();               // (launched after a kernel of this chain: wait for it)
+  pdl_launch_dependents();  // the next kernel may be dispatched now
   const uint32_t kind = S.sel->kind;
   const unsigned long long prefix = S.sel->prefix;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -891,6 +933,8 @@ __global__ void __launch_bounds__(kMgCta) k_mg_write(const float* __restrict__ m
                                                      MgScratch S, lgs_surfel_params_out out, int64_t capacity,
                                                      int32_t* __restrict__ src, uint8_t* __restrict__ role,
                                                      int64_t* __restrict__ counts) {
+  pdl_wait();               // (launched after a kernel of this chain: wait for it)
+  pdl_launch_dependents();  // the next kernel may be dispatched now
   const uint32_t stride = gridDim.x * blockDim.x;
   uint32_t n_split = 0;
   if (blockIdx.x == 0 && threadIdx.x == 0) counts[0] = S.pos[n];
@@ -938,17 +982,40 @@ __global__ void __launch_bounds__(kMgCta) k_mg_write(const float* __restrict__ m
   block_count64(n_split, &counts[5]);
 }
 
+// One CTA carries `per` rows at a time, V 32-bit words per load where the
+// rows allow it (words a multiple of V, both arrays aligned): HBM-bound.  The
+// row of a word needs a division, of 32 bits here (of 64 bits, over the whole
+// array, it bound the kernel: 1M rows of 10 words 45 us, now 23).
+constexpr int64_t kGatherRows = 128;
+template <class V>
 __global__ void __launch_bounds__(kMgCta) k_mg_gather(const int32_t* __restrict__ src, const uint8_t* __restrict__ role,
                                                       const int64_t* __restrict__ counts, int64_t capacity,
-                                                      const uint32_t* __restrict__ in, uint32_t* __restrict__ out,
-                                                      int words, int zero_children) {
+                                                      const V* __restrict__ in, V* __restrict__ out, uint32_t words,
+                                                      int64_t per, int zero_children) {
   const int64_t n_out = counts[0] < capacity ? counts[0] : capacity;
-  const int64_t total = n_out * words;
-  for (int64_t j = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; j < total;
-       j += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int64_t row = j / words;
-    const int w = static_cast<int>(j - row * words);
-    out[j] = (zero_children && role[row]) ? 0u : in[static_cast<int64_t>(src[row]) * words + w];
+  for (int64_t r0 = blockIdx.x * per; r0 < n_out; r0 += gridDim.x * per) {
+    const uint32_t rows = static_cast<uint32_t>(n_out - r0 < per ? n_out - r0 : per);
+    const uint32_t total = rows * words;
+    for (uint32_t e0 = threadIdx.x; e0 < total; e0 += 4 * kMgCta) {
+      // four words per round: their rows, then the words
+      int64_t from[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const uint32_t e = e0 + u * kMgCta;
+        from[u] = -1;
+        if (e < total) {
+          const uint32_t row = e / words;
+          const int32_t p = src[r0 + row];
+          if (!(zero_children && role[r0 + row])) from[u] = static_cast<int64_t>(p) * words + (e - row * words);
+        }
+      }
+      V v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) v[u] = from[u] >= 0 ? in[from[u]] : V{};
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (e0 + u * kMgCta < total) out[r0 * words + e0 + u * kMgCta] = v[u];
+    }
   }
 }
 
@@ -984,7 +1051,7 @@ cudaError_t launch_manage(const lgs_surfels& M, const float* lam, const float* r
   const int sms = sm_count();
   const int g = grid_for(n, sms);
   const int gc = grid_for(n > S.T ? n : S.T, sms);   // kernels that also clear the table
-  const int gs = grid_for(n, sms) < 2 * sms ? grid_for(n, sms) : 2 * sms;   // select digits
+  const int gs = grid_for(n, sms) < 4 * sms ? grid_for(n, sms) : 4 * sms;   // select digits
   MgParams P;
   P.logit_prune = H.logit_prune;
   P.logit_min = H.logit_min;
@@ -1004,34 +1071,53 @@ cudaError_t launch_manage(const lgs_surfels& M, const float* lam, const float* r
   P.split_dlog = H.p.split_dlog;
   static const int planes[3][2] = {{0, 1}, {1, 2}, {2, 0}};
 
+  // every launch after the first follows a kernel of this call: dispatched
+  // while it runs (the step is a chain of 71 short launches)
   k_mg_res_keys<<<g, kMgCta, 0, s>>>(res, n, S.key, S.sel, counts);
-  launch_select(S.key, n, S.sel, S.cbuf, kDigits32, kSetupQuantile, P.q_res, gs, s);
-  k_mg_score<<<gc, kMgCta, 0, s>>>(lam, res, M.opacity_logit, n, P, score, S, counts);
+  cudaError_t e = cudaGetLastError();
+  const dim3 cta(kMgCta);
+  const auto then = [&](auto launch) {
+    if (e == cudaSuccess) e = launch();
+  };
+  then([&] { return launch_select(S.key, n, S.sel, S.cbuf, kDigits32, kSetupQuantile, P.q_res, gs, s); });
+  then([&] { return launch_dep(k_mg_score, dim3(gc), cta, 0, s, lam, res, M.opacity_logit, n, P, score, S, counts); });
   for (int p = 0; p < H.p.n_passes; ++p) {
-    launch_select(S.key, n, S.sel, S.cbuf, kDigits32, kSetupQuantile, P.q_plane, gs, s);
-    k_mg_insert<<<g, kMgCta, 0, s>>>(M.mean, M.opacity_logit, score, n, S.sel, P, planes[p][0], planes[p][1], S);
-    k_mg_measure<<<g, kMgCta, 0, s>>>(M.mean, M.quat, M.log_scale, n, P, S);
-    launch_scan(S.cnt, S.off, S.T, S.part, s);
-    k_mg_scatter<<<g, kMgCta, 0, s>>>(n, S);
-    k_mg_decide<<<sms * 4, kMgCta, 0, s>>>(score, P, S);
-    launch_select(S.key, n, S.sel, S.cbuf, kDigits64, kSetupCap, P.prune_cap, gs, s);
-    k_mg_apply_prune<<<gc, kMgCta, 0, s>>>(score, n, S, counts + 2 + p);
+    then([&] { return launch_select(S.key, n, S.sel, S.cbuf, kDigits32, kSetupQuantile, P.q_plane, gs, s); });
+    then([&] {
+      return launch_dep(k_mg_insert, dim3(g), cta, 0, s, M.mean, M.opacity_logit, score, n, S.sel, P, planes[p][0],
+                        planes[p][1], S);
+    });
+    then([&] { return launch_dep(k_mg_measure, dim3(g), cta, 0, s, M.mean, M.quat, M.log_scale, n, P, S); });
+    then([&] { return launch_scan(S.cnt, S.off, S.T, S.part, s); });
+    then([&] { return launch_dep(k_mg_scatter, dim3(g), cta, 0, s, n, S); });
+    then([&] { return launch_dep(k_mg_decide, dim3(sms * 4), cta, 0, s, score, P, S); });
+    then([&] { return launch_select(S.key, n, S.sel, S.cbuf, kDigits64, kSetupCap, P.prune_cap, gs, s); });
+    then([&] { return launch_dep(k_mg_apply_prune, dim3(gc), cta, 0, s, score, n, S, counts + 2 + p); });
   }
-  launch_select(S.key, n, S.sel, S.cbuf, kDigits32, kSetupQuantile, P.q_split, gs, s);
-  k_mg_split_keys<<<g, kMgCta, 0, s>>>(M.opacity_logit, score, n, P, S);
-  launch_select(S.key, n, S.sel, S.cbuf, kDigits64, kSetupCap, P.split_cap, gs, s);
-  k_mg_weights<<<g, kMgCta, 0, s>>>(n, S);
-  launch_scan(S.pos, S.pos, n, S.part, s);
-  k_mg_write<<<g, kMgCta, 0, s>>>(M.mean, M.quat, M.log_scale, M.opacity_logit, n, P, S, out, capacity, src, role,
-                                  counts);
-  return cudaGetLastError();
+  then([&] { return launch_select(S.key, n, S.sel, S.cbuf, kDigits32, kSetupQuantile, P.q_split, gs, s); });
+  then([&] { return launch_dep(k_mg_split_keys, dim3(g), cta, 0, s, M.opacity_logit, score, n, P, S); });
+  then([&] { return launch_select(S.key, n, S.sel, S.cbuf, kDigits64, kSetupCap, P.split_cap, gs, s); });
+  then([&] { return launch_dep(k_mg_weights, dim3(g), cta, 0, s, n, S); });
+  then([&] { return launch_scan(S.pos, S.pos, n, S.part, s); });
+  then([&] {
+    return launch_dep(k_mg_write, dim3(g), cta, 0, s, M.mean, M.quat, M.log_scale, M.opacity_logit, n, P, S, out,
+                      capacity, src, role, counts);
+  });
+  return e;
 }
 
 cudaError_t launch_manage_gather(const int32_t* src, const uint8_t* role, const int64_t* counts, int64_t capacity,
                                  const void* in, void* out, int words, int zero_children, cudaStream_t s) {
-  const int g = grid_for(static_cast<uint64_t>(capacity) * static_cast<uint64_t>(words), sm_count());
-  k_mg_gather<<<g, kMgCta, 0, s>>>(src, role, counts, capacity, static_cast<const uint32_t*>(in),
-                                   static_cast<uint32_t*>(out), words, zero_children);
+  // (the words of a CTA's rows are counted in 32 bits)
+  const int64_t per = words <= (1 << 24) ? kGatherRows : 1;
+  const int g = static_cast<int>(std::min<int64_t>((capacity + per - 1) / per, 16 * sm_count()));
+  const uintptr_t at = reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out);
+  const auto run = [&](auto* i, auto* o, int w) {
+    k_mg_gather<<<g, kMgCta, 0, s>>>(src, role, counts, capacity, i, o, static_cast<uint32_t>(w), per, zero_children);
+  };
+  if (words % 4 == 0 && at % 16 == 0) run(static_cast<const uint4*>(in), static_cast<uint4*>(out), words / 4);
+  else if (words % 2 == 0 && at % 8 == 0) run(static_cast<const uint2*>(in), static_cast<uint2*>(out), words / 2);
+  else run(static_cast<const uint32_t*>(in), static_cast<uint32_t*>(out), words);
   return cudaGetLastError();
 }
 
