@@ -442,24 +442,57 @@ struct AdamSeg {
   float lr[4];
 };
 
+__device__ __forceinline__ void adam_one(float& p, float& g, float& m, float& v, float lr, float b1, float b2,
+                                         float eps, float c1, float c2) {
+  m = b1 * m + (1.f - b1) * g;
+  v = b2 * v + (1.f - b2) * g * g;
+  p -= lr * (m * c1) / (sqrtf(v * c2) + eps);
+}
+
+// n scalars of one parameter group by the x dimension of the grid.  HBM-bound:
+// 28 B a scalar, 32 with the gradient zeroed (1M surfels, 10 M scalars: 47 us
+// at the measured copy rate).  128 consecutive scalars per warp and round, four
+// coalesced ones per lane, so 16 loads in flight: 67.7 us with one scalar per
+// thread, now 51.2 (float4 loads, which an odd group's moments do not allow,
+// measured the same; streaming cache hints 56).
+__device__ __forceinline__ void adam_group(float* __restrict__ p, float* __restrict__ g, float* __restrict__ m,
+                                           float* __restrict__ v, int64_t n, float lr, float b1, float b2, float eps,
+                                           float c1, float c2, int zero_grad) {
+  const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  const int64_t step = 4 * static_cast<int64_t>(gridDim.x) * blockDim.x;
+  for (int64_t i = (t & ~31ll) * 4 + (t & 31); i < n; i += step) {
+    float P[4], G[4], Mo[4], V[4];
+    const int k = static_cast<int>(n - i < 97 ? (n - i + 31) / 32 : 4);   // scalars of this lane
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (u < k) {
+        P[u] = p[i + 32 * u];
+        G[u] = g[i + 32 * u];
+        Mo[u] = m[i + 32 * u];
+        V[u] = v[i + 32 * u];
+      }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (u < k) {
+        adam_one(P[u], G[u], Mo[u], V[u], lr, b1, b2, eps, c1, c2);
+        p[i + 32 * u] = P[u];
+        m[i + 32 * u] = Mo[u];
+        v[i + 32 * u] = V[u];
+        if (zero_grad) g[i + 32 * u] = 0.f;
+      }
+  }
+}
+
+// CTAs per parameter group of n scalars: 1,024 scalars each, at most eight CTAs
+// per SM
+static unsigned adam_ctas(int64_t n) {
+  return static_cast<unsigned>(std::min<int64_t>(std::max<int64_t>((n + 1023) / 1024, 1), 8 * 152));
+}
+
 __global__ void __launch_bounds__(256) k_adam(AdamSeg a, float b1, float b2, float eps, float c1, float c2,
                                                int zero_grad) {
   const int sgm = blockIdx.y;
-  float* __restrict__ p = a.p[sgm];
-  float* __restrict__ g = a.g[sgm];
-  float* __restrict__ m = a.m[sgm];
-  float* __restrict__ v = a.v[sgm];
-  const float lr = a.lr[sgm];
-  for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < a.n[sgm];
-       i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.f - b1) * gi;
-    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    p[i] -= lr * (mi * c1) / (sqrtf(vi * c2) + eps);
-    if (zero_grad) g[i] = 0.f;
-  }
+  adam_group(a.p[sgm], a.g[sgm], a.m[sgm], a.v[sgm], a.n[sgm], a.lr[sgm], b1, b2, eps, c1, c2, zero_grad);
 }
 
 cudaError_t launch_adam(float* p[4], float* g[4], float* m[4], float* v[4], const int64_t cnt[4], int64_t step,
@@ -472,10 +505,8 @@ cudaError_t launch_adam(float* p[4], float* g[4], float* m[4], float* v[4], cons
   }
   const double c1 = 1.0 / (1.0 - pow(static_cast<double>(b1), static_cast<double>(step)));
   const double c2 = 1.0 / (1.0 - pow(static_cast<double>(b2), static_cast<double>(step)));
-  int64_t blocks = (mx + 255) / 256;
-  if (blocks > 4096) blocks = 4096;
-  k_adam<<<dim3(static_cast<unsigned>(blocks), 4), 256, 0, s>>>(a, b1, b2, eps, static_cast<float>(c1),
-                                                                 static_cast<float>(c2), zero_grad);
+  k_adam<<<dim3(adam_ctas(mx), 4), 256, 0, s>>>(a, b1, b2, eps, static_cast<float>(c1), static_cast<float>(c2),
+                                                zero_grad);
   return cudaGetLastError();
 }
 
@@ -494,21 +525,7 @@ struct AdamBatch {
 __global__ void __launch_bounds__(256) k_adam_batch(const __grid_constant__ AdamBatch a, float b1, float b2, float eps,
                                                     int zero_grad) {
   const int sgm = blockIdx.y, map = sgm >> 2;
-  float* __restrict__ p = a.p[sgm];
-  float* __restrict__ g = a.g[sgm];
-  float* __restrict__ m = a.m[sgm];
-  float* __restrict__ v = a.v[sgm];
-  const float lr = a.lr[sgm], c1 = a.c1[map], c2 = a.c2[map];
-  for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < a.n[sgm];
-       i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.f - b1) * gi;
-    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    p[i] -= lr * (mi * c1) / (sqrtf(vi * c2) + eps);
-    if (zero_grad) g[i] = 0.f;
-  }
+  adam_group(a.p[sgm], a.g[sgm], a.m[sgm], a.v[sgm], a.n[sgm], a.lr[sgm], b1, b2, eps, a.c1[map], a.c2[map], zero_grad);
 }
 
 cudaError_t launch_adam_batch(const lgs_adam_map* maps, int n_maps, float b1, float b2, float eps, int zero_grad,
@@ -534,9 +551,7 @@ cudaError_t launch_adam_batch(const lgs_adam_map* maps, int n_maps, float b1, fl
     a.c1[k] = static_cast<float>(1.0 / (1.0 - pow(static_cast<double>(b1), static_cast<double>(M.step))));
     a.c2[k] = static_cast<float>(1.0 / (1.0 - pow(static_cast<double>(b2), static_cast<double>(M.step))));
   }
-  int64_t blocks = (mx + 255) / 256;
-  if (blocks > 2048) blocks = 2048;
-  k_adam_batch<<<dim3(static_cast<unsigned>(blocks), 4 * n_maps), 256, 0, s>>>(a, b1, b2, eps, zero_grad);
+  k_adam_batch<<<dim3(adam_ctas(mx), 4 * n_maps), 256, 0, s>>>(a, b1, b2, eps, zero_grad);
   return cudaGetLastError();
 }
 
