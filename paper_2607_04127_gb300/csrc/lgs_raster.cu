@@ -1487,9 +1487,94 @@ __global__ void __launch_bounds__(kMaxTileThreads)
 // independent, so a frame offers several times more warps than pixel
 // blocks.
 // ---------------------------------------------------------------------------
-constexpr int kBwdChunkCta = 256;
+constexpr int kBwdChunkCta = 128;
 
-__global__ void __launch_bounds__(kBwdChunkCta)
+// A hit's 12 moments are summed over its pixels in two phases.  Phase A walks
+// the chunk's hits one by one, as every lane's recurrence of T and S needs; a
+// lane whose pixel composited the hit leaves its contribution (g, u, v, ct;
+// w sg gS) in the warp's next free slots of shared memory, and the hit takes
+// one lane for every kBwdPer of its contributions.  Phase B, once the lanes
+// or the slots are all taken, has every lane sum its own and add the moments
+// with three 16-byte reductions.  Contributions wait across chunks and tiles:
+// the sums need nothing of where they came from but the item.
+//
+// Bound by issue (about 70 % of the cycles) and the latency of the chunk's six
+// dependent reads.  Before, the 12 moments were summed over the warp with
+// shuffles hit by hit and added by 12 lanes with scalar atomics: 162
+// instructions a hit on the street frame (200k surfels, 128 x 1024), of whose
+// 32 lanes 8 held a contribution; now 120.  Kernel 131 -> 112 us; on 8 keyframes
+// of a dense 1M map (12 lanes of 32) 1195 -> 1166 us, on six batched maps
+// 733 -> 707 us; the steps 336 -> 315, 5945 -> 5890 and 4285 -> 4258 us.
+// Shares and slots, the three steps' gains: 4 and 96 6.6, 0.9, 0.6 %; 6 and 96
+// 5.1, 0.7, 0.2 %; 8 and 160 6.6, 0.8, -0.9 % (more shared memory leaves less
+// L1 to the batched maps' reads).  An item's three vectors leave by three
+// neighbouring lanes, as one request: by one lane after the other the
+// keyframes' kernel took 65 us more.  Others, street frame and keyframes: four
+// lanes per hit for 8 hits at a time 117 and 1190 us (the longest of the 8
+// decides), every lane walking its own pixel's bits 118 and 1279 us (its record
+// reads from shared memory conflict), two hits' evaluations at a time 130 and
+// 1687 us (128 registers), the next chunk claimed ahead 135 and 1162 us (a
+// street frame has four chunks per warp: the last ones no longer balance).
+constexpr uint32_t kBwdPer = 4;      // contributions a lane sums
+constexpr uint32_t kBwdSlots = 96;   // at least a hit's 32, and 32 lanes' sums
+
+struct BwdWarp {
+  WarpRecs rec;
+  float4 a[kBwdSlots];   // (g, u, v, ct)
+  float4 b[kBwdSlots];   // (w sg gS, 0)
+  uint32_t item[32];     // items of the staged hits
+  uint32_t who[kChunk];  // the chunk's hits, last first: the pixels that composited them
+  uint8_t entry[kChunk]; // and their entries of the chunk
+};
+
+// 16-byte aligned vector reduction into global memory.
+__device__ __forceinline__ void red_add4(float* p, float x, float y, float z, float w) {
+  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
+}
+
+// Phase B: the lane sums the contributions in its slots (first, first + step,
+// ... below end) and adds the 12 moments to its item.
+__device__ __forceinline__ void bwd_flush(BwdWarp& sb, int lane, uint32_t first, uint32_t end, uint32_t step, uint32_t item,
+                                          float* __restrict__ g13) {
+  __syncwarp();
+  float v[12];
+#pragma unroll
+  for (int q = 0; q < 12; ++q) v[q] = 0.f;
+  for (uint32_t i = first; i < end; i += step) {
+    const float4 a = sb.a[i], b = sb.b[i];
+    const float ug = a.y * a.x, vg = a.z * a.x;
+    v[0] += a.x;
+    v[1] += ug;
+    v[2] += vg;
+    v[3] = fmaf(a.y, ug, v[3]);
+    v[4] = fmaf(a.z, vg, v[4]);
+    v[5] = fmaf(a.y, vg, v[5]);
+    v[6] += a.w;
+    v[7] = fmaf(a.w, a.y, v[7]);
+    v[8] = fmaf(a.w, a.z, v[8]);
+    v[9] += b.x;
+    v[10] += b.y;
+    v[11] += b.z;
+  }
+  // an item's three vectors by neighbouring lanes, so that they leave as one request
+  static_assert(kBwdSlots >= 96, "32 lanes' sums");
+  __syncwarp();
+  sb.a[3 * lane] = make_float4(v[0], v[1], v[2], v[3]);
+  sb.a[3 * lane + 1] = make_float4(v[4], v[5], v[6], v[7]);
+  sb.a[3 * lane + 2] = make_float4(v[8], v[9], v[10], v[11]);
+  __syncwarp();
+  const uint32_t has = __ballot_sync(0xffffffffu, first < end);
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+    const int at = 32 * r + lane, src = at / 3;
+    const uint32_t it = __shfl_sync(0xffffffffu, item, src);
+    const float4 x = sb.a[at];
+    if ((has >> src) & 1u) red_add4(g13 + 16 * static_cast<int64_t>(it) + 4 * (at - 3 * src), x.x, x.y, x.z, x.w);
+  }
+  __syncwarp();
+}
+
+__global__ void __launch_bounds__(kBwdChunkCta, 7)
     k_bwd_c(const Desc* __restrict__ D, const uint2* __restrict__ ranges, const uint32_t* __restrict__ pv,
             const float4* __restrict__ rec, const float4* __restrict__ box, float* __restrict__ g13,
             const uint32_t* __restrict__ cbase, const float* __restrict__ ckpt, const uint32_t* __restrict__ cmask,
@@ -1497,11 +1582,13 @@ __global__ void __launch_bounds__(kBwdChunkCta)
             uint32_t bq_capk, Status* __restrict__ st) {
   pdl_wait();               // (launched after a kernel of this chain: wait for it)
   pdl_launch_dependents();  // the next kernel may be dispatched now
-  __shared__ WarpRecs s_w[kBwdChunkCta / 32];
-  __shared__ uint32_t s_item[kBwdChunkCta / 32][32];
+  __shared__ BwdWarp s_w[kBwdChunkCta / 32];
   const int lane = threadIdx.x & 31;
-  WarpRecs& sw = s_w[threadIdx.x >> 5];
-  uint32_t* si = s_item[threadIdx.x >> 5];
+  BwdWarp& sb = s_w[threadIdx.x >> 5];
+  WarpRecs& sw = sb.rec;
+  uint32_t* si = sb.item;
+  // contributions that wait for phase B: slots and lanes taken, the lane's share
+  uint32_t used = 0, lanes = 0, w_first = 0, w_end = 0, w_step = 1, w_item = 0;
   const int npx = D->th * D->tw, wpt = npx >> 5;
   // the forward's queues, claimed in class order: lane l < kBwdClasses holds
   // class l's size (clamped to its capacity) and the items before its end
@@ -1561,79 +1648,92 @@ __global__ void __launch_bounds__(kBwdChunkCta)
         S += gA * q[npx] + gSt * q[2 * npx] + gSx * q[3 * npx] + gSy * q[4 * npx] + gSz * q[5 * npx];
       }
     }
-    // entries [k_lo, k_hi) of the list, walked down in 32-entry steps: a
-    // step's hits are the entries some pixel of the warp composited (the
-    // forward's window masks), and a lane takes the ones its pixel did
+    // entries [k_lo, k_hi) of the list: the chunk's hits are the entries some
+    // pixel of the warp composited (the forward's window masks), listed last
+    // first with the pixels that did; their records are staged 32 hits at a time
     const uint32_t len = rg.y - rg.x;
     const int k_hi = static_cast<int>(min(min(static_cast<uint32_t>(k_lo) + kChunk, len),
                                           static_cast<uint32_t>(__reduce_max_sync(0xffffffffu, act ? nc : 0))));
-    for (int k0 = k_lo + ((k_hi - k_lo + 31) / 32 - 1) * 32; k0 >= k_lo; k0 -= 32) {
+    constexpr int kWin = kChunk / 32;
+    uint32_t word[kWin];
+    const int64_t cm = (static_cast<int64_t>(cbase[tile]) * 4 + static_cast<uint32_t>(k_lo) / 32) * npx + vt;
+#pragma unroll
+    for (int q = 0; q < kWin; ++q) {
       // entries below the pixel's n_contrib only (a long list's pixels stop
       // on their own, so their words past it are not this step's)
-      const int lim = nc - k0;
-      uint32_t word = 0u;
-      if (act && lim > 0) {
-        word = __ldg(cmask + (static_cast<int64_t>(cbase[tile]) * 4 + static_cast<uint32_t>(k0) / 32) * npx + vt);
-        if (lim < 32) word &= (1u << lim) - 1u;
-      }
-      uint32_t m = __reduce_or_sync(0xffffffffu, word);
+      const int lim = nc - k_lo - 32 * q;
+      word[q] = act && lim > 0 && k_lo + 32 * q < k_hi ? __ldg(cmask + cm + static_cast<int64_t>(q) * npx) : 0u;
+      if (lim < 32) word[q] &= lim > 0 ? (1u << lim) - 1u : 0u;
+    }
+    uint32_t hits = 0;
+    __syncwarp();   // (the item before no longer reads the list)
+#pragma unroll
+    for (int q = kWin - 1; q >= 0; --q) {
+      const uint32_t m = __reduce_or_sync(0xffffffffu, word[q]);
       if (!m) continue;
-      const bool hit = (m >> lane) & 1u;
-      const uint32_t item = hit ? __ldg(pv + rg.x + k0 + lane) : 0u;
+      const uint32_t px = warp_transpose(word[q], lane);
+      if ((m >> lane) & 1u) {
+        const uint32_t at = hits + static_cast<uint32_t>(__popc((m >> lane) >> 1));
+        sb.who[at] = px;
+        sb.entry[at] = static_cast<uint8_t>(32 * q + lane);
+      }
+      hits += static_cast<uint32_t>(__popc(m));
+    }
+    for (uint32_t b = 0; b < hits; b += 32) {
       __syncwarp();
-      if (hit) {
+      uint32_t my_who = 0;
+      if (b + lane < hits) {
+        my_who = sb.who[b + lane];
+        const uint32_t item = __ldg(pv + rg.x + k_lo + sb.entry[b + lane]);
         stage_hit(rec, item, sw, lane);
         si[lane] = item;
       }
       __syncwarp();
-      do {
-        const int bq = 31 - __clz(m);
-        m &= ~(1u << bq);
-        // the pixel composited this entry: its evaluation (the forward's,
-        // bit for bit) is valid
-        const bool valid = (word >> bq) & 1u;
-        const float4 r0 = sw.r0[bq];
-        Eval e;
-        eval_pair(r0, sw.r1[bq], sw.r2[bq], sw.al[bq], dx, dy, dz, e);
-        // invalid lanes: zero opacity and finite inputs, so every moment is
-        // exactly 0 and T, S pass through unchanged
-        const float a = valid ? e.a : 0.f;
-        const float araw = valid ? e.araw : 0.f;
-        const float t = valid ? e.t : 0.f;
-        const float u = valid ? e.u : 0.f;
-        const float v = valid ? e.v : 0.f;
-        const float rden = valid ? e.rden : 0.f;
-        const float iom = rcp_ftz(1.0f - a);
-        const float Tk = T * iom;
-        const float sg = e.den > 0.f ? -1.f : 1.f;
-        const float gc = gA + gSt * t + sg * (gSx * r0.x + gSy * r0.y + gSz * r0.z);
-        const float w = a * Tk;
-        const float dLda = Tk * gc - S * iom;
-        S = fmaf(w, gc, S);
-        T = Tk;
-        const float g = araw < 0.99f ? araw * dLda : 0.f;
-        const float ug = u * g, vg = v * g;
-        const float ct = fmaf(w, gSt, -fmaf(ug, e.ud, vg * e.vd)) * rden;
-        const float wsg = w * sg;
-        float mv[12];
-        mv[0] = g;
-        mv[1] = ug;
-        mv[2] = vg;
-        mv[3] = u * ug;
-        mv[4] = v * vg;
-        mv[5] = u * vg;
-        mv[6] = ct;
-        mv[7] = ct * u;
-        mv[8] = ct * v;
-        mv[9] = wsg * gSx;
-        mv[10] = wsg * gSy;
-        mv[11] = wsg * gSz;
-        int idx;
-        const float red = warp_reduce12(mv, lane, idx);
-        if (idx >= 0 && red != 0.f) atomicAdd(g13 + 16 * static_cast<int64_t>(si[bq]) + idx, red);
-      } while (m);
+      const int cnt = static_cast<int>(min(32u, hits - b));
+      for (int j = 0; j < cnt; ++j) {
+        // the pixels that composited this entry: their evaluation (the
+        // forward's, bit for bit) is valid
+        const uint32_t who = __shfl_sync(0xffffffffu, my_who, j);
+        const uint32_t n = static_cast<uint32_t>(__popc(who));
+        const uint32_t nl = (n + kBwdPer - 1) / kBwdPer;
+        if (lanes + nl > 32u || used + n > kBwdSlots) {
+          bwd_flush(sb, lane, w_first, w_end, w_step, w_item, g13);
+          used = 0;
+          lanes = 0;
+          w_end = 0;
+        }
+        const uint32_t share = lane - lanes;
+        if (share < nl) {
+          w_first = used + share;
+          w_end = used + n;
+          w_step = nl;
+          w_item = si[j];
+        }
+        lanes += nl;
+        if ((who >> lane) & 1u) {
+          const float4 r0 = sw.r0[j];
+          Eval e;
+          eval_pair(r0, sw.r1[j], sw.r2[j], sw.al[j], dx, dy, dz, e);
+          const float iom = rcp_ftz(1.0f - e.a);
+          const float Tk = T * iom;
+          const float sg = e.den > 0.f ? -1.f : 1.f;
+          const float gc = gA + gSt * e.t + sg * (gSx * r0.x + gSy * r0.y + gSz * r0.z);
+          const float w = e.a * Tk;
+          const float dLda = Tk * gc - S * iom;
+          S = fmaf(w, gc, S);
+          T = Tk;
+          const float g = e.araw < 0.99f ? e.araw * dLda : 0.f;
+          const float ct = fmaf(w, gSt, -fmaf(e.u * g, e.ud, e.v * g * e.vd)) * e.rden;
+          const float wsg = w * sg;
+          const uint32_t slot = used + static_cast<uint32_t>(__popc(who & ((1u << lane) - 1u)));
+          sb.a[slot] = make_float4(g, e.u, e.v, ct);
+          sb.b[slot] = make_float4(wsg * gSx, wsg * gSy, wsg * gSz, 0.f);
+        }
+        used += n;
+      }
     }
   }
+  if (lanes) bwd_flush(sb, lane, w_first, w_end, w_step, w_item, g13);
   // (the claim counter and the queue sizes are zeroed for the next backward
   // by k_preprocess_bwd, which follows on the stream; no statistics counters: the backward's contributions are the forward's
   // composited pairs, counted there)
