@@ -215,6 +215,55 @@ __device__ __forceinline__ void for_each_in_set(const TileSet& t, const FrameDev
   }
 }
 
+// A lane's tile set within the warp: its first row's tile 0 and the frame's
+// column count with it (a warp's items may lie in two frames).
+struct WarpSet {
+  uint32_t row0, ntc;   // global id of tile (r0, 0); columns of the frame
+  int nr, c0, nc;
+};
+
+__device__ __forceinline__ WarpSet warp_set(const TileSet& t, const FrameDev& F) {
+  return WarpSet{F.tile_base + static_cast<uint32_t>(t.r0 * F.ntc), static_cast<uint32_t>(F.ntc), t.r1 - t.r0 + 1, t.c0,
+                 t.nc};
+}
+
+// Calls fn(tile) for every tile of every lane's set; all lanes call it.  A set
+// of up to kOwnTiles tiles is walked by its lane, a larger one by the whole
+// warp: a surfel beside the sensor meets hundreds of tiles, and its CTA waited
+// for its lane (8 keyframes of a 1M map: the kernel 744 -> 603 us; a street
+// frame, 200k surfels, and six batched maps as before, 21 and 272 us).  Line at
+// 8: 642, 26 and 381 us (the warp takes the sets in turn, with a broadcast each);
+// 20: 612, 21.6, 272; 64: 596, 22.6, 273.  Several items per thread were worse
+// (1.41 ms at 6): the near surfels are neighbours in the map, so they come to
+// the same CTAs.
+constexpr int kOwnTiles = 32;
+
+template <class Fn>
+__device__ __forceinline__ void for_warp_sets(const WarpSet& w, int lane, Fn fn) {
+  const int n = w.nr * w.nc;
+  if (n > 0 && n <= kOwnTiles) {
+    for (int r = 0; r < w.nr; ++r)
+      for (int k = 0; k < w.nc; ++k) {
+        uint32_t jc = static_cast<uint32_t>(w.c0 + k);
+        if (jc >= w.ntc) jc -= w.ntc;
+        fn(w.row0 + static_cast<uint32_t>(r) * w.ntc + jc);
+      }
+  }
+  for (uint32_t big = __ballot_sync(0xffffffffu, n > kOwnTiles); big; big &= big - 1) {
+    const int l = __ffs(big) - 1;
+    const uint32_t row0 = __shfl_sync(0xffffffffu, w.row0, l), ntc = __shfl_sync(0xffffffffu, w.ntc, l);
+    const uint32_t c0 = __shfl_sync(0xffffffffu, static_cast<uint32_t>(w.c0), l);
+    const uint32_t nc = __shfl_sync(0xffffffffu, static_cast<uint32_t>(w.nc), l);
+    const uint32_t m = __shfl_sync(0xffffffffu, static_cast<uint32_t>(n), l);
+    for (uint32_t i = lane; i < m; i += 32) {
+      const uint32_t r = i / nc;
+      uint32_t jc = c0 + (i - r * nc);
+      if (jc >= ntc) jc -= ntc;
+      fn(row0 + r * ntc + jc);
+    }
+  }
+}
+
 __device__ __forceinline__ uint2 pack_set(const TileSet& t) {
   return make_uint2(static_cast<uint32_t>(t.r0) | (static_cast<uint32_t>(t.r1 < 0 ? 0 : t.r1) << 16),
                     static_cast<uint32_t>(t.c0) | (static_cast<uint32_t>(t.nc) << 16));
@@ -276,6 +325,11 @@ __global__ void __launch_bounds__(256) k_preprocess(const Desc* __restrict__ D, 
     __syncthreads();
   }
   uint32_t c = 0;
+  WarpSet ws{0u, 1u, 0, 0, 0};
+  const auto count = [&](uint32_t t) {
+    if (aw.local) atomicAdd(s_cnt + (t - aw.base), 1u);
+    else atomicAdd(tcount + t, 1u);
+  };
   if (live) {
     const int f = frame_of_item(*D, item);
     const FrameDev& F = D->f[f];
@@ -290,12 +344,8 @@ __global__ void __launch_bounds__(256) k_preprocess(const Desc* __restrict__ D, 
     key[item] = __float_as_uint(g.r);
     const float4 pb = pixel_box(g, F);
     TileSet ts;
-    const auto count = [&](uint32_t t) {
-      if (aw.local) atomicAdd(s_cnt + (t - aw.base), 1u);
-      else atomicAdd(tcount + t, 1u);
-    };
     if (tile_set(g, F, tab, pb, ts)) {
-      for_each_in_set(ts, F, count);
+      ws = warp_set(ts, F);
       c = static_cast<uint32_t>((ts.r1 - ts.r0 + 1) * ts.nc);
       tset[item] = pack_set(ts);
     } else {
@@ -331,6 +381,8 @@ __global__ void __launch_bounds__(256) k_preprocess(const Desc* __restrict__ D, 
     out[3] = make_float4(alpha, su, sv, 0.f);
     box[item] = cull_box(g, F, pb, tux, tuy, tuz, tvx, tvy, tvz, su, sv);
   }
+  __syncwarp();
+  for_warp_sets(ws, threadIdx.x & 31, count);
   // visible-item count, one atomic per warp
   const uint32_t vis = __ballot_sync(0xffffffffu, c > 0);
   if ((threadIdx.x & 31) == 0 && vis) atomicAdd(&st->n_vis, static_cast<unsigned int>(__popc(vis)));
@@ -503,6 +555,14 @@ __global__ void __launch_bounds__(kScanCta) k_tile_scan(uint32_t* __restrict__ t
 // ---------------------------------------------------------------------------
 // Emission into the tile buckets
 // ---------------------------------------------------------------------------
+// Bound by the latency of its dependent steps (set, shared counter, run,
+// 8-byte scattered store) and the CTA's three barriers.  One shared array, whose
+// counters become the runs' next slots, instead of counters and bases: 16 KB
+// less per CTA and one access less per pair; 8 keyframes of a 1M map 577 -> 517
+// us, six batched maps 291 -> 279, a street frame (200k surfels) 13.7 -> 13.9.
+// Large sets stay with their lanes here (by the whole warp 633, 282 and 14.4
+// us: the fill is held up by its stores, not by the enumeration); several
+// items per thread 570 to 635 us, CTAs of 128 and 512 threads 544 and 598.
 __global__ void __launch_bounds__(256) k_emit(const Desc* __restrict__ D, const float* __restrict__ tab,
                                                const uint32_t* __restrict__ key, const uint32_t* __restrict__ cnt,
                                                const uint2* __restrict__ tset, uint32_t* __restrict__ tcur,
@@ -510,7 +570,7 @@ __global__ void __launch_bounds__(256) k_emit(const Desc* __restrict__ D, const 
                                                unsigned long long* __restrict__ pkey) {
   pdl_wait();               // (launched after a kernel of this chain: wait for it)
   pdl_launch_dependents();  // the next kernel may be dispatched now
-  __shared__ uint32_t s_cnt[kAggTiles], s_base[kAggTiles];
+  __shared__ uint32_t s_pos[kAggTiles];
   if (st->overflow) return;
   const int64_t item = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   const AggWin aw = agg_window(*D);
@@ -559,26 +619,21 @@ __global__ void __launch_bounds__(256) k_emit(const Desc* __restrict__ D, const 
     }
     return;
   }
-  // shared counters: count, reserve one run per touched tile, then fill it
-  for (uint32_t t = threadIdx.x; t < aw.n; t += blockDim.x) s_cnt[t] = 0u;
+  // shared counters: count, reserve one run per touched tile (the counter
+  // becomes the run's next slot), then fill it
+  for (uint32_t t = threadIdx.x; t < aw.n; t += blockDim.x) s_pos[t] = 0u;
   __syncthreads();
   if (c) {
-    const uint32_t n = tiles([&](uint32_t t) { atomicAdd(s_cnt + (t - aw.base), 1u); });
+    const uint32_t n = tiles([&](uint32_t t) { atomicAdd(s_pos + (t - aw.base), 1u); });
     if (n != c) st->check = 1u;
   }
   __syncthreads();
   for (uint32_t t = threadIdx.x; t < aw.n; t += blockDim.x) {
-    const uint32_t m = s_cnt[t];
-    if (m) {
-      s_base[t] = atomicAdd(tcur + aw.base + t, m);
-      s_cnt[t] = 0u;
-    }
+    const uint32_t m = s_pos[t];
+    if (m) s_pos[t] = atomicAdd(tcur + aw.base + t, m);
   }
   __syncthreads();
-  if (c) tiles([&](uint32_t t) {
-    const uint32_t lt = t - aw.base;
-    put(t, s_base[lt] + atomicAdd(s_cnt + lt, 1u));
-  });
+  if (c) tiles([&](uint32_t t) { put(t, atomicAdd(s_pos + (t - aw.base), 1u)); });
 }
 
 // ---------------------------------------------------------------------------
