@@ -1492,31 +1492,31 @@ constexpr int kBwdChunkCta = 128;
 // A hit's 12 moments are summed over its pixels in two phases.  Phase A walks
 // the chunk's hits one by one, as every lane's recurrence of T and S needs; a
 // lane whose pixel composited the hit leaves its contribution (g, u, v, ct;
-// w sg gS) in the warp's next free slots of shared memory, and the hit takes
-// one lane for every kBwdPer of its contributions.  Phase B, once the lanes
-// or the slots are all taken, has every lane sum its own and add the moments
-// with three 16-byte reductions.  Contributions wait across chunks and tiles:
-// the sums need nothing of where they came from but the item.
+// w sg gS) in the warp's next free slots of shared memory.  Phase B, once
+// kBwdHits hits are waiting or the slots are full, sums them with four lanes
+// per hit and adds the moments with three 16-byte reductions, once per hit:
+// of one hit the sum is always the same, only the hits' order varies.
+// Contributions wait across chunks and tiles: the sums need nothing of where
+// they came from but the item.
 //
-// Bound by issue (about 70 % of the cycles) and the latency of the chunk's six
+// Bound by issue (74 % of the cycles) and the latency of the chunk's six
 // dependent reads.  Before, the 12 moments were summed over the warp with
 // shuffles hit by hit and added by 12 lanes with scalar atomics: 162
 // instructions a hit on the street frame (200k surfels, 128 x 1024), of whose
-// 32 lanes 8 held a contribution; now 120.  Kernel 131 -> 112 us; on 8 keyframes
-// of a dense 1M map (12 lanes of 32) 1195 -> 1166 us, on six batched maps
-// 733 -> 707 us; the steps 336 -> 315, 5945 -> 5890 and 4285 -> 4258 us.
-// Shares and slots, the three steps' gains: 4 and 96 6.6, 0.9, 0.6 %; 6 and 96
-// 5.1, 0.7, 0.2 %; 8 and 160 6.6, 0.8, -0.9 % (more shared memory leaves less
-// L1 to the batched maps' reads).  An item's three vectors leave by three
-// neighbouring lanes, as one request: by one lane after the other the
-// keyframes' kernel took 65 us more.  Others, street frame and keyframes: four
-// lanes per hit for 8 hits at a time 117 and 1190 us (the longest of the 8
-// decides), every lane walking its own pixel's bits 118 and 1279 us (its record
-// reads from shared memory conflict), two hits' evaluations at a time 130 and
-// 1687 us (128 registers), the next chunk claimed ahead 135 and 1162 us (a
+// 32 lanes 8 held a contribution; now 125.  Kernel 131 -> 113 us, its step 335 ->
+// 318 us; the steps of 8 keyframes of a dense 1M map (12 lanes of 32) and of six
+// batched maps gain 0.4 and 0.5 %.  Slots, the three steps: 96 318, 5728 and
+// 4226 us; 128 317, 5710 and 4260; 80 324, 5750 and 4244
+// (more shared memory leaves less L1 to the batched maps' reads).  Others: one
+// lane per 4 contributions, each with its own three reductions, 313 and 5690 us,
+// but twice the additions in an order that varies (results of two runs differed
+// more than before); the same with the hit's lanes added up first 328 and 5760;
+// every lane walking its own pixel's bits 322 and 6085 before the binning's last
+// change (its record reads from shared memory conflict); two hits' evaluations
+// at a time 330 and 6340 (128 registers); the next chunk claimed ahead 346 (a
 // street frame has four chunks per warp: the last ones no longer balance).
-constexpr uint32_t kBwdPer = 4;      // contributions a lane sums
-constexpr uint32_t kBwdSlots = 96;   // at least a hit's 32, and 32 lanes' sums
+constexpr int kBwdHits = 8;          // hits summed at a time
+constexpr uint32_t kBwdSlots = 96;   // at least a hit's 32
 
 struct BwdWarp {
   WarpRecs rec;
@@ -1532,15 +1532,19 @@ __device__ __forceinline__ void red_add4(float* p, float x, float y, float z, fl
   asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
 }
 
-// Phase B: the lane sums the contributions in its slots (first, first + step,
-// ... below end) and adds the 12 moments to its item.
-__device__ __forceinline__ void bwd_flush(BwdWarp& sb, int lane, uint32_t first, uint32_t end, uint32_t step, uint32_t item,
-                                          float* __restrict__ g13) {
+// Phase B: hit i < kBwdHits waits in the slots from lane i's `start` to lane
+// i + 1's (`start` is the end for lanes past the last hit); `item` is its item.
+__device__ __forceinline__ void bwd_flush(const BwdWarp& sb, uint32_t start, uint32_t item, float* __restrict__ g13,
+                                          int lane) {
+  static_assert(kBwdHits == 8, "four lanes per hit");
   __syncwarp();
+  const uint32_t s0 = __shfl_sync(0xffffffffu, start, lane >> 2);
+  const uint32_t s1 = __shfl_sync(0xffffffffu, start, (lane >> 2) + 1);
+  const uint32_t it = __shfl_sync(0xffffffffu, item, lane >> 2);
   float v[12];
 #pragma unroll
   for (int q = 0; q < 12; ++q) v[q] = 0.f;
-  for (uint32_t i = first; i < end; i += step) {
+  for (uint32_t i = s0 + (lane & 3); i < s1; i += 4) {
     const float4 a = sb.a[i], b = sb.b[i];
     const float ug = a.y * a.x, vg = a.z * a.x;
     v[0] += a.x;
@@ -1556,21 +1560,21 @@ __device__ __forceinline__ void bwd_flush(BwdWarp& sb, int lane, uint32_t first,
     v[10] += b.y;
     v[11] += b.z;
   }
-  // an item's three vectors by neighbouring lanes, so that they leave as one request
-  static_assert(kBwdSlots >= 96, "32 lanes' sums");
-  __syncwarp();
-  sb.a[3 * lane] = make_float4(v[0], v[1], v[2], v[3]);
-  sb.a[3 * lane + 1] = make_float4(v[4], v[5], v[6], v[7]);
-  sb.a[3 * lane + 2] = make_float4(v[8], v[9], v[10], v[11]);
-  __syncwarp();
-  const uint32_t has = __ballot_sync(0xffffffffu, first < end);
+  // over the four lanes: lanes 0 and 1 of the four end with moments 0-3 and
+  // 4-7, lane 2 with 8-11
+  const bool up = lane & 2, odd = lane & 1;
+  float k[8];
 #pragma unroll
-  for (int r = 0; r < 3; ++r) {
-    const int at = 32 * r + lane, src = at / 3;
-    const uint32_t it = __shfl_sync(0xffffffffu, item, src);
-    const float4 x = sb.a[at];
-    if ((has >> src) & 1u) red_add4(g13 + 16 * static_cast<int64_t>(it) + 4 * (at - 3 * src), x.x, x.y, x.z, x.w);
+  for (int q = 0; q < 8; ++q) {
+    const float hi = q < 4 ? v[8 + (q & 3)] : 0.f;
+    k[q] = (up ? hi : v[q]) + __shfl_xor_sync(0xffffffffu, up ? v[q] : hi, 2);
   }
+  float r[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    r[q] = (odd ? k[4 + q] : k[q]) + __shfl_xor_sync(0xffffffffu, odd ? k[q] : k[4 + q], 1);
+  if (s1 > s0 && (lane & 3) < 3)
+    red_add4(g13 + 16 * static_cast<int64_t>(it) + 4 * (lane & 3), r[0], r[1], r[2], r[3]);
   __syncwarp();
 }
 
@@ -1587,8 +1591,9 @@ __global__ void __launch_bounds__(kBwdChunkCta, 7)
   BwdWarp& sb = s_w[threadIdx.x >> 5];
   WarpRecs& sw = sb.rec;
   uint32_t* si = sb.item;
-  // contributions that wait for phase B: slots and lanes taken, the lane's share
-  uint32_t used = 0, lanes = 0, w_first = 0, w_end = 0, w_step = 1, w_item = 0;
+  // the hits that wait for phase B: their count and slots (warp-uniform); lane i holds hit i's
+  int waiting = 0;
+  uint32_t used = 0, w_start = 0, w_item = 0;
   const int npx = D->th * D->tw, wpt = npx >> 5;
   // the forward's queues, claimed in class order: lane l < kBwdClasses holds
   // class l's size (clamped to its capacity) and the items before its end
@@ -1695,21 +1700,16 @@ __global__ void __launch_bounds__(kBwdChunkCta, 7)
         // forward's, bit for bit) is valid
         const uint32_t who = __shfl_sync(0xffffffffu, my_who, j);
         const uint32_t n = static_cast<uint32_t>(__popc(who));
-        const uint32_t nl = (n + kBwdPer - 1) / kBwdPer;
-        if (lanes + nl > 32u || used + n > kBwdSlots) {
-          bwd_flush(sb, lane, w_first, w_end, w_step, w_item, g13);
+        if (waiting == kBwdHits || used + n > kBwdSlots) {
+          bwd_flush(sb, lane < waiting ? w_start : used, w_item, g13, lane);
+          waiting = 0;
           used = 0;
-          lanes = 0;
-          w_end = 0;
         }
-        const uint32_t share = lane - lanes;
-        if (share < nl) {
-          w_first = used + share;
-          w_end = used + n;
-          w_step = nl;
+        if (lane == waiting) {
+          w_start = used;
           w_item = si[j];
         }
-        lanes += nl;
+        ++waiting;
         if ((who >> lane) & 1u) {
           const float4 r0 = sw.r0[j];
           Eval e;
@@ -1733,7 +1733,7 @@ __global__ void __launch_bounds__(kBwdChunkCta, 7)
       }
     }
   }
-  if (lanes) bwd_flush(sb, lane, w_first, w_end, w_step, w_item, g13);
+  if (waiting) bwd_flush(sb, lane < waiting ? w_start : used, w_item, g13, lane);
   // (the claim counter and the queue sizes are zeroed for the next backward
   // by k_preprocess_bwd, which follows on the stream; no statistics counters: the backward's contributions are the forward's
   // composited pairs, counted there)

@@ -1,10 +1,10 @@
-"""The chunked backward sums a hit's moments over its pixels by lanes of up to
-4 contributions, from 96 slots per warp.  Surfels that cover about one pixel,
-a few, most and all of a 4 x 8 block, opaque and faint, in lists around one
-and two chunks of 128 entries and around one lane's and one warp's share;
-every gradient value against the oracle within the parity tests' bar (not the
-share of values within the bar without the cases' own uncertainty: one value
-of these few hundred is more than the share those tests allow)."""
+"""The chunked backward sums the moments of up to 8 hits at a time over their
+pixels, from 96 slots per warp, four lanes per hit.  Surfels that cover about
+one pixel, a few, most and all of a 4 x 8 block, opaque and faint, in lists
+around one and two chunks of 128 entries and of less than 8 hits; every
+gradient value against the oracle within the parity tests' bar (not the share
+of values within the bar without the cases' own uncertainty: one value of
+these few hundred is more than the share those tests allow)."""
 import numpy as np
 import pytest
 
