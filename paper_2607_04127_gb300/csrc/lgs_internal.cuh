@@ -81,8 +81,8 @@ struct Desc {
 };
 
 // Queues of the chunked backward's work items, in the order warps claim
-// them: class 0 holds the chunks a warp block walks in full (and every chunk
-// of a long list), classes 1 .. kBwdClasses-1 the chunk in which the block's
+// them: class 0 holds the chunks a warp block walks in full, classes
+// 1 .. kBwdClasses-1 the chunk in which the block's
 // last composited entry lies, by decreasing length of its walked part.  The
 // costliest items go first, so the backward ends on short ones.  Built at
 // the start of every backward from the forward's per-block last entries.
@@ -156,7 +156,9 @@ struct WsPtrs {
   uint32_t* dead;          // [long lists][tile pixels] first segment known to stop the pixel (~0 between forwards)
   uint32_t* cmask;         // [chunks][4 windows][tile pixels] entries each pixel composited, one bit per entry
   uint2* groups;           // [pairs / 512 + 1] ranges of the long buckets' groups (st->n_groups of them)
-  uint32_t* bwm;           // [tiles][warp blocks] the block's largest n_contrib (short lists; written by k_fwd_s)
+  uint32_t* bwm;           // [tiles][warp blocks] the block's largest n_contrib, 0 outside the frame.  Every forward that
+                           // the chunked backward may follow sets every word: k_fwd_s those of tiles with short
+                           // lists, k_long_masks (0) and k_fwd_long (the maximum) those of long ones
   uint2* bq;               // backward work queues: (chunk * blocks per tile + block, tile); class 0 first
   uint32_t bq_cap0, bq_capk;
 };

@@ -881,6 +881,9 @@ __global__ void __launch_bounds__(256, 3)
     const uint2 it = __ldg(seg.item + id / blocks);
     const uint32_t li = it.x, sg = it.y, tile = __ldg(seg.longt + li);
     const int vt = static_cast<int>(id % blocks) * 32 + lane;
+    // (step (2) takes the maximum over the block's pixels; a block outside the
+    // frame has none, and the backward's queues read its word all the same)
+    if (sg == 0 && lane == 0) bwm[tile * blocks + id % blocks] = 0u;
     const TileCtx tc = tile_ctx(D, tile, ranges, vt);
     uint32_t* dead = seg.dead + static_cast<int64_t>(li) * npx + vt;
     bool done = !tc.inside || __ldcg(dead) < sg;
@@ -893,7 +896,6 @@ __global__ void __launch_bounds__(256, 3)
     // the checkpoints and the segment's sums start empty (step (2) writes the
     // chunks and segments in which the pixel composites something)
     const int64_t cb = static_cast<int64_t>(cbase[tile]);
-    if (sg == 0 && lane == 0) bwm[tile * blocks + id % blocks] = 0u;   // (step (2) takes the maximum)
     for (uint32_t c = sg * kSegChunks; c * kChunk < end - tc.start; ++c)
 #pragma unroll
       for (int k = 0; k < kCkptSlots; ++k) ckpt[((cb + c) * kCkptSlots + k) * npx + vt] = 0.f;
@@ -1871,11 +1873,13 @@ __global__ void __launch_bounds__(256) k_bwd_prep(const Desc* __restrict__ D, co
   for (uint32_t t0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); t0 < n_tiles; t0 += gridDim.x * blockDim.x) {
     const uint32_t tile = t0 + static_cast<uint32_t>(lane);
     const bool ok = tile < n_tiles;
+    // (no word exceeds the list: a queued chunk is always one of the tile's)
+    const uint2 rg = ok ? ranges[tile] : make_uint2(0u, 0u);
     uint32_t wm[kMaxBlocks];
     uint32_t nfull = 0, nf_max = 0;
 #pragma unroll
     for (int b = 0; b < kMaxBlocks; ++b) {
-      wm[b] = ok && static_cast<uint32_t>(b) < blocks ? bwm[tile * blocks + b] : 0u;
+      wm[b] = ok && static_cast<uint32_t>(b) < blocks ? min(bwm[tile * blocks + b], rg.y - rg.x) : 0u;
       nfull += wm[b] / kChunk;
       nf_max = max(nf_max, wm[b] / kChunk);
     }
