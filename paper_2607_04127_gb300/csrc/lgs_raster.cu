@@ -1630,7 +1630,9 @@ __global__ void __launch_bounds__(kBwdChunkCta, 7)
     const int64_t pix = static_cast<int64_t>(r) * F.W + col;
     const uint2 rg = ranges[tile];
     const int k_lo = static_cast<int>(c * kChunk);
-    const int nc = inside ? F.nc[pix] : 0;
+    // n_contrib comes from the caller: never walk past the tile's list (its
+    // chunks, segments and window masks end there)
+    const int nc = inside ? min(F.nc[pix], static_cast<int>(rg.y - rg.x)) : 0;
     const bool act = nc > k_lo;
     float dx = 0.f, dy = 0.f, dz = 0.f;
     float T = 1.f, S = 0.f, gA = 0.f, gSt = 0.f, gSx = 0.f, gSy = 0.f, gSz = 0.f;
@@ -1961,7 +1963,8 @@ __global__ void __launch_bounds__(256) k_bwd_prep(const Desc* __restrict__ D, co
     const int vt = static_cast<int>(blk) * 32 + lane;
     const TileCtx tc = tile_ctx(*D, tile, ranges, vt);
     const FrameDev& F = D->f[tc.f];
-    const int nc = tc.inside ? F.nc[tc.pix] : 0;
+    // (the caller's n_contrib, at most the list)
+    const int nc = tc.inside ? min(F.nc[tc.pix], static_cast<int>(tc.end - tc.start)) : 0;
     const int ns = nc > 0 ? (nc - 1) / static_cast<int>(kSeg) + 1 : 0;   // the pixel's segments
     const int per = (__reduce_max_sync(0xffffffffu, ns) + 7) / 8;
     const int lo = part * per, hi = min(lo + per, ns);
