@@ -215,7 +215,13 @@ Layout make_layout(int64_t items, uint32_t tiles, int64_t pairs_cap, uint32_t ta
   L.cnt = take(4 * I);
   L.tset = take(8 * I);
   L.tcur = take(4 * T);
-  L.pkey = take(8 * P);
+  // a list of n > kLongList entries has ceil(n / kSeg) <= n / kSeg + 1 segments,
+  // and there are at most P / kLongList such lists
+  const size_t LL = std::min(T, P / lgs::kLongList), SG = LL ? P / lgs::kSeg + P / lgs::kLongList : 0;
+  // the sort's keys, and from the forward on (which follows the sort) the long
+  // lists' segment sums: a pair costs no more than its key with tiles of up to
+  // 128 pixels, 11 bytes with 256
+  L.pkey = L.segsum = take(std::max(8 * P, sizeof(float) * 5 * static_cast<size_t>(tile_pixels) * SG));
   L.ptile = take(4 * P);
   L.pv = take(4 * P);
   L.ranges = take(8 * T);
@@ -229,11 +235,8 @@ Layout make_layout(int64_t items, uint32_t tiles, int64_t pairs_cap, uint32_t ta
   L.cmask = take(sizeof(uint32_t) * 4 * static_cast<size_t>(tile_pixels) * static_cast<size_t>(C));
   // a bucket of n > 2048 keys has ceil(n / 1024) < n / 512 groups at most
   L.groups = take(sizeof(uint2) * (P / 512 + 1));
-  // a list of n > kLongList entries has ceil(n / kSeg) <= n / kSeg + n / kLongList segments
-  const size_t SG = P / lgs::kSeg + P / lgs::kLongList + 1, LL = std::min(T, P / lgs::kLongList + 1);
   L.segs = take(sizeof(uint2) * SG);
   L.sbase = take(4 * T);
-  L.segsum = take(sizeof(float) * 5 * static_cast<size_t>(tile_pixels) * SG);
   L.ssuf = take(sizeof(float) * static_cast<size_t>(tile_pixels) * SG);
   L.dead = take(sizeof(uint32_t) * static_cast<size_t>(tile_pixels) * LL);
   // backward queues: class 0 takes at most every (chunk, warp block) item,

@@ -139,7 +139,7 @@ struct WsPtrs {
   uint32_t* cnt;           // tile count per item
   uint2* tset;             // tile set per item: rows (first | last << 16), columns (first | count << 16)
   uint32_t* tcur;          // [tiles] pair counts, then fill cursors
-  unsigned long long* pkey;// [pairs] (depth key << 32 | item), bucketed by tile, then sorted
+  unsigned long long* pkey;// [pairs] (depth key << 32 | item), bucketed by tile (until the forward: segsum)
   uint32_t* ptile;         // [pairs] tile of every pair (sorted order)
   uint32_t* pv;            // [pairs] item of every pair (sorted order)
   uint2* ranges;           // [tiles]
@@ -151,7 +151,7 @@ struct WsPtrs {
   float* ckpt;             // [chunks][kCkptSlots][tile pixels] forward checkpoint at every chunk end
   uint2* segs;             // [segments] segments of the long lists: (long list, segment), segment by segment
   uint32_t* sbase;         // [tiles] first segment of a long list
-  float* segsum;           // [segments][5][tile pixels] a segment's sums (SegBuf)
+  float* segsum;           // [segments][5][tile pixels] a segment's sums (SegBuf); in pkey's place, which the sort is done with
   float* ssuf;             // [segments][tile pixels] the suffix of the later segments (backward)
   uint32_t* dead;          // [long lists][tile pixels] first segment known to stop the pixel (~0 between forwards)
   uint32_t* cmask;         // [chunks][4 windows][tile pixels] entries each pixel composited, one bit per entry
