@@ -34,6 +34,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "lgs_internal.cuh"
 
@@ -982,40 +983,41 @@ __global__ void __launch_bounds__(kMgCta) k_mg_write(const float* __restrict__ m
   block_count64(n_split, &counts[5]);
 }
 
-// One CTA carries `per` rows at a time, V 32-bit words per load where the
-// rows allow it (words a multiple of V, both arrays aligned): HBM-bound.  The
-// row of a word needs a division, of 32 bits here (of 64 bits, over the whole
-// array, it bound the kernel: 1M rows of 10 words 45 us, now 23).
-constexpr int64_t kGatherRows = 128;
-template <class V>
+// A CTA carries PER loads per thread at a time, whole rows or a part of a wide
+// one, V 32-bit words per load where the rows allow it (words a multiple of V,
+// both arrays aligned): HBM-bound.  The row of a word needs a division, of 32
+// bits here, from the row at which the CTA's share starts.  (Of 64 bits, over the
+// whole array, it bound the kernel: 1M rows of 10 words 28 us, now 17.4.  Shares
+// of 128 rows: 17.0, but 64 rows of 65,536 words took one CTA 946 us, now 5.9,
+// and 1M rows of one word 8.8, now 5.4.)
+template <class V, int PER>
 __global__ void __launch_bounds__(kMgCta) k_mg_gather(const int32_t* __restrict__ src, const uint8_t* __restrict__ role,
                                                       const int64_t* __restrict__ counts, int64_t capacity,
                                                       const V* __restrict__ in, V* __restrict__ out, uint32_t words,
-                                                      int64_t per, int zero_children) {
+                                                      int zero_children) {
   const int64_t n_out = counts[0] < capacity ? counts[0] : capacity;
-  for (int64_t r0 = blockIdx.x * per; r0 < n_out; r0 += gridDim.x * per) {
-    const uint32_t rows = static_cast<uint32_t>(n_out - r0 < per ? n_out - r0 : per);
-    const uint32_t total = rows * words;
-    for (uint32_t e0 = threadIdx.x; e0 < total; e0 += 4 * kMgCta) {
-      // four words per round: their rows, then the words
-      int64_t from[4];
+  constexpr int kShare = PER * kMgCta;
+  const int64_t total = n_out * words, step = static_cast<int64_t>(gridDim.x) * kShare;
+  for (int64_t e0 = static_cast<int64_t>(blockIdx.x) * kShare; e0 < total; e0 += step) {
+    const int64_t row0 = e0 >> 32 ? e0 / words : static_cast<uint32_t>(e0) / words;
+    const uint32_t first = static_cast<uint32_t>(e0 - row0 * words) + threadIdx.x;   // (words < 2^31)
+    // the words' rows, then the words
+    int64_t from[PER];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const uint32_t e = e0 + u * kMgCta;
-        from[u] = -1;
-        if (e < total) {
-          const uint32_t row = e / words;
-          const int32_t p = src[r0 + row];
-          if (!(zero_children && role[r0 + row])) from[u] = static_cast<int64_t>(p) * words + (e - row * words);
-        }
+    for (int u = 0; u < PER; ++u) {
+      from[u] = -1;
+      if (e0 + threadIdx.x + u * kMgCta < total) {
+        const uint32_t e = first + u * kMgCta, r = e / words;
+        const int32_t p = src[row0 + r];
+        if (!(zero_children && role[row0 + r])) from[u] = static_cast<int64_t>(p) * words + (e - r * words);
       }
-      V v[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) v[u] = from[u] >= 0 ? in[from[u]] : V{};
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (e0 + u * kMgCta < total) out[r0 * words + e0 + u * kMgCta] = v[u];
     }
+    V v[PER];
+#pragma unroll
+    for (int u = 0; u < PER; ++u) v[u] = from[u] >= 0 ? in[from[u]] : V{};
+#pragma unroll
+    for (int u = 0; u < PER; ++u)
+      if (e0 + threadIdx.x + u * kMgCta < total) out[e0 + threadIdx.x + u * kMgCta] = v[u];
   }
 }
 
@@ -1108,12 +1110,17 @@ cudaError_t launch_manage(const lgs_surfels& M, const float* lam, const float* r
 
 cudaError_t launch_manage_gather(const int32_t* src, const uint8_t* role, const int64_t* counts, int64_t capacity,
                                  const void* in, void* out, int words, int zero_children, cudaStream_t s) {
-  // (the words of a CTA's rows are counted in 32 bits)
-  const int64_t per = words <= (1 << 24) ? kGatherRows : 1;
-  const int g = static_cast<int>(std::min<int64_t>((capacity + per - 1) / per, 16 * sm_count()));
   const uintptr_t at = reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out);
+  const int sms = sm_count();
   const auto run = [&](auto* i, auto* o, int w) {
-    k_mg_gather<<<g, kMgCta, 0, s>>>(src, role, counts, capacity, i, o, static_cast<uint32_t>(w), per, zero_children);
+    // four loads per thread once one each would fill the chip
+    const int64_t total = capacity * w;
+    const bool wide = total > static_cast<int64_t>(8) * sms * kMgCta;
+    const int64_t share = (wide ? 4 : 1) * kMgCta;
+    const int g = static_cast<int>(std::min<int64_t>((total + share - 1) / share, 16 * sms));
+    using V = std::remove_cv_t<std::remove_pointer_t<decltype(o)>>;
+    (wide ? k_mg_gather<V, 4> : k_mg_gather<V, 1>)<<<g, kMgCta, 0, s>>>(src, role, counts, capacity, i, o,
+                                                                        static_cast<uint32_t>(w), zero_children);
   };
   if (words % 4 == 0 && at % 16 == 0) run(static_cast<const uint4*>(in), static_cast<uint4*>(out), words / 4);
   else if (words % 2 == 0 && at % 8 == 0) run(static_cast<const uint2*>(in), static_cast<uint2*>(out), words / 2);
