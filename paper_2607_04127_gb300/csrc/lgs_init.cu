@@ -271,29 +271,35 @@ __global__ void __launch_bounds__(kIniSortCta) k_ini_scatter(const uint32_t* __r
 }
 
 // Boxes of the leaves (32 points, one warp) and of the nodes (32 leaves, one
-// CTA): lo / hi corners as float4.
+// CTA): lo / hi corners as float4, the smallest original index of the points in
+// lo.w (as bits).
 __global__ void __launch_bounds__(1024) k_ini_boxes(const float4* __restrict__ sp, uint32_t n,
                                                     float4* __restrict__ leaf, float4* __restrict__ node) {
   pdl_wait();               // (launched after a kernel of this chain: wait for it)
   pdl_launch_dependents();  // the next kernel may be dispatched now
   __shared__ float s_lo[32][3], s_hi[32][3];
+  __shared__ uint32_t s_id[32];
   const uint32_t i = blockIdx.x * 1024 + threadIdx.x;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+  uint32_t id = 0xffffffffu;
   if (i < n) {
     const float4 p = sp[i];
     lo[0] = hi[0] = p.x;
     lo[1] = hi[1] = p.y;
     lo[2] = hi[2] = p.z;
+    id = __float_as_uint(p.w);
   }
   warp_min_max(lo, hi);
+  id = __reduce_min_sync(0xffffffffu, id);
   if (lane == 0) {
     for (int a = 0; a < 3; ++a) {
       s_lo[wid][a] = lo[a];
       s_hi[wid][a] = hi[a];
     }
+    s_id[wid] = id;
     if (i < n) {
-      leaf[2 * (i >> 5)] = make_float4(lo[0], lo[1], lo[2], 0.f);
+      leaf[2 * (i >> 5)] = make_float4(lo[0], lo[1], lo[2], __uint_as_float(id));
       leaf[2 * (i >> 5) + 1] = make_float4(hi[0], hi[1], hi[2], 0.f);
     }
   }
@@ -304,8 +310,9 @@ __global__ void __launch_bounds__(1024) k_ini_boxes(const float4* __restrict__ s
     hi[a] = s_hi[lane][a];
   }
   warp_min_max(lo, hi);
+  id = __reduce_min_sync(0xffffffffu, s_id[lane]);
   if (lane == 0) {
-    node[2 * blockIdx.x] = make_float4(lo[0], lo[1], lo[2], 0.f);
+    node[2 * blockIdx.x] = make_float4(lo[0], lo[1], lo[2], __uint_as_float(id));
     node[2 * blockIdx.x + 1] = make_float4(hi[0], hi[1], hi[2], 0.f);
   }
 }
@@ -316,16 +323,36 @@ __device__ __forceinline__ float dist2(float ax, float ay, float az, float bx, f
   return fadd(fadd(fmul(dx, dx), fmul(dy, dy)), fmul(dz, dz));
 }
 
-// Bits of a lower bound of the squared distance from (x, y, z) to any point
-// of a box (the margin covers the roundings); non-negative, so the bits order
-// as the values do.
-__device__ __forceinline__ uint32_t box_gap_bits(const float4* __restrict__ box, float x, float y, float z) {
-  const float4 lo = __ldg(box), hi = __ldg(box + 1);
-  const float gx = fmaxf(0.f, fmaxf(lo.x - x, x - hi.x));
-  const float gy = fmaxf(0.f, fmaxf(lo.y - y, y - hi.y));
-  const float gz = fmaxf(0.f, fmaxf(lo.z - z, z - hi.z));
-  return __float_as_uint((gx * gx + gy * gy + gz * gz) * 0.99999f);
-}
+// A box as a query sees it: the bits of a lower bound of the squared distance
+// from (x, y, z) to any point of it (the margin covers the roundings;
+// non-negative, so the bits order as the values do), and the smallest index of
+// its points.  A box that is not there or has been visited holds kKnnNone.
+constexpr uint32_t kKnnNone = 0xffffffffu;
+struct KnnBox {
+  uint32_t gap, id;
+  __device__ __forceinline__ KnnBox(const float4* __restrict__ box, bool there, float x, float y, float z)
+      : gap(kKnnNone), id(kKnnNone) {
+    if (!there) return;
+    const float4 lo = __ldg(box), hi = __ldg(box + 1);
+    const float gx = fmaxf(0.f, fmaxf(lo.x - x, x - hi.x));
+    const float gy = fmaxf(0.f, fmaxf(lo.y - y, y - hi.y));
+    const float gz = fmaxf(0.f, fmaxf(lo.z - z, z - hi.z));
+    gap = __float_as_uint((gx * gx + gy * gy + gz * gz) * 0.99999f);
+    id = __float_as_uint(lo.w);
+  }
+  // The lane whose box is the nearest that can hold a smaller key than the k-th
+  // of `best` (wd: its distance bits), -1 if none can: at a gap of just wd, by a
+  // smaller index.  (Coincident points, say a sensor's empty returns, all lie at
+  // gap 0 = wd: without the indices each of them visited the leaves of all, 18 ms
+  // with 50k of 102k points coincident, now 0.22.)
+  __device__ __forceinline__ int nearest(uint32_t wd, unsigned long long best, int k) const {
+    const uint32_t m = __reduce_min_sync(0xffffffffu, gap);
+    if (m < wd) return __ffs(__ballot_sync(0xffffffffu, gap == m)) - 1;
+    if (m > wd || m == kKnnNone) return -1;
+    const uint32_t wid = __shfl_sync(0xffffffffu, static_cast<uint32_t>(best), k - 1);
+    return __ffs(__ballot_sync(0xffffffffu, gap == m && id < wid)) - 1;
+  }
+};
 
 // Compare-exchange with lane ^ j: the smaller key stays where `low` holds.
 __device__ __forceinline__ void cas_lane(unsigned long long& v, int j, bool low) {
@@ -334,7 +361,6 @@ __device__ __forceinline__ void cas_lane(unsigned long long& v, int j, bool low)
 }
 
 constexpr int kKnnCta = 256;
-constexpr uint32_t kKnnNone = 0xffffffffu;   // a box that is not there or has been visited
 // Candidates of a leaf taken one by one (about 14 instructions each) up to
 // this many, by a bitonic sort and merge (about 190) beyond; 6 to 12 measured
 // the same, 18 two percent slower.
@@ -349,7 +375,7 @@ constexpr int kKnnOneByOne = 12;
 // k-th neighbour radii of a scan span 0.03 to 16 m: a CTA per 256 queries,
 // pruning with the widest of its radii and lasting as long as its worst
 // query, took 5.27 ms on the 102k points of a 128 x 1024 scan, this 0.136 ms
-// (k = 20; the whole call 5.35 -> 0.189 ms, 51k points 2.73 -> 0.111 ms).
+// (k = 20; the whole call 5.35 -> 0.191 ms, 51k points 2.73 -> 0.111 ms).
 __global__ void __launch_bounds__(kKnnCta) k_ini_knn(const float4* __restrict__ sp, uint32_t n,
                                                      const float4* __restrict__ leaf_box, uint32_t n_leaf,
                                                      const float4* __restrict__ node_box, uint32_t n_node, int k,
@@ -369,26 +395,18 @@ __global__ void __launch_bounds__(kKnnCta) k_ini_knn(const float4* __restrict__ 
   for (uint32_t t = 0; t < n_batch; ++t) {
     const uint32_t batch = t == 0 ? batch0 : (t <= batch0 ? t - 1 : t);
     const uint32_t nd = 32 * batch + lane;
-    uint32_t un = nd < n_node ? box_gap_bits(node_box + 2 * nd, me.x, me.y, me.z) : kKnnNone;
+    KnnBox un(node_box + 2 * nd, nd < n_node, me.x, me.y, me.z);
     while (true) {
-      int a = static_cast<int>(node0 & 31u);
-      if (!first) {
-        const uint32_t m = __reduce_min_sync(0xffffffffu, un);
-        if (m == kKnnNone || m > wd) break;
-        a = __ffs(__ballot_sync(0xffffffffu, un == m)) - 1;
-      }
-      if (lane == a) un = kKnnNone;
+      const int a = first ? static_cast<int>(node0 & 31u) : un.nearest(wd, best, k);
+      if (a < 0) break;
+      if (lane == a) un.gap = kKnnNone;
       const uint32_t lf = 32 * (32 * batch + a) + lane;
-      uint32_t ul = lf < n_leaf ? box_gap_bits(leaf_box + 2 * lf, me.x, me.y, me.z) : kKnnNone;
+      KnnBox ul(leaf_box + 2 * lf, lf < n_leaf, me.x, me.y, me.z);
       while (true) {
-        int b = static_cast<int>(leaf0 & 31u);
-        if (!first) {
-          const uint32_t m = __reduce_min_sync(0xffffffffu, ul);
-          if (m == kKnnNone || m > wd) break;
-          b = __ffs(__ballot_sync(0xffffffffu, ul == m)) - 1;
-        }
+        const int b = first ? static_cast<int>(leaf0 & 31u) : ul.nearest(wd, best, k);
+        if (b < 0) break;
         first = false;
-        if (lane == b) ul = kKnnNone;
+        if (lane == b) ul.gap = kKnnNone;
         const uint32_t base = 32 * (32 * (32 * batch + a) + b);
         const uint32_t i = base + lane;
         evaluated += min(32u, n - base);
