@@ -233,8 +233,9 @@ Layout make_layout(int64_t items, uint32_t tiles, int64_t pairs_cap, uint32_t ta
   L.cbase = take(4 * T);
   L.ckpt = take(sizeof(float) * lgs::kCkptSlots * static_cast<size_t>(tile_pixels) * static_cast<size_t>(C));
   L.cmask = take(sizeof(uint32_t) * 4 * static_cast<size_t>(tile_pixels) * static_cast<size_t>(C));
-  // a bucket of n > 2048 keys has ceil(n / 1024) < n / 512 groups at most
-  L.groups = take(sizeof(uint2) * (P / 512 + 1));
+  // a bucket of n > 2048 keys has at most ceil(n / 1024) groups, and as many
+  // again where groups are partitioned a second time: together < n / 256
+  L.groups = take(sizeof(uint2) * (P / 256 + 1));
   L.segs = take(sizeof(uint2) * SG);
   L.sbase = take(4 * T);
   L.ssuf = take(sizeof(float) * static_cast<size_t>(tile_pixels) * SG);

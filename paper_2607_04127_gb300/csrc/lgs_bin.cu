@@ -647,15 +647,19 @@ __global__ void __launch_bounds__(256) k_emit(const Desc* __restrict__ D, const 
 // coarse bin's width).  Both maps are monotone in the depth, so the keys of
 // one fine bin are adjacent in the result: they are placed together and each
 // finds its rank by comparing the 64-bit keys of its bin.  A bucket with more
-// than kDense keys in one fine bin (mostly equal depths) takes a bitonic sort
-// in place instead.  Bound by issue and by its nine barriers, at about 60
-// instructions per key; a merge sort, one pass per doubling, took 28 us on the
-// street frame (1.27 M keys in 1,916 buckets) and 524 us on 8 keyframes of a
-// 1M map (21.6 M keys in buckets up to 2,048), this 18 and 113 us.
+// than kDense keys in one fine bin (mostly equal depths) takes a bitonic sort up
+// to kBitonicMax keys, a merge sort beyond.  Bound by issue and by its nine
+// barriers, at about 60 instructions per key; a merge sort, one pass per
+// doubling, took 28 us on the street frame (1.27 M keys in 1,916 buckets) and
+// 524 us on 8 keyframes of a 1M map (21.6 M keys in buckets up to 2,048), this 18
+// and 113 us.
 constexpr int kSortCta = 256;
 constexpr int kSortPer = kSortMax / kSortCta;
 constexpr uint32_t kCoarse = 256;
 constexpr uint32_t kDense = 64;
+// (200 tiles of 100 equal depths, the binning: 31.4 us, merged 33.4; of 2,000
+// equal depths 75.7 and 61.4)
+constexpr uint32_t kBitonicMax = 256;
 static_assert(kCoarse == kSortCta && kSortPer == 8, "one coarse bin per thread, eight fine bins per thread");
 
 struct SortSmem {
@@ -728,10 +732,76 @@ __device__ __noinline__ void smem_bitonic(unsigned long long* key, uint32_t n) {
     }
 }
 
+__device__ __forceinline__ void cas_reg(unsigned long long& a, unsigned long long& b) {
+  const unsigned long long x = a, y = b;
+  a = x > y ? y : x;
+  b = x > y ? x : y;
+}
+
+// Shared-memory index of merged key x: one slot left free after every 8 keys, so
+// that the 8-key rows of consecutive threads start in different banks.
+__device__ __forceinline__ uint32_t pad8(uint32_t x) { return x + (x >> 3); }
+static_assert(sizeof(SortSmem) >= 8 * (kSortMax + kSortMax / 8), "the merge sort's rows reach past the keys");
+
+// Merge sort of s.key[0, n), 0 < n <= kSortMax; key i is left at s.key[pad8(i)]
+// (over the bins).  Every thread sorts 8 keys in registers (Batcher's odd-even
+// merge network), then pairs of runs are merged, every thread 8 outputs from
+// their merge-path start, read into registers before any is stored.  Every
+// thread of the CTA calls it after a barrier; it ends with one.
+__device__ __noinline__ void smem_merge(SortSmem& s, uint32_t n) {
+  const uint32_t t = threadIdx.x, rows = (n + 7) / 8, N = 8 * rows;
+  unsigned long long* const buf = s.key;
+  unsigned long long k[8];
+#pragma unroll
+  for (int r = 0; r < 8; ++r) k[r] = t < rows && t + r * rows < n ? buf[t + r * rows] : ~0ull;
+  cas_reg(k[0], k[1]); cas_reg(k[2], k[3]); cas_reg(k[4], k[5]); cas_reg(k[6], k[7]);
+  cas_reg(k[0], k[2]); cas_reg(k[1], k[3]); cas_reg(k[4], k[6]); cas_reg(k[5], k[7]);
+  cas_reg(k[1], k[2]); cas_reg(k[5], k[6]);
+  cas_reg(k[0], k[4]); cas_reg(k[1], k[5]); cas_reg(k[2], k[6]); cas_reg(k[3], k[7]);
+  cas_reg(k[2], k[4]); cas_reg(k[3], k[5]);
+  cas_reg(k[1], k[2]); cas_reg(k[3], k[4]); cas_reg(k[5], k[6]);
+  __syncthreads();
+  if (t < rows)
+#pragma unroll
+    for (int r = 0; r < 8; ++r) buf[9 * t + r] = k[r];
+  for (uint32_t L = 8; L < N; L <<= 1) {
+    // (up to L = 128 the threads of a pair of runs are of one warp)
+    if (L <= 128) __syncwarp();
+    else __syncthreads();
+    if (t < rows) {
+      const uint32_t d = 8 * t & (2 * L - 1);   // first output in the pair
+      const uint32_t a0 = 8 * t - d, b0 = a0 + L;
+      const uint32_t la = min(L, N - a0), lb = b0 < N ? min(L, N - b0) : 0u;
+      uint32_t lo = d > lb ? d - lb : 0u, hi = d < la ? d : la;
+      while (lo < hi) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (buf[pad8(a0 + mid)] > buf[pad8(b0 + d - mid - 1)]) hi = mid;
+        else lo = mid + 1;
+      }
+      uint32_t i = lo, j = d - lo;
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        // (ties, which only the padding has, go to the first run, as in the search)
+        const unsigned long long a = i < la ? buf[pad8(a0 + i)] : ~0ull, b = j < lb ? buf[pad8(b0 + j)] : ~0ull;
+        const bool first = j >= lb || (i < la && a <= b);
+        k[r] = first ? a : b;
+        i += first;
+        j += !first;
+      }
+    }
+    if (L <= 128) __syncwarp();
+    else __syncthreads();
+    if (t < rows)
+#pragma unroll
+      for (int r = 0; r < 8; ++r) buf[9 * t + r] = k[r];
+  }
+  __syncthreads();
+}
+
 // The n <= kSortMax keys get(0) .. get(n - 1) sorted, their items written to
 // out (get may read what out overwrites: every key is read first).  Called by
 // the whole CTA; the caller separates two calls by a barrier.
-template <class Get>
+template <bool MERGE, class Get>
 __device__ __forceinline__ void sort_small(const Get& get, uint32_t n, uint32_t* out, SortSmem& s) {
   const uint32_t t = threadIdx.x;
   const int wid = t >> 5;
@@ -810,8 +880,12 @@ __device__ __forceinline__ void sort_small(const Get& get, uint32_t n, uint32_t*
     if (r * kSortCta + t < n) s.key[s.fine[fo[r] & 0xffffu] + (fo[r] >> 16)] = k[r];
   __syncthreads();
   if (dense) {
-    smem_bitonic(s.key, n);
-    for (uint32_t i = t; i < n; i += kSortCta) out[i] = static_cast<uint32_t>(s.key[i]);
+    // (MERGE: in the tiles' kernel; the groups' one would need more registers
+    // for it, 5 % of six batched maps' step)
+    const bool merge = MERGE && n > kBitonicMax;
+    if (merge) smem_merge(s, n);
+    else smem_bitonic(s.key, n);
+    for (uint32_t i = t; i < n; i += kSortCta) out[i] = static_cast<uint32_t>(s.key[merge ? pad8(i) : i]);
     return;
   }
   for (uint32_t i = t; i < n; i += kSortCta) {
@@ -827,7 +901,7 @@ __device__ __forceinline__ void sort_small(const Get& get, uint32_t n, uint32_t*
 
 // ---- buckets beyond 2048 keys: partitioned into groups ------------------------
 // k_long_split: one CTA takes a bucket (claimed in the tile scan's
-// longest-first order).  The depth map above with kLongCoarse bins estimates
+// longest-first order).  A depth map like the one above with kLongCoarse bins estimates
 // every key's rank, and the keys of one group of 2^sh estimated ranks (1,024,
 // more beyond 2 M keys) are scattered to one range of a second key buffer made
 // of the pair-tile and item arrays (high and low 32 bits; the pair tiles are
@@ -837,9 +911,15 @@ __device__ __forceinline__ void sort_small(const Get& get, uint32_t n, uint32_t*
 // it is spread over the chip; one CTA per bucket, merging chunks through
 // global memory, was bound by the longest bucket's serial passes (6 maps with
 // buckets up to 292 k keys, 28.9 M long keys: 3.49 -> 0.58 + 0.27 ms; 8
-// keyframes of a 1M map, 25.6 M long keys: 1.04 -> 0.18 + 0.25 ms).  A group of more than kSortMax keys (depths
-// that cluster far below a bin's width) is sorted by its CTA with sorted
-// chunks and merge passes through global memory.
+// keyframes of a 1M map, 25.6 M long keys: 1.04 -> 0.18 + 0.25 ms).
+// A group of more than kSortMax keys (depths that cluster far below a bin's
+// width, a smooth wall in a bucket with a near and a far surfel, or equal ones)
+// is partitioned once more, by the same CTA, with its own range of (depth, item).
+// What then still exceeds kSortMax (clusters
+// within clusters) is sorted by its CTA with sorted chunks and merge passes
+// through global memory.  (10,000 keys on a wall with 1 mm of noise between a near
+// and a far surfel, the binning: 202 us when the large groups were merged, 79 with
+// one CTA per bucket, now 57; 300,000 equal depths 7.8, 3.1 and 0.75 ms.)
 constexpr int kLongCta = 1024;
 constexpr uint32_t kLongCoarse = 2048;
 constexpr uint32_t kMaxGroups = 2048;
@@ -966,16 +1046,25 @@ struct SegPlan {
   uint32_t blocks;   // warp blocks per tile
 };
 
-// fn(key) for the n keys X[0, n) in turn, four loads in flight per thread.
+// fn(key) for n keys in turn, four loads in flight per thread.
 template <class Fn>
-__device__ __forceinline__ void for_keys(const unsigned long long* __restrict__ X, uint32_t n, Fn fn) {
+__device__ __forceinline__ void for_keys(const unsigned long long* X, uint32_t n, Fn fn) {
   for (uint32_t i0 = threadIdx.x; i0 < n; i0 += 4 * kLongCta) {
     unsigned long long x[4];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) x[u] = i0 + u * kLongCta < n ? __ldg(X + i0 + u * kLongCta) : 0ull;
+    for (int u = 0; u < 4; ++u) x[u] = i0 + u * kLongCta < n ? X[i0 + u * kLongCta] : 0ull;
 #pragma unroll
     for (int u = 0; u < 4; ++u)
       if (i0 + u * kLongCta < n) fn(x[u]);
+  }
+}
+
+template <class Fn>
+__device__ __forceinline__ void for_keys(const KeyBuf& Y, uint32_t n, Fn fn) {
+  for (uint32_t i0 = threadIdx.x; i0 < n; i0 += 2 * kLongCta) {
+    const unsigned long long a = Y.get(i0), b = i0 + kLongCta < n ? Y.get(i0 + kLongCta) : 0ull;
+    fn(a);
+    if (i0 + kLongCta < n) fn(b);
   }
 }
 
@@ -1039,37 +1128,170 @@ __device__ void plan_segments(const uint2* __restrict__ ranges, Status* __restri
   __syncthreads();
 }
 
+// Bins of the values above `base` (those below count as base, those beyond the
+// last bin as its end), monotone in the value: rounded conversion and product.
+template <class V>
+struct Bins {
+  V base;
+  float scale;
+  __device__ __forceinline__ uint32_t bin(V v, float& frac) const {
+    const float x = fmul(static_cast<float>(max(v, base) - base), scale);
+    const uint32_t c = min(static_cast<uint32_t>(x), kLongCoarse - 1u);
+    frac = fsub(x, static_cast<float>(c));
+    return c;
+  }
+  // Estimated rank from the bins' exclusive counts: monotone in v.
+  __device__ __forceinline__ uint32_t rank(V v, const uint32_t* start) const {
+    float frac;
+    const uint32_t c = bin(v, frac);
+    const uint32_t b = start[c], m = start[c + 1] - b;
+    return b + min(static_cast<uint32_t>(fmul(frac, static_cast<float>(m))), m - 1u);
+  }
+  __device__ __forceinline__ bool wide() const { return scale < 0.25f; }   // more than four values a bin
+  // All bins over the range of bin c (and a little more: the bounds are rounded).
+  __device__ __forceinline__ void narrow(uint32_t c) {
+    const float width = 1.0f / scale;
+    base += static_cast<V>(fmaxf((static_cast<float>(c) - 0.02f) * width, 0.0f));
+    scale = static_cast<float>(kLongCoarse) / (1.04f * width + 1.0f);
+  }
+};
+
+template <class V>
+__device__ __forceinline__ Bins<V> bins_over(V lo, V hi) {
+  return Bins<V>{lo, static_cast<float>(kLongCoarse) / (static_cast<float>(hi - lo) + 1.0f)};
+}
+
+struct SplitSmem {
+  uint32_t hist[2 * kLongCta];       // counts per bin, then per group, then group cursors
+  uint32_t start[kLongCoarse + 2];   // the keys before each bin
+  uint32_t w[32], mm[4], claim, at, next;
+};
+
+// One partition of n keys: each(fn) calls fn(value, key) for all of them, the
+// bins estimate ranks, and the keys of one group of 2^sh estimated ranks go to
+// one range: put(place, key).  While one bin holds most keys, the bins are
+// spread over its range alone.  Gives the thread's groups 2t and 2t + 1: their
+// counts, and first places (to `early`, before the keys move).  hist is zero on
+// entry.
+template <class V, class Each, class Early, class Put>
+__device__ __forceinline__ void partition(const Each& each, Bins<V> bins, uint32_t n, uint32_t sh, SplitSmem& s,
+                                          uint2& c, const Early& early, const Put& put) {
+  const uint32_t t = threadIdx.x;
+  while (true) {
+    each([&](V v, unsigned long long) {
+      float frac;
+      atomicAdd(&s.hist[bins.bin(v, frac)], 1u);
+    });
+    __syncthreads();
+    c = make_uint2(s.hist[2 * t], s.hist[2 * t + 1]);
+    // (every round narrows the range by more than a thousand times)
+    if (!__syncthreads_or(max(c.x, c.y) > n / 2) || !bins.wide()) break;
+    if (max(c.x, c.y) > n / 2) s.next = 2 * t + (c.y > c.x);
+    s.hist[2 * t] = s.hist[2 * t + 1] = 0u;
+    __syncthreads();
+    bins.narrow(s.next);
+  }
+  const uint2 first = long_exclusive(c, s.w);
+  s.start[2 * t] = first.x;
+  s.start[2 * t + 1] = first.y;
+  if (t == 0) s.start[kLongCoarse] = n;
+  s.hist[2 * t] = s.hist[2 * t + 1] = 0u;   // (every thread has read its own counts only)
+  __syncthreads();
+  each([&](V v, unsigned long long) { atomicAdd(&s.hist[bins.rank(v, s.start) >> sh], 1u); });
+  __syncthreads();
+  c = make_uint2(s.hist[2 * t], s.hist[2 * t + 1]);
+  const uint2 at = long_exclusive(c, s.w);
+  s.hist[2 * t] = at.x;
+  s.hist[2 * t + 1] = at.y;
+  early(at);
+  __syncthreads();
+  each([&](V v, unsigned long long x) { put(atomicAdd(&s.hist[bins.rank(v, s.start) >> sh], 1u), x); });
+}
+
+__device__ __forceinline__ uint32_t group_shift(uint32_t n) {
+  uint32_t sh = kGroupBits;
+  while (((n - 1) >> sh) >= kMaxGroups) ++sh;
+  return sh;
+}
+
+// The second partition, of the n keys at `first` of the split buffer (through the
+// key array, which the first one is done with): by (depth, item) as one number,
+// the depths above the lowest times the items' span plus the item, so that
+// equal depths spread by item.
+__device__ __noinline__ void split_again(uint32_t first, uint32_t n, unsigned long long* pkey, uint32_t* ptile,
+                                         uint32_t* pv, uint2* groups, Status* st, SplitSmem& s) {
+  const uint32_t t = threadIdx.x;
+  const KeyBuf Y{nullptr, ptile + first, pv + first};
+  if (t < 4) s.mm[t] = t & 1u ? 0u : ~0u;
+  s.hist[2 * t] = s.hist[2 * t + 1] = 0u;
+  __syncthreads();
+  uint32_t dlo = ~0u, dhi = 0u, ilo = ~0u, ihi = 0u;
+  for_keys(Y, n, [&](unsigned long long x) {
+    dlo = min(dlo, static_cast<uint32_t>(x >> 32));
+    dhi = max(dhi, static_cast<uint32_t>(x >> 32));
+    ilo = min(ilo, static_cast<uint32_t>(x));
+    ihi = max(ihi, static_cast<uint32_t>(x));
+  });
+  dlo = __reduce_min_sync(0xffffffffu, dlo);
+  dhi = __reduce_max_sync(0xffffffffu, dhi);
+  ilo = __reduce_min_sync(0xffffffffu, ilo);
+  ihi = __reduce_max_sync(0xffffffffu, ihi);
+  if ((t & 31) == 0) {
+    atomicMin(&s.mm[0], dlo);
+    atomicMax(&s.mm[1], dhi);
+    atomicMin(&s.mm[2], ilo);
+    atomicMax(&s.mm[3], ihi);
+  }
+  __syncthreads();
+  dlo = s.mm[0];
+  ilo = s.mm[2];
+  const unsigned long long span = static_cast<unsigned long long>(s.mm[3] - ilo) + 1ull;
+  const unsigned long long most = (s.mm[1] - dlo) * span + (span - 1ull);
+  const uint32_t sh = group_shift(n), n_groups = ((n - 1) >> sh) + 1;
+  if (t == 0) s.at = atomicAdd(&st->n_groups, n_groups);
+  uint2 c;
+  partition([&](auto fn) {
+              for_keys(Y, n, [&](unsigned long long x) {
+                fn((static_cast<uint32_t>(x >> 32) - dlo) * span + (static_cast<uint32_t>(x) - ilo), x);
+              });
+            },
+            bins_over(0ull, most), n, sh, s, c,
+            [&](uint2 at) {
+              if (2 * t < n_groups) groups[s.at + 2 * t] = make_uint2(first + at.x, first + at.x + c.x);
+              if (2 * t + 1 < n_groups) groups[s.at + 2 * t + 1] = make_uint2(first + at.y, first + at.y + c.y);
+            },
+            [&](uint32_t pos, unsigned long long x) { pkey[first + pos] = x; });
+  __syncthreads();
+  for (uint32_t i = t; i < n; i += kLongCta) Y.put(i, __ldcg(pkey + first + i));
+}
+
 __global__ void __launch_bounds__(kLongCta, 2)
     k_long_split(const uint2* __restrict__ ranges, Status* __restrict__ st, const uint32_t* __restrict__ order,
-                 uint32_t n_tiles, const unsigned long long* __restrict__ pkey, uint32_t* __restrict__ ptile,
-                 uint32_t* __restrict__ pv, uint2* __restrict__ groups, SegPlan plan) {
+                 uint32_t n_tiles, unsigned long long* pkey, uint32_t* ptile, uint32_t* pv,
+                 uint2* __restrict__ groups, SegPlan plan) {
   pdl_launch_dependents();  // the next kernel may be dispatched now
-  __shared__ uint32_t s_hist[2 * kLongCta];     // counts per bin, then per group, then group cursors
-  __shared__ uint32_t s_start[kLongCoarse + 2]; // the bucket's keys before each bin
-  __shared__ uint32_t s_w[32], s_mm[2], s_claim, s_at;
+  __shared__ SplitSmem s;
   if (st->overflow || st->n_big == 0) return;
   const uint32_t t = threadIdx.x;
-  if (blockIdx.x == gridDim.x - 1 && st->n_long) plan_segments(ranges, st, plan, s_hist, s_w);
+  if (blockIdx.x == gridDim.x - 1 && st->n_long) plan_segments(ranges, st, plan, s.hist, s.w);
   while (true) {
     // buckets in the tile scan's longest-first order; the long ones come
     // first, so the first list of a shorter class ends the work
     __syncthreads();
     if (t == 0) {
-      s_claim = atomicAdd(&st->long_sort_counter, 1u);
-      s_mm[0] = ~0u;
-      s_mm[1] = 0u;
+      s.claim = atomicAdd(&st->long_sort_counter, 1u);
+      s.mm[0] = ~0u;
+      s.mm[1] = 0u;
     }
-    s_hist[2 * t] = s_hist[2 * t + 1] = 0u;
+    s.hist[2 * t] = s.hist[2 * t + 1] = 0u;
     __syncthreads();
-    const uint32_t k = s_claim;
+    const uint32_t k = s.claim;
     if (k >= n_tiles) return;
     const uint2 rg = ranges[order[k]];
     const uint32_t n = rg.y - rg.x;
     if (order_bucket(n) > order_bucket(kSortMax + 1)) return;   // a shorter class: no long list follows
     if (n <= kSortMax) continue;
-    uint32_t sh = kGroupBits;
-    while (((n - 1) >> sh) >= kMaxGroups) ++sh;
-    const uint32_t n_groups = ((n - 1) >> sh) + 1;
+    const uint32_t sh = group_shift(n), n_groups = ((n - 1) >> sh) + 1;
     const unsigned long long* X = pkey + rg.x;
     // the bucket's depth range
     uint32_t lo = ~0u, hi = 0u;
@@ -1080,39 +1302,50 @@ __global__ void __launch_bounds__(kLongCta, 2)
     lo = __reduce_min_sync(0xffffffffu, lo);
     hi = __reduce_max_sync(0xffffffffu, hi);
     if ((t & 31) == 0) {
-      atomicMin(&s_mm[0], lo);
-      atomicMax(&s_mm[1], hi);
+      atomicMin(&s.mm[0], lo);
+      atomicMax(&s.mm[1], hi);
     }
+    if (t == 0) s.at = atomicAdd(&st->n_groups, n_groups);
     __syncthreads();
-    const DepthMap map(s_mm[0], s_mm[1], kLongCoarse);
-    for_keys(X, n, [&](unsigned long long x) {
-      float frac;
-      atomicAdd(&s_hist[map.bin(static_cast<uint32_t>(x >> 32), frac)], 1u);
-    });
-    __syncthreads();
-    const uint2 first = long_exclusive(make_uint2(s_hist[2 * t], s_hist[2 * t + 1]), s_w);
-    s_start[2 * t] = first.x;
-    s_start[2 * t + 1] = first.y;
-    if (t == 0) s_start[kLongCoarse] = n;
-    s_hist[2 * t] = s_hist[2 * t + 1] = 0u;   // (every thread has read its own counts only)
-    __syncthreads();
-    for_keys(X, n, [&](unsigned long long x) {
-      atomicAdd(&s_hist[map.rank(static_cast<uint32_t>(x >> 32), s_start) >> sh], 1u);
-    });
-    __syncthreads();
-    const uint2 c = make_uint2(s_hist[2 * t], s_hist[2 * t + 1]);
-    const uint2 at = long_exclusive(c, s_w);
-    s_hist[2 * t] = at.x;
-    s_hist[2 * t + 1] = at.y;
-    if (t == 0) s_at = atomicAdd(&st->n_groups, n_groups);
-    __syncthreads();
-    if (2 * t < n_groups) groups[s_at + 2 * t] = make_uint2(rg.x + at.x, rg.x + at.x + c.x);
-    if (2 * t + 1 < n_groups) groups[s_at + 2 * t + 1] = make_uint2(rg.x + at.y, rg.x + at.y + c.y);
-    for_keys(X, n, [&](unsigned long long x) {
-      const uint32_t pos = rg.x + atomicAdd(&s_hist[map.rank(static_cast<uint32_t>(x >> 32), s_start) >> sh], 1u);
-      ptile[pos] = static_cast<uint32_t>(x >> 32);
-      pv[pos] = static_cast<uint32_t>(x);
-    });
+    uint2 c;
+    partition([&](auto fn) {
+                for_keys(X, n, [&](unsigned long long x) { fn(static_cast<uint32_t>(x >> 32), x); });
+              },
+              bins_over(s.mm[0], s.mm[1]), n, sh, s, c,
+              [&](uint2 at) {
+                // (an empty range where split_again stores the groups instead)
+                const uint2 e = make_uint2(c.x > kSortMax ? 0u : c.x, c.y > kSortMax ? 0u : c.y);
+                if (2 * t < n_groups) groups[s.at + 2 * t] = make_uint2(rg.x + at.x, rg.x + at.x + e.x);
+                if (2 * t + 1 < n_groups) groups[s.at + 2 * t + 1] = make_uint2(rg.x + at.y, rg.x + at.y + e.y);
+              },
+              [&](uint32_t pos, unsigned long long x) {
+                ptile[rg.x + pos] = static_cast<uint32_t>(x >> 32);
+                pv[rg.x + pos] = static_cast<uint32_t>(x);
+              });
+    // the groups of more than kSortMax keys, one after the other
+    if (__syncthreads_or(c.x > kSortMax || c.y > kSortMax)) {
+      // (a group's cursor now stands at its end)
+      const uint2 end = make_uint2(s.hist[2 * t], s.hist[2 * t + 1]);
+      for (uint32_t from = 0;;) {
+        __syncthreads();
+        if (t == 0) s.next = ~0u;
+        __syncthreads();
+        if (c.y > kSortMax && 2 * t + 1 >= from) atomicMin(&s.next, 2 * t + 1);
+        if (c.x > kSortMax && 2 * t >= from) atomicMin(&s.next, 2 * t);
+        __syncthreads();
+        const uint32_t g = s.next;
+        if (g == ~0u) break;
+        if (t == g / 2) {
+          s.mm[0] = g & 1u ? c.y : c.x;
+          s.mm[1] = g & 1u ? end.y : end.x;
+        }
+        __syncthreads();
+        const uint32_t m = s.mm[0], e = s.mm[1];
+        __syncthreads();
+        split_again(rg.x + e - m, m, pkey, ptile, pv, groups, st, s);
+        from = g + 1;
+      }
+    }
   }
 }
 
@@ -1132,18 +1365,18 @@ __global__ void __launch_bounds__(kSortCta) k_tile_sort(const uint2* __restrict_
     const uint2 rg = ranges[blockIdx.x];
     const uint32_t n = rg.y - rg.x;
     if (n == 0 || n > kSortMax) return;   // empty, or k_long_split's
-    sort_small([&](uint32_t i) { return pkey[rg.x + i]; }, n, pv + rg.x, s);
+    sort_small<true>([&](uint32_t i) { return pkey[rg.x + i]; }, n, pv + rg.x, s);
     return;
   }
   if (!GROUPS) return;
-  const uint32_t first = TILES ? n_tiles : 0u, n_groups = st->n_groups;
-  for (uint32_t g = blockIdx.x - first; g < n_groups; g += gridDim.x - first) {
+  const uint32_t cta0 = TILES ? n_tiles : 0u, n_groups = st->n_groups;
+  for (uint32_t g = blockIdx.x - cta0; g < n_groups; g += gridDim.x - cta0) {
     const uint2 rg = groups[g];
     const uint32_t n = rg.y - rg.x;
     const KeyBuf Y{nullptr, ptile + rg.x, pv + rg.x};
     __syncthreads();   // the previous group's shared memory is no longer read
     if (n == 0) continue;
-    if (n <= kSortMax) sort_small([&](uint32_t i) { return Y.get(i); }, n, Y.lo, s);
+    if (n <= kSortMax) sort_small<false>([&](uint32_t i) { return Y.get(i); }, n, Y.lo, s);
     else merge_sort_global(KeyBuf{pkey + rg.x, nullptr, nullptr}, Y, n, s);
   }
 }

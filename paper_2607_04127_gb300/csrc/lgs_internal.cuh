@@ -155,7 +155,7 @@ struct WsPtrs {
   float* ssuf;             // [segments][tile pixels] the suffix of the later segments (backward)
   uint32_t* dead;          // [long lists][tile pixels] first segment known to stop the pixel (~0 between forwards)
   uint32_t* cmask;         // [chunks][4 windows][tile pixels] entries each pixel composited, one bit per entry
-  uint2* groups;           // [pairs / 512 + 1] ranges of the long buckets' groups (st->n_groups of them)
+  uint2* groups;           // [pairs / 256 + 1] ranges of the long buckets' groups (st->n_groups of them)
   uint32_t* bwm;           // [tiles][warp blocks] the block's largest n_contrib, 0 outside the frame.  Every forward that
                            // the chunked backward may follow sets every word: k_fwd_s those of tiles with short
                            // lists, k_long_masks (0) and k_fwd_long (the maximum) those of long ones
