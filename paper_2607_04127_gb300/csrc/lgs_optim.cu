@@ -399,8 +399,8 @@ cudaError_t launch_loss(const Layout&, const WsPtrs& w, const Desc& h, const lgs
 }
 
 // Before a forward with the image-loss epilogue: the mask counts (the
-// epilogue normalises by them) and the scale regulariser; the forward's
-// long-list kernel writes the loss vector when every pixel is done.  Also
+// epilogue normalises by them) and the scale regulariser; the last CTA of the
+// forward's tile kernel writes the loss vector when every pixel is done.  Also
 // zeroes the forward's tile counter.
 cudaError_t launch_loss_counts(const WsPtrs& w, const Desc& h, const lgs_loss_params& p, bool scale_grad,
                                cudaStream_t s) {
@@ -483,10 +483,13 @@ __device__ __forceinline__ void adam_group(float* __restrict__ p, float* __restr
   }
 }
 
-// CTAs per parameter group of n scalars: 1,024 scalars each, at most eight CTAs
-// per SM
+// CTAs of each parameter group (a launch has four groups a map): 1,024 scalars
+// each up to eight CTAs per SM and group, several rounds beyond
 static unsigned adam_ctas(int64_t n) {
-  return static_cast<unsigned>(std::min<int64_t>(std::max<int64_t>((n + 1023) / 1024, 1), 8 * 152));
+  int dev = 0, sms = 152;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return static_cast<unsigned>(std::min<int64_t>(std::max<int64_t>((n + 1023) / 1024, 1), 8 * sms));
 }
 
 __global__ void __launch_bounds__(256) k_adam(AdamSeg a, float b1, float b2, float eps, float c1, float c2,
