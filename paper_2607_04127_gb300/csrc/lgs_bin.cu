@@ -406,6 +406,8 @@ constexpr uint32_t kLenCache = 4096;   // tiles whose list length the scan keeps
 // longer ones split into groups first (k_long_split), in this longest-first
 // order.
 constexpr uint32_t kSortMax = 2048;
+// Buckets of up to kWarpSort keys are sorted by one warp.
+constexpr uint32_t kWarpSort = 64;
 constexpr int kOrderBuckets = 33;
 __device__ __forceinline__ int order_bucket(uint32_t n) { return kOrderBuckets - 1 - (n ? 32 - __clz(n) : 0); }
 
@@ -1249,7 +1251,7 @@ __device__ __noinline__ void split_again(uint32_t first, uint32_t n, unsigned lo
   const unsigned long long most = (s.mm[1] - dlo) * span + (span - 1ull);
   const uint32_t sh = group_shift(n), n_groups = ((n - 1) >> sh) + 1;
   if (t == 0) s.at = atomicAdd(&st->n_groups, n_groups);
-  uint2 c;
+  uint2 c = make_uint2(0u, 0u);
   partition([&](auto fn) {
               for_keys(Y, n, [&](unsigned long long x) {
                 fn((static_cast<uint32_t>(x >> 32) - dlo) * span + (static_cast<uint32_t>(x) - ilo), x);
@@ -1307,7 +1309,7 @@ __global__ void __launch_bounds__(kLongCta, 2)
     }
     if (t == 0) s.at = atomicAdd(&st->n_groups, n_groups);
     __syncthreads();
-    uint2 c;
+    uint2 c = make_uint2(0u, 0u);
     partition([&](auto fn) {
                 for_keys(X, n, [&](unsigned long long x) { fn(static_cast<uint32_t>(x >> 32), x); });
               },
@@ -1349,28 +1351,66 @@ __global__ void __launch_bounds__(kLongCta, 2)
   }
 }
 
-// TILES: CTAs below n_tiles take the bucket of their tile, if it has at most
-// kSortMax keys.  GROUPS: the CTAs after them take the long buckets' groups
-// (their keys in the split buffer) in turn.  (One kernel for both needs more
-// registers than the tiles alone: street frame 18 against 28 us.)
+// A bucket of n <= kWarpSort keys sorted by one warp, kWarpKeys keys a lane: a
+// key's place is the number of smaller ones.
+constexpr int kWarpKeys = kWarpSort / 32;
+__device__ __forceinline__ void sort_warp(const unsigned long long* key, uint32_t n, uint32_t* out) {
+  const uint32_t lane = threadIdx.x & 31;
+  unsigned long long k[kWarpKeys];
+  uint32_t rank[kWarpKeys];
+#pragma unroll
+  for (int q = 0; q < kWarpKeys; ++q) {
+    k[q] = lane + 32 * q < n ? key[lane + 32 * q] : ~0ull;
+    rank[q] = 0;
+  }
+#pragma unroll
+  for (int p = 0; p < kWarpKeys; ++p)
+    for (uint32_t j = 0; j < 32 && j + 32 * p < n; ++j) {
+      const unsigned long long x = __shfl_sync(0xffffffffu, k[p], j);
+#pragma unroll
+      for (int q = 0; q < kWarpKeys; ++q) rank[q] += x < k[q];
+    }
+#pragma unroll
+  for (int q = 0; q < kWarpKeys; ++q)
+    if (lane + 32 * q < n) out[rank[q]] = static_cast<uint32_t>(k[q]);
+}
+
+// TILES: CTAs below n_tiles take the bucket of their tile, if it has more than
+// kWarpSort and at most kSortMax keys; a warp of the next tiles / 8 CTAs each that
+// of its tile, if it has fewer (with a CTA for every tile, a frame of few surfels
+// was bound by 2,048 CTAs' barriers over a few keys each: 3,000 surfels on a
+// 128 x 1024 frame, the binning 47 us, now 35; on four 146 without the inline path,
+// now 130; warps up to 128 keys 2 us slower from 16,000 surfels on).  GROUPS: the
+// CTAs after them take the long buckets' groups (their keys in the split buffer)
+// in turn.  Both in one kernel take 106 registers, the tiles alone 60, so that one
+// is held at 64 (street frame, 16,000 surfels, the binning 49 us, now 40).
+constexpr uint32_t kSortWarps = kSortCta / 32;
+static unsigned tile_sort_ctas(uint32_t n_tiles) { return n_tiles + (n_tiles + kSortWarps - 1) / kSortWarps; }
 template <bool TILES, bool GROUPS>
-__global__ void __launch_bounds__(kSortCta) k_tile_sort(const uint2* __restrict__ ranges,
+__global__ void __launch_bounds__(kSortCta, TILES && GROUPS ? 4 : 0) k_tile_sort(const uint2* __restrict__ ranges,
                                                          const Status* __restrict__ st, uint32_t n_tiles,
                                                          unsigned long long* pkey, uint32_t* ptile, uint32_t* pv,
                                                          const uint2* __restrict__ groups) {
   if (GROUPS) pdl_wait();   // (launched after k_long_split: wait for it)
   __shared__ SortSmem s;
   if (st->overflow) return;
-  if (TILES && (!GROUPS || blockIdx.x < n_tiles)) {
-    const uint2 rg = ranges[blockIdx.x];
+  const uint32_t tile_ctas = TILES ? n_tiles + (n_tiles + kSortWarps - 1) / kSortWarps : 0u;
+  if (TILES && (!GROUPS || blockIdx.x < tile_ctas)) {
+    const bool own = blockIdx.x < n_tiles;
+    const uint32_t tile = own ? blockIdx.x : (blockIdx.x - n_tiles) * kSortWarps + (threadIdx.x >> 5);
+    if (tile >= n_tiles) return;
+    const uint2 rg = ranges[tile];
     const uint32_t n = rg.y - rg.x;
-    if (n == 0 || n > kSortMax) return;   // empty, or k_long_split's
-    sort_small<true>([&](uint32_t i) { return pkey[rg.x + i]; }, n, pv + rg.x, s);
+    if (!own) {
+      if (n <= kWarpSort) sort_warp(pkey + rg.x, n, pv + rg.x);
+    } else if (n > kWarpSort && n <= kSortMax) {   // (longer: k_long_split's)
+      sort_small<true>([&](uint32_t i) { return pkey[rg.x + i]; }, n, pv + rg.x, s);
+    }
     return;
   }
   if (!GROUPS) return;
-  const uint32_t cta0 = TILES ? n_tiles : 0u, n_groups = st->n_groups;
-  for (uint32_t g = blockIdx.x - cta0; g < n_groups; g += gridDim.x - cta0) {
+  const uint32_t n_groups = st->n_groups;
+  for (uint32_t g = blockIdx.x - tile_ctas; g < n_groups; g += gridDim.x - tile_ctas) {
     const uint2 rg = groups[g];
     const uint32_t n = rg.y - rg.x;
     const KeyBuf Y{nullptr, ptile + rg.x, pv + rg.x};
@@ -1400,11 +1440,13 @@ cudaError_t launch_fill_tile_of_pair(const WsPtrs& w, uint32_t n_tiles, cudaStre
 // ---------------------------------------------------------------------------
 // How the long buckets (more than kSortMax keys) are sorted, by the largest
 // map of the call.  None can arise up to kSortMax surfels.  From kSideItems
-// surfels on, k_long_split and the groups' sort run on the side stream
-// alongside the short buckets' sort (1M surfels, 8 keyframes: 0.43 ms beside
-// 0.11); below, long buckets are few and the fork and join would cost a small
-// frame, which the host's launches bound, more (2,000-surfel room, bin and
-// forward: 53 us with them, 37 to 43 us without).
+// surfels on, k_long_split and the groups' sort run on the side stream alongside
+// the short buckets' sort; below, inline, without the fork and join that the host
+// has to issue.  Binning, inline and side: 3,000 surfels on a 64 x 1024 frame
+// 30.9 and 34.6 us, 8,000 32.6 and 34.8, 32,000 34.3 and 35.3, 64,000 36.5 and
+// 36.4; on a 128 x 1024 frame 35.0 / 36.3, 37.0 / 37.2, 43.4 / 43.1, 44.3 / 45.0;
+// four such frames of 125,000 surfels 322 and 318; 1M surfels, 8 keyframes 0.43 ms
+// of long buckets beside 0.11.
 constexpr int64_t kSideItems = 32768;
 enum LongPath { kLongNone, kLongInline, kLongSide };
 static LongPath long_path(int64_t max_n) {
@@ -1450,11 +1492,11 @@ cudaError_t launch_bin(const Layout& L, const WsPtrs& w, int n_frames, int64_t n
       k_long_split<<<2 * sms, kLongCta, 0, s>>>(w.ranges, w.st, w.work, n_tiles, w.pkey, w.ptile, w.pv, w.groups,
                                                   plan);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
-      return launch_dep(k_tile_sort<true, true>, dim3(n_tiles + group_ctas), dim3(kSortCta), 0, s, w.ranges, w.st,
+      return launch_dep(k_tile_sort<true, true>, dim3(tile_sort_ctas(n_tiles) + group_ctas), dim3(kSortCta), 0, s, w.ranges, w.st,
                         n_tiles, w.pkey, w.ptile, w.pv, w.groups);
     }
     if (path == kLongSide && (e = cudaEventRecord(side.fork, s)) != cudaSuccess) return e;
-    k_tile_sort<true, false><<<n_tiles, kSortCta, 0, s>>>(w.ranges, w.st, n_tiles, w.pkey, w.ptile, w.pv, w.groups);
+    k_tile_sort<true, false><<<tile_sort_ctas(n_tiles), kSortCta, 0, s>>>(w.ranges, w.st, n_tiles, w.pkey, w.ptile, w.pv, w.groups);
     if ((e = cudaGetLastError()) != cudaSuccess || path == kLongNone) return e;
     // (the side stream has the higher priority: its CTAs take the slots that
     // short buckets free, and the launches do not delay the short buckets)
