@@ -1375,26 +1375,28 @@ __device__ __forceinline__ void sort_warp(const unsigned long long* key, uint32_
     if (lane + 32 * q < n) out[rank[q]] = static_cast<uint32_t>(k[q]);
 }
 
-// TILES: CTAs below n_tiles take the bucket of their tile, if it has more than
-// kWarpSort and at most kSortMax keys; a warp of the next tiles / 8 CTAs each that
-// of its tile, if it has fewer (with a CTA for every tile, a frame of few surfels
-// was bound by 2,048 CTAs' barriers over a few keys each: 3,000 surfels on a
-// 128 x 1024 frame, the binning 47 us, now 35; on four 146 without the inline path,
-// now 130; warps up to 128 keys 2 us slower from 16,000 surfels on).  GROUPS: the
-// CTAs after them take the long buckets' groups (their keys in the split buffer)
-// in turn.  Both in one kernel take 106 registers, the tiles alone 60, so that one
-// is held at 64 (street frame, 16,000 surfels, the binning 49 us, now 40).
+// TILES: CTAs below n_tiles take the bucket of their tile, if it has at most
+// kSortMax keys.  In a sparse call (below kSparse items a tile) they leave buckets
+// of up to kWarpSort keys to a warp each of n_warp more CTAs: with a CTA for every
+// tile, a frame of few surfels was bound by 2,048 CTAs' barriers over a few keys
+// each.  Binning of a 128 x 1024 frame, without and with the warps: 3,000 surfels 47
+// and 35 us; 16,000 49 and 40; 64,000 (31 items a tile) 43.8 and 44.1; 200,000 55.9
+// and 57.5;
+// warps up to 128 keys were 2 us slower from 16,000 surfels on.  GROUPS: the CTAs
+// after them take the long buckets' groups (their keys in the split buffer) in
+// turn.  Both in one kernel take 106 registers, the tiles alone 60, so that one is
+// held at 64 (16,000 surfels 49 us on 106).
 constexpr uint32_t kSortWarps = kSortCta / 32;
-static unsigned tile_sort_ctas(uint32_t n_tiles) { return n_tiles + (n_tiles + kSortWarps - 1) / kSortWarps; }
+constexpr int64_t kSparse = 32;
 template <bool TILES, bool GROUPS>
 __global__ void __launch_bounds__(kSortCta, TILES && GROUPS ? 4 : 0) k_tile_sort(const uint2* __restrict__ ranges,
                                                          const Status* __restrict__ st, uint32_t n_tiles,
-                                                         unsigned long long* pkey, uint32_t* ptile, uint32_t* pv,
-                                                         const uint2* __restrict__ groups) {
+                                                         uint32_t n_warp, unsigned long long* pkey, uint32_t* ptile,
+                                                         uint32_t* pv, const uint2* __restrict__ groups) {
   if (GROUPS) pdl_wait();   // (launched after k_long_split: wait for it)
   __shared__ SortSmem s;
   if (st->overflow) return;
-  const uint32_t tile_ctas = TILES ? n_tiles + (n_tiles + kSortWarps - 1) / kSortWarps : 0u;
+  const uint32_t tile_ctas = TILES ? n_tiles + n_warp : 0u;
   if (TILES && (!GROUPS || blockIdx.x < tile_ctas)) {
     const bool own = blockIdx.x < n_tiles;
     const uint32_t tile = own ? blockIdx.x : (blockIdx.x - n_tiles) * kSortWarps + (threadIdx.x >> 5);
@@ -1403,7 +1405,7 @@ __global__ void __launch_bounds__(kSortCta, TILES && GROUPS ? 4 : 0) k_tile_sort
     const uint32_t n = rg.y - rg.x;
     if (!own) {
       if (n <= kWarpSort) sort_warp(pkey + rg.x, n, pv + rg.x);
-    } else if (n > kWarpSort && n <= kSortMax) {   // (longer: k_long_split's)
+    } else if (n > (n_warp ? kWarpSort : 0u) && n <= kSortMax) {   // (longer: k_long_split's)
       sort_small<true>([&](uint32_t i) { return pkey[rg.x + i]; }, n, pv + rg.x, s);
     }
     return;
@@ -1486,17 +1488,19 @@ cudaError_t launch_bin(const Layout& L, const WsPtrs& w, int n_frames, int64_t n
     // the tile scan found none), then the CTAs that sort their groups
     const LongPath path = long_path(max_n);
     const unsigned group_ctas = 4 * sms;
+    const uint32_t n_warp = n_items < kSparse * n_tiles ? (n_tiles + kSortWarps - 1) / kSortWarps : 0u;
     const SegPlan plan{w.longt, w.sbase, w.segs, w.dead, blocks};
     cudaError_t e = cudaSuccess;
     if (path == kLongInline) {
       k_long_split<<<2 * sms, kLongCta, 0, s>>>(w.ranges, w.st, w.work, n_tiles, w.pkey, w.ptile, w.pv, w.groups,
                                                   plan);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
-      return launch_dep(k_tile_sort<true, true>, dim3(tile_sort_ctas(n_tiles) + group_ctas), dim3(kSortCta), 0, s, w.ranges, w.st,
-                        n_tiles, w.pkey, w.ptile, w.pv, w.groups);
+      return launch_dep(k_tile_sort<true, true>, dim3(n_tiles + n_warp + group_ctas), dim3(kSortCta), 0, s, w.ranges, w.st,
+                        n_tiles, n_warp, w.pkey, w.ptile, w.pv, w.groups);
     }
     if (path == kLongSide && (e = cudaEventRecord(side.fork, s)) != cudaSuccess) return e;
-    k_tile_sort<true, false><<<tile_sort_ctas(n_tiles), kSortCta, 0, s>>>(w.ranges, w.st, n_tiles, w.pkey, w.ptile, w.pv, w.groups);
+    k_tile_sort<true, false><<<n_tiles + n_warp, kSortCta, 0, s>>>(w.ranges, w.st, n_tiles, n_warp, w.pkey, w.ptile,
+                                                                   w.pv, w.groups);
     if ((e = cudaGetLastError()) != cudaSuccess || path == kLongNone) return e;
     // (the side stream has the higher priority: its CTAs take the slots that
     // short buckets free, and the launches do not delay the short buckets)
@@ -1504,7 +1508,7 @@ cudaError_t launch_bin(const Layout& L, const WsPtrs& w, int n_frames, int64_t n
     k_long_split<<<2 * sms, kLongCta, 0, side.s>>>(w.ranges, w.st, w.work, n_tiles, w.pkey, w.ptile, w.pv, w.groups,
                                                    plan);
     if ((e = cudaGetLastError()) == cudaSuccess)
-      e = launch_dep(k_tile_sort<false, true>, dim3(group_ctas), dim3(kSortCta), 0, side.s, w.ranges, w.st, 0u,
+      e = launch_dep(k_tile_sort<false, true>, dim3(group_ctas), dim3(kSortCta), 0, side.s, w.ranges, w.st, 0u, 0u,
                      w.pkey, w.ptile, w.pv, w.groups);
     if (e == cudaSuccess) e = cudaEventRecord(side.join, side.s);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(s, side.join, 0);
