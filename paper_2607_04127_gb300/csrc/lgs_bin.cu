@@ -18,8 +18,8 @@
 //   k_long_split  buckets of more than 2048 keys: partitioned by depth into
 //                 groups of about 1024 keys, one CTA per bucket, longest first
 //   k_tile_sort   sort every shorter bucket and every group by the 64-bit key,
-//                 one CTA each, by distribution in shared memory; write the
-//                 item list
+//                 one CTA each (in sparse calls a warp each of the shortest), by
+//                 distribution in shared memory; write the item list
 // The result is the order of the key (tile, depth, item): per tile, by depth,
 // ties by item index.
 #include <cuda_runtime.h>
@@ -914,12 +914,12 @@ __device__ __forceinline__ void sort_small(const Get& get, uint32_t n, uint32_t*
 // global memory, was bound by the longest bucket's serial passes (6 maps with
 // buckets up to 292 k keys, 28.9 M long keys: 3.49 -> 0.58 + 0.27 ms; 8
 // keyframes of a 1M map, 25.6 M long keys: 1.04 -> 0.18 + 0.25 ms).
-// A group of more than kSortMax keys (depths that cluster far below a bin's
-// width, a smooth wall in a bucket with a near and a far surfel, or equal ones)
-// is partitioned once more, by the same CTA, with its own range of (depth, item).
-// What then still exceeds kSortMax (clusters
-// within clusters) is sorted by its CTA with sorted chunks and merge passes
-// through global memory.  (10,000 keys on a wall with 1 mm of noise between a near
+// While one bin holds most keys (a smooth wall in a bucket with a near and a far
+// surfel) the bins are spread over its range alone.  A group of more than kSortMax
+// keys (several such clusters, or equal depths) is partitioned once more, by the
+// same CTA, with its own range of (depth, item).  What then still exceeds kSortMax
+// (clusters within clusters) is sorted by its CTA with sorted chunks and merge
+// passes through global memory.  (10,000 keys on a wall with 1 mm of noise between a near
 // and a far surfel, the binning: 202 us when the large groups were merged, 79 with
 // one CTA per bucket, now 57; 300,000 equal depths 7.8, 3.1 and 0.75 ms.)
 constexpr int kLongCta = 1024;
@@ -1379,13 +1379,12 @@ __device__ __forceinline__ void sort_warp(const unsigned long long* key, uint32_
 // kSortMax keys.  In a sparse call (below kSparse items a tile) they leave buckets
 // of up to kWarpSort keys to a warp each of n_warp more CTAs: with a CTA for every
 // tile, a frame of few surfels was bound by 2,048 CTAs' barriers over a few keys
-// each.  Binning of a 128 x 1024 frame, without and with the warps: 3,000 surfels 47
-// and 35 us; 16,000 49 and 40; 64,000 (31 items a tile) 43.8 and 44.1; 200,000 55.9
-// and 57.5;
-// warps up to 128 keys were 2 us slower from 16,000 surfels on.  GROUPS: the CTAs
-// after them take the long buckets' groups (their keys in the split buffer) in
-// turn.  Both in one kernel take 106 registers, the tiles alone 60, so that one is
-// held at 64 (16,000 surfels 49 us on 106).
+// each.  Binning of a 128 x 1024 frame, without and with the warps: 3,000 surfels 41
+// and 35 us, 16,000 42 and 40, 64,000 (31 items a tile) 43.8 and 44.1, 200,000 55.9
+// and 57.5; warps up to 128 keys were 2 us slower from 16,000 surfels on.  GROUPS:
+// the CTAs after them take the long buckets' groups (their keys in the split
+// buffer) in turn.  Both in one kernel take 106 registers, the tiles alone 60, so
+// that one is held at 64 (16,000 surfels 49 us with 106, now 40).
 constexpr uint32_t kSortWarps = kSortCta / 32;
 constexpr int64_t kSparse = 32;
 template <bool TILES, bool GROUPS>

@@ -1733,9 +1733,9 @@ __global__ void __launch_bounds__(kBwdChunkCta, 7)
     }
   }
   if (waiting) bwd_flush(sb, lane < waiting ? w_start : used, w_item, g13, lane);
-  // (the claim counter and the queue sizes are zeroed for the next backward
-  // by k_preprocess_bwd, which follows on the stream; no statistics counters: the backward's contributions are the forward's
-  // composited pairs, counted there)
+  // (the claim counter and the queue sizes are zeroed for the next backward by
+  // k_preprocess_bwd, which follows on the stream; no statistics counters: the
+  // backward's contributions are the forward's composited pairs, counted there)
 }
 
 // Long lists in the backward of the tunings without chunks: a work item is one
