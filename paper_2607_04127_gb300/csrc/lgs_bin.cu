@@ -914,14 +914,18 @@ __device__ __forceinline__ void sort_small(const Get& get, uint32_t n, uint32_t*
 // global memory, was bound by the longest bucket's serial passes (6 maps with
 // buckets up to 292 k keys, 28.9 M long keys: 3.49 -> 0.58 + 0.27 ms; 8
 // keyframes of a 1M map, 25.6 M long keys: 1.04 -> 0.18 + 0.25 ms).
-// While one bin holds most keys (a smooth wall in a bucket with a near and a far
-// surfel) the bins are spread over its range alone.  A group of more than kSortMax
-// keys (several such clusters, or equal depths) is partitioned once more, by the
-// same CTA, with its own range of (depth, item).  What then still exceeds kSortMax
-// (clusters within clusters) is sorted by its CTA with sorted chunks and merge
-// passes through global memory.  (10,000 keys on a wall with 1 mm of noise between a near
-// and a far surfel, the binning: 202 us when the large groups were merged, 79 with
-// one CTA per bucket, now 57; 300,000 equal depths 7.8, 3.1 and 0.75 ms.)
+// A bucket with a group of more than kSortMax keys is partitioned anew, by the same
+// CTA when its other buckets are done: while one bin holds most keys (a smooth wall
+// in a bucket with a near and a far surfel) the bins are spread over its range
+// alone, and a group that is still too large (several such clusters, or equal
+// depths) is partitioned once more with its own range of (depth, item).  What then
+// still exceeds kSortMax (clusters within clusters) is sorted by its CTA with sorted
+// chunks and merge passes through global memory.  (10,000 keys on a wall with 1 mm
+// of noise between a near and a far surfel, the binning: 196 us when the large
+// groups were merged, 74 with one CTA per bucket, now 59; 300,000 equal depths 7.8,
+// 3.1 and 0.85 ms.  All of it stays out of the loop over the buckets, which has 32
+// registers: a call in it made the longest bucket of six maps 499 -> 776 us alone,
+// its loads no longer four at a time.)
 constexpr int kLongCta = 1024;
 constexpr uint32_t kLongCoarse = 2048;
 constexpr uint32_t kMaxGroups = 2048;
@@ -1167,18 +1171,19 @@ struct SplitSmem {
   uint32_t hist[2 * kLongCta];       // counts per bin, then per group, then group cursors
   uint32_t start[kLongCoarse + 2];   // the keys before each bin
   uint32_t w[32], mm[4], claim, at, next;
+  uint32_t clustered;   // head of the list of this CTA's clustered buckets (1 + order position, 0 at the end)
 };
 
 // One partition of n keys: each(fn) calls fn(value, key) for all of them, the
 // bins estimate ranks, and the keys of one group of 2^sh estimated ranks go to
 // one range: put(place, key).  While one bin holds most keys, the bins are
-// spread over its range alone.  Gives the thread's groups 2t and 2t + 1: their
-// counts, and first places (to `early`, before the keys move).  hist is zero on
-// entry.
+// spread over its range alone.  early(counts, first places) gets the thread's
+// groups 2t and 2t + 1 before the keys move.  hist is zero on entry.
 template <class V, class Each, class Early, class Put>
 __device__ __forceinline__ void partition(const Each& each, Bins<V> bins, uint32_t n, uint32_t sh, SplitSmem& s,
-                                          uint2& c, const Early& early, const Put& put) {
+                                          const Early& early, const Put& put) {
   const uint32_t t = threadIdx.x;
+  uint2 c;
   while (true) {
     each([&](V v, unsigned long long) {
       float frac;
@@ -1205,7 +1210,7 @@ __device__ __forceinline__ void partition(const Each& each, Bins<V> bins, uint32
   const uint2 at = long_exclusive(c, s.w);
   s.hist[2 * t] = at.x;
   s.hist[2 * t + 1] = at.y;
-  early(at);
+  early(c, at);
   __syncthreads();
   each([&](V v, unsigned long long x) { put(atomicAdd(&s.hist[bins.rank(v, s.start) >> sh], 1u), x); });
 }
@@ -1216,14 +1221,14 @@ __device__ __forceinline__ uint32_t group_shift(uint32_t n) {
   return sh;
 }
 
-// The second partition, of the n keys at `first` of the split buffer (through the
-// key array, which the first one is done with): by (depth, item) as one number,
-// the depths above the lowest times the items' span plus the item, so that
-// equal depths spread by item.
-__device__ __noinline__ void split_again(uint32_t first, uint32_t n, unsigned long long* pkey, uint32_t* ptile,
-                                         uint32_t* pv, uint2* groups, Status* st, SplitSmem& s) {
+// The second partition, of the n keys at `first` of the split buffer (the arrays'
+// pointers are those of this range; through the key array, which the first one is
+// done with): by (depth, item) as one number, the depths above the lowest times the
+// items' span plus the item, so that equal depths spread by item.
+__device__ __noinline__ void split_again(SplitSmem& s, uint32_t first, uint32_t n, unsigned long long* pkey,
+                                         uint32_t* ptile, uint32_t* pv, uint2* groups, uint32_t* all_groups) {
   const uint32_t t = threadIdx.x;
-  const KeyBuf Y{nullptr, ptile + first, pv + first};
+  const KeyBuf Y{nullptr, ptile, pv};
   if (t < 4) s.mm[t] = t & 1u ? 0u : ~0u;
   s.hist[2 * t] = s.hist[2 * t + 1] = 0u;
   __syncthreads();
@@ -1250,31 +1255,97 @@ __device__ __noinline__ void split_again(uint32_t first, uint32_t n, unsigned lo
   const unsigned long long span = static_cast<unsigned long long>(s.mm[3] - ilo) + 1ull;
   const unsigned long long most = (s.mm[1] - dlo) * span + (span - 1ull);
   const uint32_t sh = group_shift(n), n_groups = ((n - 1) >> sh) + 1;
-  if (t == 0) s.at = atomicAdd(&st->n_groups, n_groups);
-  uint2 c = make_uint2(0u, 0u);
+  if (t == 0) s.at = atomicAdd(all_groups, n_groups);
   partition([&](auto fn) {
               for_keys(Y, n, [&](unsigned long long x) {
                 fn((static_cast<uint32_t>(x >> 32) - dlo) * span + (static_cast<uint32_t>(x) - ilo), x);
               });
             },
-            bins_over(0ull, most), n, sh, s, c,
-            [&](uint2 at) {
+            bins_over(0ull, most), n, sh, s,
+            [&](uint2 c, uint2 at) {
               if (2 * t < n_groups) groups[s.at + 2 * t] = make_uint2(first + at.x, first + at.x + c.x);
               if (2 * t + 1 < n_groups) groups[s.at + 2 * t + 1] = make_uint2(first + at.y, first + at.y + c.y);
             },
-            [&](uint32_t pos, unsigned long long x) { pkey[first + pos] = x; });
+            [&](uint32_t pos, unsigned long long x) { pkey[pos] = x; });
   __syncthreads();
-  for (uint32_t i = t; i < n; i += kLongCta) Y.put(i, __ldcg(pkey + first + i));
+  for (uint32_t i = t; i < n; i += kLongCta) Y.put(i, __ldcg(pkey + i));
+}
+
+// The first bucket of the CTA's list, whose depths cluster: partitioned with bins
+// spread over the cluster, then the groups of more than kSortMax keys once more,
+// one after the other.
+__device__ __noinline__ void split_clustered(SplitSmem& s, unsigned long long* pkey, uint32_t* ptile, uint32_t* pv,
+                                             uint2* groups, uint32_t* all_groups, const uint2* ranges,
+                                             const uint32_t* order, const uint32_t* next) {
+  const uint32_t t = threadIdx.x, k = s.clustered - 1;
+  const uint2 rg = ranges[order[k]];
+  const uint32_t first = rg.x, n = rg.y - rg.x;
+  const uint32_t sh = group_shift(n), n_groups = ((n - 1) >> sh) + 1;
+  const unsigned long long* X = pkey + first;
+  __syncthreads();   // (every thread has read the list's head)
+  if (t == 0) {
+    s.clustered = next[k];
+    s.mm[0] = ~0u;
+    s.mm[1] = 0u;
+  }
+  __syncthreads();
+  uint32_t lo = ~0u, hi = 0u;
+  for_keys(X, n, [&](unsigned long long x) {
+    lo = min(lo, static_cast<uint32_t>(x >> 32));
+    hi = max(hi, static_cast<uint32_t>(x >> 32));
+  });
+  atomicMin(&s.mm[0], __reduce_min_sync(0xffffffffu, lo));
+  atomicMax(&s.mm[1], __reduce_max_sync(0xffffffffu, hi));
+  if (t == 0) s.at = atomicAdd(all_groups, n_groups);
+  s.hist[2 * t] = s.hist[2 * t + 1] = 0u;
+  __syncthreads();
+  partition([&](auto fn) { for_keys(X, n, [&](unsigned long long x) { fn(static_cast<uint32_t>(x >> 32), x); }); },
+            bins_over(s.mm[0], s.mm[1]), n, sh, s,
+            [&](uint2 c, uint2 at) {
+              // (an empty range where split_again stores the groups instead)
+              const uint2 e = make_uint2(c.x > kSortMax ? 0u : c.x, c.y > kSortMax ? 0u : c.y);
+              if (2 * t < n_groups) groups[s.at + 2 * t] = make_uint2(first + at.x, first + at.x + e.x);
+              if (2 * t + 1 < n_groups) groups[s.at + 2 * t + 1] = make_uint2(first + at.y, first + at.y + e.y);
+            },
+            [&](uint32_t pos, unsigned long long x) {
+              ptile[first + pos] = static_cast<uint32_t>(x >> 32);
+              pv[first + pos] = static_cast<uint32_t>(x);
+            });
+  __syncthreads();
+  // (every cursor stands at its group's end, where the next group starts)
+  const uint32_t a = t ? s.hist[2 * t - 1] : 0u;
+  const uint2 end = make_uint2(s.hist[2 * t], s.hist[2 * t + 1]), c = make_uint2(end.x - a, end.y - end.x);
+  for (uint32_t from = 0;;) {
+    __syncthreads();
+    if (t == 0) s.next = ~0u;
+    __syncthreads();
+    if (c.y > kSortMax && 2 * t + 1 >= from) atomicMin(&s.next, 2 * t + 1);
+    if (c.x > kSortMax && 2 * t >= from) atomicMin(&s.next, 2 * t);
+    __syncthreads();
+    const uint32_t g = s.next;
+    if (g == ~0u) return;   // (after a barrier: the next call may rewrite everything)
+    if (t == g / 2) {
+      s.mm[0] = g & 1u ? c.y : c.x;
+      s.mm[1] = g & 1u ? end.y : end.x;
+    }
+    __syncthreads();
+    const uint32_t m = s.mm[0], e = s.mm[1];
+    __syncthreads();
+    const uint32_t at = first + e - m;
+    split_again(s, at, m, pkey + at, ptile + at, pv + at, groups, all_groups);
+    from = g + 1;
+  }
 }
 
 __global__ void __launch_bounds__(kLongCta, 2)
     k_long_split(const uint2* __restrict__ ranges, Status* __restrict__ st, const uint32_t* __restrict__ order,
-                 uint32_t n_tiles, unsigned long long* pkey, uint32_t* ptile, uint32_t* pv,
-                 uint2* __restrict__ groups, SegPlan plan) {
+                 uint32_t n_tiles, unsigned long long* pkey, uint32_t* __restrict__ ptile,
+                 uint32_t* __restrict__ pv, uint2* __restrict__ groups, uint32_t* __restrict__ next, SegPlan plan) {
   pdl_launch_dependents();  // the next kernel may be dispatched now
   __shared__ SplitSmem s;
   if (st->overflow || st->n_big == 0) return;
   const uint32_t t = threadIdx.x;
+  if (t == 0) s.clustered = 0u;
   if (blockIdx.x == gridDim.x - 1 && st->n_long) plan_segments(ranges, st, plan, s.hist, s.w);
   while (true) {
     // buckets in the tile scan's longest-first order; the long ones come
@@ -1288,10 +1359,10 @@ __global__ void __launch_bounds__(kLongCta, 2)
     s.hist[2 * t] = s.hist[2 * t + 1] = 0u;
     __syncthreads();
     const uint32_t k = s.claim;
-    if (k >= n_tiles) return;
+    if (k >= n_tiles) break;
     const uint2 rg = ranges[order[k]];
     const uint32_t n = rg.y - rg.x;
-    if (order_bucket(n) > order_bucket(kSortMax + 1)) return;   // a shorter class: no long list follows
+    if (order_bucket(n) > order_bucket(kSortMax + 1)) break;   // a shorter class: no long list follows
     if (n <= kSortMax) continue;
     const uint32_t sh = group_shift(n), n_groups = ((n - 1) >> sh) + 1;
     const unsigned long long* X = pkey + rg.x;
@@ -1307,48 +1378,47 @@ __global__ void __launch_bounds__(kLongCta, 2)
       atomicMin(&s.mm[0], lo);
       atomicMax(&s.mm[1], hi);
     }
+    __syncthreads();
+    const DepthMap map(s.mm[0], s.mm[1], kLongCoarse);
+    for_keys(X, n, [&](unsigned long long x) {
+      float frac;
+      atomicAdd(&s.hist[map.bin(static_cast<uint32_t>(x >> 32), frac)], 1u);
+    });
+    __syncthreads();
+    const uint2 first = long_exclusive(make_uint2(s.hist[2 * t], s.hist[2 * t + 1]), s.w);
+    s.start[2 * t] = first.x;
+    s.start[2 * t + 1] = first.y;
+    if (t == 0) s.start[kLongCoarse] = n;
+    s.hist[2 * t] = s.hist[2 * t + 1] = 0u;   // (every thread has read its own counts only)
+    __syncthreads();
+    for_keys(X, n, [&](unsigned long long x) {
+      atomicAdd(&s.hist[map.rank(static_cast<uint32_t>(x >> 32), s.start) >> sh], 1u);
+    });
+    __syncthreads();
+    const uint2 c = make_uint2(s.hist[2 * t], s.hist[2 * t + 1]);
+    if (__syncthreads_or(max(c.x, c.y) > kSortMax)) {
+      // (listed, and partitioned when this CTA's other buckets are done: a call
+      // here would cost the loop its registers)
+      if (t == 0) {
+        next[k] = s.clustered;
+        s.clustered = k + 1;
+      }
+      continue;
+    }
+    const uint2 at = long_exclusive(c, s.w);
+    s.hist[2 * t] = at.x;
+    s.hist[2 * t + 1] = at.y;
     if (t == 0) s.at = atomicAdd(&st->n_groups, n_groups);
     __syncthreads();
-    uint2 c = make_uint2(0u, 0u);
-    partition([&](auto fn) {
-                for_keys(X, n, [&](unsigned long long x) { fn(static_cast<uint32_t>(x >> 32), x); });
-              },
-              bins_over(s.mm[0], s.mm[1]), n, sh, s, c,
-              [&](uint2 at) {
-                // (an empty range where split_again stores the groups instead)
-                const uint2 e = make_uint2(c.x > kSortMax ? 0u : c.x, c.y > kSortMax ? 0u : c.y);
-                if (2 * t < n_groups) groups[s.at + 2 * t] = make_uint2(rg.x + at.x, rg.x + at.x + e.x);
-                if (2 * t + 1 < n_groups) groups[s.at + 2 * t + 1] = make_uint2(rg.x + at.y, rg.x + at.y + e.y);
-              },
-              [&](uint32_t pos, unsigned long long x) {
-                ptile[rg.x + pos] = static_cast<uint32_t>(x >> 32);
-                pv[rg.x + pos] = static_cast<uint32_t>(x);
-              });
-    // the groups of more than kSortMax keys, one after the other
-    if (__syncthreads_or(c.x > kSortMax || c.y > kSortMax)) {
-      // (a group's cursor now stands at its end)
-      const uint2 end = make_uint2(s.hist[2 * t], s.hist[2 * t + 1]);
-      for (uint32_t from = 0;;) {
-        __syncthreads();
-        if (t == 0) s.next = ~0u;
-        __syncthreads();
-        if (c.y > kSortMax && 2 * t + 1 >= from) atomicMin(&s.next, 2 * t + 1);
-        if (c.x > kSortMax && 2 * t >= from) atomicMin(&s.next, 2 * t);
-        __syncthreads();
-        const uint32_t g = s.next;
-        if (g == ~0u) break;
-        if (t == g / 2) {
-          s.mm[0] = g & 1u ? c.y : c.x;
-          s.mm[1] = g & 1u ? end.y : end.x;
-        }
-        __syncthreads();
-        const uint32_t m = s.mm[0], e = s.mm[1];
-        __syncthreads();
-        split_again(rg.x + e - m, m, pkey, ptile, pv, groups, st, s);
-        from = g + 1;
-      }
-    }
+    if (2 * t < n_groups) groups[s.at + 2 * t] = make_uint2(rg.x + at.x, rg.x + at.x + c.x);
+    if (2 * t + 1 < n_groups) groups[s.at + 2 * t + 1] = make_uint2(rg.x + at.y, rg.x + at.y + c.y);
+    for_keys(X, n, [&](unsigned long long x) {
+      const uint32_t pos = rg.x + atomicAdd(&s.hist[map.rank(static_cast<uint32_t>(x >> 32), s.start) >> sh], 1u);
+      ptile[pos] = static_cast<uint32_t>(x >> 32);
+      pv[pos] = static_cast<uint32_t>(x);
+    });
   }
+  while (s.clustered) split_clustered(s, pkey, ptile, pv, groups, &st->n_groups, ranges, order, next);
 }
 
 // A bucket of n <= kWarpSort keys sorted by one warp, kWarpKeys keys a lane: a
@@ -1492,7 +1562,7 @@ cudaError_t launch_bin(const Layout& L, const WsPtrs& w, int n_frames, int64_t n
     cudaError_t e = cudaSuccess;
     if (path == kLongInline) {
       k_long_split<<<2 * sms, kLongCta, 0, s>>>(w.ranges, w.st, w.work, n_tiles, w.pkey, w.ptile, w.pv, w.groups,
-                                                  plan);
+                                                  w.tcur, plan);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
       return launch_dep(k_tile_sort<true, true>, dim3(n_tiles + n_warp + group_ctas), dim3(kSortCta), 0, s, w.ranges, w.st,
                         n_tiles, n_warp, w.pkey, w.ptile, w.pv, w.groups);
@@ -1505,7 +1575,7 @@ cudaError_t launch_bin(const Layout& L, const WsPtrs& w, int n_frames, int64_t n
     // short buckets free, and the launches do not delay the short buckets)
     if ((e = cudaStreamWaitEvent(side.s, side.fork, 0)) != cudaSuccess) return e;
     k_long_split<<<2 * sms, kLongCta, 0, side.s>>>(w.ranges, w.st, w.work, n_tiles, w.pkey, w.ptile, w.pv, w.groups,
-                                                   plan);
+                                                   w.tcur, plan);
     if ((e = cudaGetLastError()) == cudaSuccess)
       e = launch_dep(k_tile_sort<false, true>, dim3(group_ctas), dim3(kSortCta), 0, side.s, w.ranges, w.st, 0u, 0u,
                      w.pkey, w.ptile, w.pv, w.groups);

@@ -138,7 +138,7 @@ struct WsPtrs {
   uint32_t* key;           // depth key per item
   uint32_t* cnt;           // tile count per item
   uint2* tset;             // tile set per item: rows (first | last << 16), columns (first | count << 16)
-  uint32_t* tcur;          // [tiles] pair counts, then fill cursors
+  uint32_t* tcur;          // [tiles] pair counts, then fill cursors, then the long sort's lists of clustered buckets
   unsigned long long* pkey;// [pairs] (depth key << 32 | item), bucketed by tile (until the forward: segsum)
   uint32_t* ptile;         // [pairs] tile of every pair (sorted order)
   uint32_t* pv;            // [pairs] item of every pair (sorted order)
